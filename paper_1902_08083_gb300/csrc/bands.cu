@@ -8,7 +8,7 @@
 // bottom-up pass per band then fills the band records of every cell:
 //   bA[X].b  = fp32(sum_i w_i alpha_b,i / sum_i w_i)          (Sec. 2.2.3, 2.3)
 //   bLc[X].b = fp32(sum_j L_b,j)
-//   nB[X].w  = max over the bands of fp32(alpha_max,b - alpha_min,b)
+//   nB[X].w (and nR[X].y) = max over the bands of fp32(alpha_max,b - alpha_min,b)
 // The last line makes a cell refine (Eq. refcrit) when any band asks for it. The
 // directional alpha_min / alpha_max recursion and the FP64 operation order are those
 // of the single-band moments.
@@ -38,6 +38,7 @@ struct BandArgs {
   float* bA;            // per cell, 4 slots
   float* bLc;           // per cell, 4 slots
   float4* nB;
+  float4* nR;
   int b;
 };
 
@@ -122,7 +123,10 @@ __global__ void band_moments_level_kernel(BandArgs A, int Lv) {
     A.bA[4 * (size_t)X + A.b] = __double2float_rn(__ddiv_rn(m.WA, A.nW[X]));
     A.bLc[4 * (size_t)X + A.b] = __double2float_rn(m.L);
     const float dal = __double2float_rn(__dsub_rn(amax, amin));
-    if (dal > A.nB[X].w) A.nB[X].w = dal;
+    if (dal > A.nB[X].w) {
+      A.nB[X].w = dal;
+      A.nR[X].y = dal;
+    }
   }
 }
 
@@ -206,6 +210,7 @@ int build_tree_bands_impl(const float* gas_xyz, const float* alpha_bands, const 
     A.bA = reinterpret_cast<float*>(t->bA);
     A.bLc = reinterpret_cast<float*>(t->bLc);
     A.nB = t->nB;
+    A.nR = t->nR;
     for (int b = 0; b < nb; ++b) {
       band_alpha_kernel<<<grid_of(n, 256), 256, 0, s>>>(alpha_bands + (size_t)b * n, t->perm, n,
                                                          as, st);

@@ -236,6 +236,7 @@ struct TopoArrays {
   int4* nghi;
   int4* nT;    // x child, y parent, z src_first, w src_count
   int* ndepth;
+  unsigned long long* nD;  // path from the root (TreeView::nD)
   int* nsplit;  // first particle of the upper child, -1 for a leaf
   int* nbit;    // split key bit
   int* leaf_of;
@@ -256,6 +257,7 @@ __global__ void topo_init_kernel(TopoArrays A, int n) {
     A.nghi[kRoot] = make_int4(kGridMax, kGridMax, kGridMax, 0);
     A.nT[kRoot] = make_int4(-1, 0, 0, 0);
     A.ndepth[kRoot] = 0;
+    A.nD[kRoot] = A.nD[0] = 1ull << 63;
     // entry 0 is unused: make it an inert leaf
     A.nT[0] = make_int4(-1, 0, 0, 0);
   }
@@ -364,6 +366,9 @@ __device__ __forceinline__ void topo_emit_level(const TopoArrays& A, int L) {
       A.nT[child + 1] = make_int4(-1, X, 0, 0);
       A.ndepth[child] = L + 1;
       A.ndepth[child + 1] = L + 1;
+      const unsigned long long way = __ldcg(&A.nD[X]), end = 1ull << (62 - L);
+      A.nD[child] = way ^ (3ull * end);
+      A.nD[child + 1] = way | end;
     }
     running += total;
   }
@@ -489,7 +494,7 @@ struct MomentArrays {
   float4* nB;
   float4* nS;
   float* nl2;
-  float2* nSP;
+  float4* nR;
   float h;
 };
 
@@ -590,14 +595,17 @@ __device__ __forceinline__ void moments_cell(const MomentArrays& A, int X) {
     A.nB[X] = make_float4(bhi[0], bhi[1], bhi[2], dal);
     A.nS[X] = make_float4(c[0], c[1], c[2], Lf);
     A.nl2[X] = l2;
+    float plane = 0.0f;
+    unsigned link = 3u;  // a leaf
     if (t.x >= 0) {
       const int ax = A.nglo[X].w;
       const int4 u = A.nglo[t.x + 1];
-      A.nSP[X] = make_float2(rel_plane(A.h, ax == 0 ? u.x : (ax == 1 ? u.y : u.z)),
-                             __int_as_float(ax));
-    } else {
-      A.nSP[X] = make_float2(0.0f, __int_as_float(-1));
+      plane = rel_plane(A.h, ax == 0 ? u.x : (ax == 1 ? u.y : u.z));
+      link = ((unsigned)t.x >> 1) << 2 | (unsigned)ax;  // children are the pair (2k, 2k + 1)
     }
+    A.nR[X] = make_float4(abar, dal, plane, __uint_as_float(link));
+    // entry 0: an empty leaf
+    if (X == kRoot) A.nR[0] = make_float4(0.0f, 0.0f, 0.0f, __uint_as_float(3u));
   }
 }
 
@@ -704,6 +712,7 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   t->nghi = keep.get<int4>(cap);
   t->nT = keep.get<int4>(cap);
   t->ndepth = keep.get<int>(cap);
+  t->nD = keep.get<unsigned long long>(cap);
   t->src = keep.get<float4>(ns);
   t->src_order = keep.get<int>(ns);
   t->src_leaf = keep.get<int>(ns);
@@ -770,6 +779,7 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   TA.nghi = t->nghi;
   TA.nT = t->nT;
   TA.ndepth = t->ndepth;
+  TA.nD = t->nD;
   TA.nsplit = nsplit;
   TA.nbit = nbit;
   TA.leaf_of = t->leaf_of;
@@ -820,7 +830,7 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   t->nB = keep.get<float4>(ncell);
   t->nS = keep.get<float4>(ncell);
   t->nl2 = keep.get<float>(ncell);
-  t->nSP = keep.get<float2>(ncell);
+  t->nR = keep.get<float4>(ncell);
   t->nW = keep.get<double>(ncell);
   Moments* mom = tmp.get<Moments>(ncell);
   if (!keep.ok || !tmp.ok) {
@@ -832,7 +842,6 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   cudaMemsetAsync(t->nB, 0, sizeof(float4), s);
   cudaMemsetAsync(t->nS, 0, sizeof(float4), s);
   cudaMemsetAsync(t->nl2, 0, sizeof(float), s);
-  cudaMemsetAsync(t->nSP, 0, sizeof(float2), s);
   cudaMemsetAsync(t->nW, 0, sizeof(double), s);
   MomentArrays MA;
   MA.nT = t->nT;
@@ -850,7 +859,7 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   MA.nB = t->nB;
   MA.nS = t->nS;
   MA.nl2 = t->nl2;
-  MA.nSP = t->nSP;
+  MA.nR = t->nR;
   MA.h = t->h;
   // one launch per level, sized to the level (measured faster than one cooperative
   // launch over all levels: 0.26 against 0.66 ms per build at 2^22)

@@ -1,0 +1,801 @@
+// The flux walk of the warp variants (2 and 3): source walk, reverse rays and flux sum.
+//
+// The 32 lanes of a warp (32 consecutive sinks in Morton order) walk one depth-first
+// stack in shared memory, with a mask of the lanes that still need each cell. A lane
+// that accepts a cell, or reaches a source of an opened leaf, keeps that ray waiting; when a
+// lane with a waiting ray gets another, the waiting rays of all lanes are traced together.
+//
+// A ray is a list of pieces along [0, 1] (p + t d). All of them are cut from the clip of
+// the common ancestor A of the sink's leaf S and the source's cell C: a cell's interval
+// at its split plane, at t = (plane - p) * (1/d), gives the intervals of its children. On
+// the same fp32 planes this is exactly the children's own slab clip, since boxes nest, the
+// per-face t is monotone in the plane, and min and max are exact. So
+//   * the two paths from A to C and to S are followed by cell records, one cut a level,
+//     and only the siblings that the ray crosses become pieces (the C side in a
+//     first-in-first-out list, in the ray's order; the S side on the stack above it);
+//   * a piece that Eq. refcrit refines is cut in two: the nearer child goes on, the
+//     farther one waits on the stack with the end of its interval. Pieces are taken in the
+//     ray's order, so a piece begins where the one before it ended, and an entry is
+//     (cell, end).
+// Cell 0 is an empty leaf: the entry (0, t) moves the ray on to t. It stands where the
+// pieces do not follow one another, which only rounding brings about: a sink or a source
+// within an ulp of its cell's face, on the other side.
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "trevr_internal.cuh"
+#include "walk_common.cuh"
+
+namespace trevr {
+
+namespace {
+
+// pieces of a ray: at most 62 on either path and the path's end, one waiting child per level
+// of the piece that is being refined, and three entries for each sibling that rounding puts on
+// the other side of the path (at most one plane per axis and end lies within an ulp; kSpare
+// bounds them whatever the domain's planes are)
+constexpr int kPieces = 4 * kDepth;
+constexpr int kSpare = 20;
+static_assert(3 * kDepth + 3 * kSpare <= kPieces, "the list holds every piece of a ray");
+
+struct CutStack {
+  int node[kDepth + 2];
+  unsigned mask[kDepth + 2];
+};
+
+// ---------------------------------------------------------------------------
+// Sub-bucket particle trace (Sec. 2.2.3, 3.1.3). The absorption below the bucket
+// scale is the SPH field sum_j alpha_j w_j W(|x - x_j|, h_j), W(r, h) = w(r/h)/(pi h^3)
+// the cubic spline of support 2h. Along a ray at impact parameter b from x_j, with s
+// measured from the closest approach, the column over [s0, s1] is
+// (Phi(x, s1/h) - Phi(x, s0/h)) / (pi h^2), x = b^2/h^2, where Phi(x, sigma) is the
+// integral of w(sqrt(x + t^2)) over t in [0, sigma]: odd in sigma and constant beyond
+// the support. Phi comes from the tree's pre-computed table (the paper's pre-computed
+// kernel integral), bilinear in (x, sigma).
+__device__ __forceinline__ float kint_phi(const float4* __restrict__ tab, float x, float sigma) {
+  const float a = fminf(fabsf(sigma), 2.0f);
+  const float fx = x * (0.25f * (float)kKintNX), fs = a * (0.5f * (float)kKintNS);
+  const int i = min((int)fx, kKintNX - 1), j = min((int)fs, kKintNS - 1);
+  const float u = fx - (float)i, v = fs - (float)j;
+  const float4 c = __ldg(tab + (size_t)i * kKintNS + j);  // the cell's four corners
+  const float p0 = fmaf(v, c.y - c.x, c.x);
+  const float p1 = fmaf(v, c.w - c.z, c.z);
+  const float p = fmaf(u, p1 - p0, p0);
+  return sigma < 0.0f ? -p : p;
+}
+
+// Per-warp queue of the neighbours whose support meets the chord, so that the
+// quadrature runs on full warps: (x, sigma_0, sigma_1, alpha w / (pi h^2)).
+struct SubQueue {
+  float4 g[64];
+};
+
+// Optical depth of lane src's chord p + t d, t in [t0, t1], through the particles
+// listed for its leaf, the receiving particle (sorted index si) left out. The 32
+// lanes of the warp test one neighbour each per round, with the next round's
+// entries already loading; the neighbours that reach the chord are queued in shared
+// memory and integrated 32 at a time: (Phi(x, sigma_1) - Phi(x, sigma_0)) times
+// alpha w / (pi h^2), with x = b^2 / h^2 and sigma = s / h. Every lane must call it;
+// all lanes return the sum.
+__device__ __forceinline__ float sub_bucket_tau_warp(const TreeView& T, int src, int box, int si,
+                                                     float px, float py, float pz, float dx,
+                                                     float dy, float dz, float s2, float len,
+                                                     float t0, float t1) {
+  const unsigned FULL = 0xffffffffu;
+  const unsigned lane = threadIdx.x & 31u;
+  __shared__ SubQueue queues[4];  // one per warp of a 128-thread block
+  SubQueue& Q = queues[threadIdx.x >> 5];
+  box = __shfl_sync(FULL, box, src);
+  si = __shfl_sync(FULL, si, src);
+  px = __shfl_sync(FULL, px, src);
+  py = __shfl_sync(FULL, py, src);
+  pz = __shfl_sync(FULL, pz, src);
+  dx = __shfl_sync(FULL, dx, src);
+  dy = __shfl_sync(FULL, dy, src);
+  dz = __shfl_sync(FULL, dz, src);
+  s2 = __shfl_sync(FULL, s2, src);
+  len = __shfl_sync(FULL, len, src);
+  t0 = __shfl_sync(FULL, t0, src);
+  t1 = __shfl_sync(FULL, t1, src);
+  const float inv_s2 = 1.0f / s2;
+  float part = 0.0f;
+  int qn = 0;  // queued entries (warp-uniform)
+  const unsigned k0 = __ldg(&T.nbr_first[box]), k1 = __ldg(&T.nbr_first[box + 1]);
+  int2 nja = make_int2(-1, 0);  // the next round's entries
+  float4 nq = make_float4(0.0f, 0.0f, 0.0f, 1.0f);
+  if (k0 + lane < k1) {
+    nja = __ldg(&T.nbr_ja[k0 + lane]);
+    nq = __ldg(&T.nbr_sp[k0 + lane]);
+  }
+  for (unsigned base = k0; base < k1; base += 32u) {
+    const unsigned k = base + lane;
+    const int2 ja = nja;
+    const float4 q = nq;
+    if (k + 32u < k1) {
+      nja = __ldg(&T.nbr_ja[k + 32u]);
+      nq = __ldg(&T.nbr_sp[k + 32u]);
+    }
+    const float a = __int_as_float(ja.y);
+    bool pass = false;
+    float x = 0.0f, sa = 0.0f, sb = 0.0f;
+    if (k < k1 && ja.x != si && a > 0.0f) {
+      const float ux = q.x - px, uy = q.y - py, uz = q.z - pz;
+      const float tc = (ux * dx + uy * dy + uz * dz) * inv_s2;
+      const float ex = ux - tc * dx, ey = uy - tc * dy, ez = uz - tc * dz;
+      const float b2 = ex * ex + ey * ey + ez * ez;
+      const float ih = q.w;
+      x = b2 * ih * ih;
+      sa = ((t0 - tc) * len) * ih;
+      sb = ((t1 - tc) * len) * ih;
+      if (x < 4.0f) {  // the chord [sa, sb] must meet the support |sigma| < sqrt(4 - x)
+        const float u22 = 4.0f - x;
+        pass = (sb > 0.0f || sb * sb < u22) && (sa < 0.0f || sa * sa < u22);
+      }
+    }
+    const unsigned m = __ballot_sync(FULL, pass);
+    if (pass) {
+      const float ih = q.w;
+      Q.g[qn + __popc(m & ((1u << lane) - 1u))] =
+          make_float4(x, sa, sb, a * (ih * ih * 0.318309886f));
+    }
+    qn += __popc(m);
+    __syncwarp();
+    if (qn >= 32) {
+      const float4 g = Q.g[qn - 32 + (int)lane];
+      part += g.w * (kint_phi(T.kint4, g.x, g.z) - kint_phi(T.kint4, g.x, g.y));
+      qn -= 32;
+      __syncwarp();
+    }
+  }
+  if ((int)lane < qn) {
+    const float4 g = Q.g[lane];
+    part += g.w * (kint_phi(T.kint4, g.x, g.z) - kint_phi(T.kint4, g.x, g.y));
+  }
+  __syncwarp();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(FULL, part, o);
+  return part;
+}
+
+__device__ __forceinline__ unsigned cell_link(const float4& r) { return __float_as_uint(r.w); }
+__device__ __forceinline__ bool is_leaf(unsigned link) { return (link & 3u) == 3u; }
+__device__ __forceinline__ int lower_child(unsigned link) { return (int)((link >> 1) & ~1u); }
+
+// A ray from the sink p: direction d, and 1/d per axis. Along an axis that the ray does not
+// move on, 1/d is the largest float: (plane - p) * inv is then <= 0 for p >= plane and
+// beyond 1 for p < plane, so the cuts give the half-open boxes [lo, hi) of that case.
+struct Line {
+  float px, py, pz, dx, dy, dz, ix, iy, iz, s2, len;
+  __device__ __forceinline__ static float inverse(float d) {
+    return d != 0.0f ? __frcp_rn(d) : 3.402823466e38f;
+  }
+  __device__ __forceinline__ void aim(float qx, float qy, float qz) {
+    dx = __fsub_rn(qx, px);
+    dy = __fsub_rn(qy, py);
+    dz = __fsub_rn(qz, pz);
+    s2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+    len = __fsqrt_rn(s2);
+    ix = inverse(dx);
+    iy = inverse(dy);
+    iz = inverse(dz);
+  }
+  // where the ray crosses the split plane of r; forward: it goes to the upper child
+  __device__ __forceinline__ float cross(const float4& r, bool& forward) const {
+    const unsigned ax = cell_link(r) & 3u;
+    const float p = ax == 0u ? px : (ax == 1u ? py : pz);
+    const float i = ax == 0u ? ix : (ax == 1u ? iy : iz);
+    forward = i > 0.0f;
+    return __fmul_rn(__fsub_rn(r.z, p), i);
+  }
+  __device__ __forceinline__ void clip_axis(float lo, float hi, float p, float i, float& t0,
+                                            float& t1) const {
+    const float ta = __fmul_rn(__fsub_rn(lo, p), i), tb = __fmul_rn(__fsub_rn(hi, p), i);
+    t0 = fmaxf(t0, fminf(ta, tb));
+    t1 = fminf(t1, fmaxf(ta, tb));
+  }
+  __device__ __forceinline__ void clip(const float4& lo, const float4& hi, float& t0,
+                                       float& t1) const {
+    t0 = 0.0f;
+    t1 = 1.0f;
+    clip_axis(lo.x, hi.x, px, ix, t0, t1);
+    clip_axis(lo.y, hi.y, py, iy, t0, t1);
+    clip_axis(lo.z, hi.z, pz, iz, t0, t1);
+  }
+};
+
+// Background sources (Sec. 2.2.4): the centre of luminosity of an accepted cell moved
+// radially onto the sphere of radius P.bg_radius around the domain centre o (side / 2 in
+// coordinates relative to the lower corner), in fp32 as d = c - o,
+// s = sqrt((dx^2 + dy^2) + dz^2), q = o + d * (R / s); and the leaf that holds q (grid
+// coordinates clamped to the grid), found by descending the cut planes from the root, with
+// its path.
+__device__ __forceinline__ void bg_end(const TreeView& T, const WalkParams& P, float& qx,
+                                       float& qy, float& qz, int& Y, unsigned long long& way) {
+  const float o = __fmul_rn(T.side, 0.5f);
+  const float ddx = __fsub_rn(qx, o), ddy = __fsub_rn(qy, o), ddz = __fsub_rn(qz, o);
+  const float sn = __fsqrt_rn(__fadd_rn(__fadd_rn(__fmul_rn(ddx, ddx), __fmul_rn(ddy, ddy)),
+                                        __fmul_rn(ddz, ddz)));
+  if (sn > 0.0f) {
+    const float kk = __fdiv_rn(P.bg_radius, sn);
+    qx = __fadd_rn(o, __fmul_rn(ddx, kk));
+    qy = __fadd_rn(o, __fmul_rn(ddy, kk));
+    qz = __fadd_rn(o, __fmul_rn(ddz, kk));
+  }
+  const float scale = __fdiv_rn(2097152.0f, T.side);
+  const float q[3] = {qx, qy, qz};
+  int g[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    float t = __fmul_rn(q[d], scale);
+    if (!(t >= 0.0f)) t = 0.0f;
+    const unsigned v = __float2uint_rz(t);
+    g[d] = (int)(v > (unsigned)(kGridMax - 1) ? (unsigned)(kGridMax - 1) : v);
+  }
+  Y = kRoot;
+  for (int it = 0; it < kDepth - 1; ++it) {
+    const int ch = __ldg(&T.nT[Y].x);
+    if (ch < 0) break;
+    const int ax = __ldg(&T.nglo[Y].w);
+    const int4 up = __ldg(&T.nglo[ch + 1]);
+    const int gv = ax == 0 ? g[0] : (ax == 1 ? g[1] : g[2]);
+    const int plane = ax == 0 ? up.x : (ax == 1 ? up.y : up.z);
+    Y = gv >= plane ? ch + 1 : ch;
+  }
+  way = __ldg(&T.nD[Y]);
+}
+
+__device__ __forceinline__ int way_depth(unsigned long long way) {
+  return 64 - __ffsll((long long)way);
+}
+
+// The sink of a lane: sorted index, leaf, and the leaf's path.
+struct Sink {
+  int i, S;
+  unsigned long long way;
+};
+
+// One ray per lane that is `on`, from its sink to `ent` (a cell, or ~source); every lane of
+// the warp must call it. The loop ends: a refined piece goes on at a child, whose number is
+// larger than its parent's, and every entry of the list is taken once.
+// STOP: a ray whose running optical depth passes P.tau_stop ends and adds nothing (Sec. 4).
+// NB > 1: every band sums its own optical depth over the shared segments.
+// SUB: a leaf whose own particles ask for refinement is integrated through them.
+// TD: the top-down ray walk: A is the only piece, and Eq. refcrit alone splits it.
+template <bool MOM, bool BG, bool STOP, int NB, bool SUB, bool CNT, bool TD>
+__device__ __forceinline__ void cut_ray(const TreeView& T, const WalkParams& P, const float tref,
+                                        const bool on, const int ent, const Sink& K, Line& ray,
+                                        int2* __restrict__ piece, SinkCounters& cnt, CSum* F,
+                                        Moments* mom) {
+  const unsigned FULL = 0xffffffffu;
+  float L = 0.0f;
+  int C = kRoot;
+  bool active = false;
+  int n_fifo = 0, n = 0, head = 0;  // pieces [head, n_fifo) in order, [n_fifo, n) a stack
+  int box = 0;
+  float t0 = 0.0f, t1 = 0.0f;
+  ray.s2 = ray.len = 1.0f;
+  if (on) {
+    float qx, qy, qz;
+    unsigned long long wayC;
+    if (ent < 0) {
+      const float4 y = __ldg(&T.src[~ent]);
+      qx = y.x;
+      qy = y.y;
+      qz = y.z;
+      L = y.w;
+      C = __ldg(&T.src_leaf[~ent]);
+      wayC = __ldg(&T.nD[C]);
+    } else {
+      const float4 s = __ldg(&T.nS[ent]);
+      qx = s.x;
+      qy = s.y;
+      qz = s.z;
+      L = s.w;
+      C = ent;
+      if (BG) bg_end(T, P, qx, qy, qz, C, wayC);
+      else wayC = __ldg(&T.nD[C]);
+    }
+    ray.aim(qx, qy, qz);
+    if (!(ray.s2 < P.smin2)) {  // a source on top of the sink adds nothing
+      active = true;
+      const int dS = way_depth(K.way), dC = way_depth(wayC);
+      const int ds = min(min(__clzll((long long)(K.way ^ wayC)), dS), dC);
+      // A: down from the root along the shared path
+      unsigned long long way = K.way;
+      int cell = kRoot;
+      float4 r = __ldg(&T.nR[kRoot]);
+      for (int k = 0; k < ds; ++k) {
+        cell = lower_child(cell_link(r)) + (int)(way >> 63);
+        way <<= 1;
+        r = __ldg(&T.nR[cell]);
+      }
+      float a, b;
+      ray.clip(__ldg(&T.nA[cell]), __ldg(&T.nB[cell]), a, b);
+      if (TD || ds == dS || ds == dC) {  // one piece: A, or S = C
+        if (CNT) ++cnt.clip;
+        if (a < b) {
+          box = cell;
+          t0 = a;
+          t1 = b;
+        }
+      } else {
+        if (CNT) cnt.clip += dS + dC - 2 * ds;
+        if (!(a < b)) a = b = 0.0f;  // the clip may be at infinity (1/d overflows)
+        int spare = kSpare;
+        bool fwd;
+        const float t = ray.cross(r, fwd);
+        int up = (int)(way >> 63);
+        const int child = lower_child(cell_link(r));
+        const bool far_s = fwd == (up != 0);  // rounding only: the sink's child is the far one
+        float aC = far_s ? a : fmaxf(a, t), bC = far_s ? fminf(b, t) : b;
+        float aS = far_s ? fmaxf(a, t) : a, bS = far_s ? b : fminf(b, t);
+        const float startC = aC;
+        if (aC < bC) {  // the C side, in the ray's order
+          int X = child + (up ^ 1);
+          unsigned long long w = wayC << (ds + 1);
+          for (int k = ds + 1; k < dC && aC < bC; ++k) {
+            r = __ldg(&T.nR[X]);
+            const float tc = ray.cross(r, fwd);
+            const int u = (int)(w >> 63);
+            w <<= 1;
+            X = lower_child(cell_link(r)) + u;
+            if (fwd == (u != 0)) {  // the sibling lies before the path
+              const float e = fminf(bC, tc);
+              if (aC < e) piece[n++] = make_int2(X ^ 1, __float_as_int(e));
+              aC = fmaxf(aC, tc);
+            } else {  // behind it: rounding only
+              const float e = fmaxf(aC, tc);
+              if (e < bC && spare-- > 0) {
+                piece[n++] = make_int2(0, __float_as_int(e));
+                piece[n++] = make_int2(X ^ 1, __float_as_int(bC));
+                piece[n++] = make_int2(0, __float_as_int(aC));
+              }
+              bC = fminf(bC, tc);
+            }
+          }
+          if (aC < bC) piece[n++] = make_int2(X, __float_as_int(bC));
+        }
+        n_fifo = n;
+        if (aS < bS) {
+          if (n_fifo > 0 && bS != startC) piece[n++] = make_int2(0, __float_as_int(startC));
+          int X = child + up;
+          way <<= 1;
+          for (int k = ds + 1; k < dS && aS < bS; ++k) {
+            r = __ldg(&T.nR[X]);
+            const float tc = ray.cross(r, fwd);
+            up = (int)(way >> 63);
+            way <<= 1;
+            X = lower_child(cell_link(r)) + up;
+            if (fwd != (up != 0)) {  // the sibling lies behind the path
+              if (fmaxf(aS, tc) < bS) piece[n++] = make_int2(X ^ 1, __float_as_int(bS));
+              bS = fminf(bS, tc);
+            } else {  // before it: rounding only
+              const float e = fminf(bS, tc);
+              if (aS < e && spare-- > 0) {
+                piece[n++] = make_int2(0, __float_as_int(bS));
+                piece[n++] = make_int2(X ^ 1, __float_as_int(e));
+                piece[n++] = make_int2(0, __float_as_int(aS));
+              }
+              aS = fmaxf(aS, tc);
+            }
+          }
+          t0 = t1 = fminf(aS, 1.0f);  // beyond 1 an empty entry is next
+          if (aS < bS) {
+            box = X;
+            t1 = bS;
+          }
+        } else if (n_fifo > 0) {
+          t0 = t1 = startC;
+        }
+      }
+    }
+  }
+  const bool traced = active;
+  bool cut = false;
+  KSum tau;
+  KSum taub[NB];  // (NB > 1) optical depth of each band
+  while (__any_sync(FULL, active)) {
+    bool need_sub = false;
+    int sub_box = 0;
+    float sub_t0 = 0.0f, sub_t1 = 0.0f;
+    if (active) {
+      const float4 r = __ldg(&T.nR[box]);
+      const unsigned link = cell_link(r);
+      const float l = __fmul_rn(__fsub_rn(t1, t0), ray.len);
+      if (__fmul_rn(r.y, l) > tref && !is_leaf(link)) {
+        bool fwd;
+        const float t = ray.cross(r, fwd);
+        const int near = lower_child(link) + (fwd ? 0 : 1);
+        const bool hit_near = t > t0, hit_far = t < t1;
+        if (CNT) {
+          ++cnt.ref;
+          cnt.clip += (int)hit_near + (int)hit_far;
+        }
+        if (hit_near && hit_far) {
+          piece[n++] = make_int2(near ^ 1, __float_as_int(t1));
+          t1 = t;
+        }
+        box = hit_near ? near : near ^ 1;
+      } else {
+        if (NB > 1) {
+          const float4 ab = __ldg(&T.bA[box]);
+          taub[0].add(__fmul_rn(ab.x, l));
+          taub[1].add(__fmul_rn(ab.y, l));
+          if (NB > 2) {
+            taub[NB > 2 ? 2 : 0].add(__fmul_rn(ab.z, l));
+            taub[NB > 2 ? 3 : 0].add(__fmul_rn(ab.w, l));
+          }
+        } else if (SUB && box != 0 && is_leaf(link) && __fmul_rn(__ldg(&T.dbk[box]), l) > tref && l > 0.0f) {
+          // a bucket that still asks for refinement: its particles are traced by the
+          // whole warp at the end of this step
+          need_sub = true;
+          sub_box = box;
+          sub_t0 = t0;
+          sub_t1 = t1;
+          if (CNT) ++cnt.sub;
+        } else {
+          tau.add(__fmul_rn(r.x, l));
+        }
+        if (CNT && box != 0 && l > 0.0f) ++cnt.segs;
+        t0 = t1;
+        const bool stacked = n > n_fifo;
+        active = stacked || head < n_fifo;
+        if (STOP && tau.get() > P.tau_stop) {
+          cut = true;
+          active = false;
+        }
+        if (active) {
+          const int2 e = piece[stacked ? n - 1 : head];
+          n -= stacked ? 1 : 0;
+          head += stacked ? 0 : 1;
+          box = e.x;
+          t1 = __int_as_float(e.y);
+        }
+      }
+    }
+    if (SUB) {
+      // the leaves of this step that need the particle trace, one after another
+      unsigned m = __ballot_sync(FULL, need_sub);
+      while (m) {
+        const int src = __ffs(m) - 1;
+        m &= m - 1u;
+        const float t = sub_bucket_tau_warp(T, src, sub_box, K.i, ray.px, ray.py, ray.pz, ray.dx,
+                                            ray.dy, ray.dz, ray.s2, ray.len, sub_t0, sub_t1);
+        if ((int)(threadIdx.x & 31u) == src) tau.add(t);
+      }
+    }
+  }
+  if (!traced) return;
+  if (CNT) ++cnt.rays;
+  if (STOP && cut) {
+    if (CNT) ++cnt.cut;
+    return;
+  }
+  if (NB > 1) {
+    // the band luminosities of the source, or of the merged cell
+    const float4 Lb = ent < 0 ? __ldg(&T.bLs[~ent]) : __ldg(&T.bLc[C]);
+    const float den = kFourPi * ray.s2;
+    F[0].add(Lb.x * expf(-taub[0].get()) / den);
+    F[1].add(Lb.y * expf(-taub[1].get()) / den);
+    if (NB > 2) {
+      F[NB > 2 ? 2 : 0].add(Lb.z * expf(-taub[NB > 2 ? 2 : 0].get()) / den);
+      F[NB > 2 ? 3 : 0].add(Lb.w * expf(-taub[NB > 2 ? 3 : 0].get()) / den);
+    }
+    return;
+  }
+  const float f = L * expf(-tau.get()) / (kFourPi * ray.s2);
+  F[0].add(f);
+  if (MOM) {
+    const float il = 1.0f / ray.len;
+    const float n0 = -ray.dx * il, n1 = -ray.dy * il, n2 = -ray.dz * il;
+    mom->v[0].add(f * n0);
+    mom->v[1].add(f * n1);
+    mom->v[2].add(f * n2);
+    mom->v[3].add(f * n0 * n0);
+    mom->v[4].add(f * n1 * n1);
+    mom->v[5].add(f * n2 * n2);
+    mom->v[6].add(f * n0 * n1);
+    mom->v[7].add(f * n0 * n2);
+    mom->v[8].add(f * n1 * n2);
+  }
+}
+
+// The walk of the 32 sinks of one warp (a lane holds the sorted position i if `has`);
+// every lane of the warp must call it. MERGE: a ray waits until its lane gets
+// another; without it (variant 2) the rays to a cell are traced as soon as it is accepted.
+template <bool MERGE, bool MOM, bool BG, bool STOP, int NB, bool SUB, bool CNT, bool TD>
+__device__ __forceinline__ void cut_walk(const TreeView& T, const WalkParams& P, const bool has,
+                                         const int i, CutStack& ws, int* status,
+                                         SinkCounters& cnt, CSum* F, Moments* mom) {
+  const unsigned FULL = 0xffffffffu;
+  const unsigned lane = threadIdx.x & 31u;
+  const int stack_limit = P.stack_depth < kDepth ? P.stack_depth : kDepth;
+  // tau_ref <= 0 refines every cell: any l * spread >= 0 passes
+  const float tref = P.tau_ref <= 0.0f ? -1.0f : P.tau_ref;
+  int2 piece[kPieces];
+  Line ray;
+  ray.px = ray.py = ray.pz = 0.0f;
+  Sink K{i, 0, 1ull << 63};
+  if (has) {
+    const float4 p = T.pos[i];
+    ray.px = p.x;
+    ray.py = p.y;
+    ray.pz = p.z;
+    K.S = T.leaf_of[i];
+    K.way = __ldg(&T.nD[K.S]);
+  }
+  const unsigned live = __ballot_sync(FULL, has);
+  if (lane == 0) {
+    ws.node[0] = kRoot;
+    ws.mask[0] = live;
+  }
+  int sp = live ? 1 : 0;
+  bool wait = false;      // this lane has a ray that waits to be traced, to w_ent
+  int w_ent = 0;          // (a cell, or ~source)
+  int j = 0, j_end = 0;   // sources of the opened leaf still to be taken
+  unsigned opened = 0;    // the lanes that opened it
+  __syncwarp();
+  while (true) {
+    bool take = false;
+    int ent = 0;
+    const bool done = j >= j_end && sp == 0;
+    if (j < j_end) {
+      if (__ldg(&T.src[j].w) > 0.0f) {
+        take = (opened >> lane) & 1u;
+        ent = ~j;
+      }
+      ++j;
+    } else if (!done) {
+      --sp;
+      const int X = ws.node[sp];
+      const unsigned M = ws.mask[sp];
+      __syncwarp();
+      const float4 s = __ldg(&T.nS[X]);
+      bool open = false;
+      if (s.w > 0.0f && ((M >> lane) & 1u)) {
+        if (CNT) ++cnt.visit;
+        const float4 a = __ldg(&T.nA[X]);
+        const float4 bb = __ldg(&T.nB[X]);
+        const float ex = fmaxf(fmaxf(__fsub_rn(a.x, ray.px), __fsub_rn(ray.px, bb.x)), 0.0f);
+        const float ey = fmaxf(fmaxf(__fsub_rn(a.y, ray.py), __fsub_rn(ray.py, bb.y)), 0.0f);
+        const float ez = fmaxf(fmaxf(__fsub_rn(a.z, ray.pz), __fsub_rn(ray.pz, bb.z)), 0.0f);
+        const float r2 =
+            __fadd_rn(__fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey)), __fmul_rn(ez, ez));
+        take = __ldg(&T.nl2[X]) < __fmul_rn(P.theta2, r2);
+        open = !take;
+      }
+      ent = X;
+      const unsigned openM = __ballot_sync(FULL, open);
+      if (openM) {
+        const int4 t = __ldg(&T.nT[X]);
+        if (t.x < 0) {
+          j = t.z;
+          j_end = t.z + t.w;
+          opened = openM;
+        } else if (sp + 2 > stack_limit) {
+          if (lane == 0) atomicOr(status, kStatusStackOverflow);
+          sp = 0;
+        } else {
+          if (lane == 0) {
+            ws.node[sp] = t.x + 1;
+            ws.mask[sp] = openM;
+            ws.node[sp + 1] = t.x;
+            ws.mask[sp + 1] = openM;
+          }
+          sp += 2;
+          __syncwarp();
+        }
+      }
+    }
+    if (__any_sync(FULL, wait && (done || take || !MERGE))) {
+      cut_ray<MOM, BG, STOP, NB, SUB, CNT, TD>(T, P, tref, wait, w_ent, K, ray, piece, cnt, F,
+                                               mom);
+      wait = false;
+    }
+    if (done) break;
+    if (take) {
+      wait = true;
+      w_ent = ent;
+    }
+  }
+}
+
+// Issue-bound: the loop over a ray's pieces is ~50 instructions on one 16-byte record that
+// L1 mostly has, and what bounds the walk is how many of them it runs. Clipping every base
+// cell and refined child instead (~120 instructions on 44 bytes, 53 a ray where 35 are
+// crossed) took 118.4 ms a step at 2^22 sinks and 2^14 clumped sources; the cut pieces take
+// 56.7 ms (21.4 and 8.3 ms at 100003 sinks, tau_ref = 0.01).
+// Blocks of 128 per SM: 8 leave the plain walk its registers (61, no spills); 12 and 16 (40
+// and 32 registers) gave 58.9 and 55.9 ms at 2^22 but 9.5 and 10.1 ms at 100003 sinks, where
+// a warp's own speed counts and 8 took 8.4. The particle trace needs 4 (57.2 ms at 2^16
+// sinks, against 66.9 at 6 and 72.4 at 8), the bands 6 (8.95 ms for three at 200003 sinks,
+// 9.2 at 8).
+constexpr int cut_blocks(bool SUB, int NB) { return SUB ? 4 : NB > 1 ? 6 : 8; }
+
+template <bool MERGE, bool MOM, bool BG, bool STOP, int NB, bool SUB, bool CNT, bool TD>
+__global__ void __launch_bounds__(128, cut_blocks(SUB, NB))
+    cut_walk_kernel(TreeView T, const long long* sink_idx, int n_sink, WalkParams P, SinkOut out,
+                    unsigned long long* stats, int* status) {
+  __shared__ CutStack stacks[4];
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  SinkCounters cnt;
+  int i = 0, slot = 0;
+  float g = 0.0f;
+  bool has = false;
+  if (k < n_sink) {
+    PlainMap<false> map{&T, sink_idx, nullptr, status};
+    has = map(k, i, slot, g);
+    if (!has && sink_idx) {
+      if (out.flux)
+        for (int b = 0; b < (NB > 1 ? T.n_bands : 1); ++b)
+          out.flux[(size_t)b * out.n_out + k] = 0.0f;
+      if (out.counters) reinterpret_cast<int4*>(out.counters)[k] = make_int4(0, 0, 0, 0);
+    }
+  }
+  CSum F[NB];
+  Moments mom;
+  if (__any_sync(0xffffffffu, has))
+    cut_walk<MERGE, MOM, BG, STOP, NB, SUB, CNT, TD>(T, P, has, i, stacks[threadIdx.x >> 5],
+                                                     status, cnt, F, MOM ? &mom : nullptr);
+  if (MOM && has) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      if (out.fvec) out.fvec[(size_t)q * out.n_out + slot] = mom.v[q].get();
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+      if (out.press) out.press[(size_t)q * out.n_out + slot] = mom.v[3 + q].get();
+  }
+  if (has) {
+    if (NB > 1) {
+      // band-major output: band b of sink slot at b * n_out + slot
+#pragma unroll
+      for (int b = 0; b < NB; ++b)
+        if (out.flux && b < T.n_bands) out.flux[(size_t)b * out.n_out + slot] = F[b].get();
+    } else if (out.flux) {
+      out.flux[slot] = F[0].get();
+    }
+    if (out.counters)
+      reinterpret_cast<int4*>(out.counters)[slot] =
+          make_int4(cnt.rays, cnt.segs, cnt.visit, cnt.ref);
+  }
+  if (CNT && stats) add_stats(cnt, stats);
+}
+
+// Batched form: each work item is cut into groups of 32 consecutive sinks, one warp walk
+// per group.
+template <int BS, bool MERGE, bool CNT>
+__global__ void __launch_bounds__(BS, 1024 / BS) cut_walk_batched_kernel(
+    const TreeView* __restrict__ views, float* const* __restrict__ flux_out,
+    const int2* __restrict__ items, int n_items, int item, unsigned* counter, WalkParams P,
+    unsigned long long* stats, int* status) {
+  __shared__ CutStack stacks[BS / 32];
+  CutStack& ws = stacks[threadIdx.x >> 5];
+  const unsigned lane = threadIdx.x & 31u;
+  SinkCounters tot;
+  while (true) {
+    unsigned it = 0;
+    if (lane == 0) it = atomicAdd(counter, 1u);
+    it = __shfl_sync(0xffffffffu, it, 0);
+    if (it >= (unsigned)n_items) break;
+    const int2 w = items[it];
+    const TreeView T = views[w.x];
+    WalkParams Pt = P;  // the coincident-source cut (1e-12 side)^2 of this tree, in fp32
+    const float smin = __fmul_rn(1e-12f, T.side);
+    Pt.smin2 = __fmul_rn(smin, smin);
+    const int end = min(w.y + item, T.n_gas);
+    for (int g0 = w.y; g0 < end; g0 += 32) {
+      const int i = g0 + (int)lane;
+      const bool has = i < end;
+      CSum F;
+      cut_walk<MERGE, false, false, false, 1, false, CNT, false>(T, Pt, has, i, ws, status, tot,
+                                                                 &F, nullptr);
+      if (has) flux_out[w.x][T.perm[i]] = F.get();
+    }
+  }
+  if (CNT && stats) add_stats(tot, stats);
+}
+
+template <bool MERGE, bool MOM, bool BG, bool STOP, int NB, bool SUB, bool TD>
+cudaError_t launch(const TreeView& T, const long long* sink_idx, int n_sink, const WalkParams& wp,
+                   const SinkOut& out, unsigned long long* stats, int* status, cudaStream_t s) {
+  const int grid = (n_sink + 127) / 128;
+  if (!MOM && (out.counters || stats))
+    cut_walk_kernel<MERGE, MOM, BG, STOP, NB, SUB, !MOM, TD>
+        <<<grid, 128, 0, s>>>(T, sink_idx, n_sink, wp, out, stats, status);
+  else  // no counters asked for: the walk keeps none
+    cut_walk_kernel<MERGE, MOM, BG, STOP, NB, SUB, false, TD>
+        <<<grid, 128, 0, s>>>(T, sink_idx, n_sink, wp, out, nullptr, status);
+  note_launch();
+  return cudaGetLastError();
+}
+
+template <int BS, bool MERGE, bool CNT>
+void launch_batched(const TreeView* views, float* const* flux_out, const int2* items, int n_items,
+                    int item, unsigned* counter, const WalkParams& wp, unsigned long long* stats,
+                    int* status, int n_sm, cudaStream_t s) {
+  int per_sm = 1;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cut_walk_batched_kernel<BS, MERGE, CNT>,
+                                                BS, 0);
+  cut_walk_batched_kernel<BS, MERGE, CNT><<<n_sm * per_sm, BS, 0, s>>>(
+      views, flux_out, items, n_items, item, counter, wp, stats, status);
+}
+
+template <int BS>
+void launch_batched(const TreeView* views, float* const* flux_out, const int2* items, int n_items,
+                    int item, unsigned* counter, const WalkParams& wp, unsigned long long* stats,
+                    int* status, int n_sm, cudaStream_t s) {
+  auto go = [&](auto f) {
+    f(views, flux_out, items, n_items, item, counter, wp, stats, status, n_sm, s);
+  };
+  if (wp.variant == 3) stats ? go(launch_batched<BS, true, true>) : go(launch_batched<BS, true, false>);
+  else stats ? go(launch_batched<BS, false, true>) : go(launch_batched<BS, false, false>);
+}
+
+}  // namespace
+
+cudaError_t launch_cut_batched(const TreeView* views, float* const* flux_out, const int2* items,
+                               int n_items, int item, unsigned* counter, const WalkParams& wp,
+                               unsigned long long* stats, int* status, int block_size, int n_sm,
+                               cudaStream_t s) {
+  if (block_size <= 64)
+    launch_batched<64>(views, flux_out, items, n_items, item, counter, wp, stats, status, n_sm, s);
+  else if (block_size <= 128)
+    launch_batched<128>(views, flux_out, items, n_items, item, counter, wp, stats, status, n_sm,
+                        s);
+  else
+    launch_batched<256>(views, flux_out, items, n_items, item, counter, wp, stats, status, n_sm,
+                        s);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_walk_moments(const TreeView& T, const long long* sink_idx, int n_sink,
+                                const WalkParams& wp, float* flux_out, float* fvec, float* press,
+                                int* status, cudaStream_t s) {
+  if (n_sink <= 0) return cudaSuccess;
+  return launch<true, true, false, false, 1, false, false>(
+      T, sink_idx, n_sink, wp, SinkOut{flux_out, nullptr, fvec, press, n_sink}, nullptr, status, s);
+}
+
+// Several bands: 2 band slots for 2 bands, 4 slots for 3 or 4 (an unused slot holds
+// zeros and is not written). One band is the plain walk.
+cudaError_t launch_walk_bands(const TreeView& T, const long long* sink_idx, int n_sink,
+                              const WalkParams& wp, float* flux_out, int* counters,
+                              unsigned long long* stats, int* status, cudaStream_t s) {
+  if (n_sink <= 0) return cudaSuccess;
+  const SinkOut o{flux_out, counters, nullptr, nullptr, n_sink};
+  if (T.n_bands <= 2)
+    return launch<true, false, false, false, 2, false, false>(T, sink_idx, n_sink, wp, o, stats,
+                                                              status, s);
+  return launch<true, false, false, false, 4, false, false>(T, sink_idx, n_sink, wp, o, stats,
+                                                            status, s);
+}
+
+cudaError_t launch_cut_walk(const TreeView& T, const long long* sink_idx, int n_sink,
+                            const WalkParams& wp, float* flux_out, int* counters,
+                            unsigned long long* stats, int* status, cudaStream_t s) {
+  const SinkOut o{flux_out, counters, nullptr, nullptr, n_sink};
+  const bool bg = wp.bg_radius > 0.0f, stop = wp.tau_stop < INFINITY;
+  if (wp.sub_bucket)
+    return launch<true, false, false, false, 1, true, false>(T, sink_idx, n_sink, wp, o, stats,
+                                                             status, s);
+  if (bg && stop)
+    return launch<true, false, true, true, 1, false, false>(T, sink_idx, n_sink, wp, o, stats,
+                                                            status, s);
+  if (bg)
+    return launch<true, false, true, false, 1, false, false>(T, sink_idx, n_sink, wp, o, stats,
+                                                             status, s);
+  if (stop)
+    return launch<true, false, false, true, 1, false, false>(T, sink_idx, n_sink, wp, o, stats,
+                                                             status, s);
+  if (wp.topdown)
+    return launch<true, false, false, false, 1, false, true>(T, sink_idx, n_sink, wp, o, stats,
+                                                             status, s);
+  if (wp.variant == 3)
+    return launch<true, false, false, false, 1, false, false>(T, sink_idx, n_sink, wp, o, stats,
+                                                              status, s);
+  return launch<false, false, false, false, 1, false, false>(T, sink_idx, n_sink, wp, o, stats,
+                                                             status, s);
+}
+
+}  // namespace trevr

@@ -49,7 +49,10 @@ struct TreeView {
   const float4* nS;  // (cen.x, cen.y, cen.z, L)
   const int4* nT;    // (child or -1, parent, src_first, src_count)
   const float* nl2;  // l^2 (furthest vertex from the centre of luminosity)
-  const float2* nSP; // (split plane relative to lo, split axis as int bits), internal cells
+  const float4* nR;  // what a ray needs of a cell it cuts: (abar, alpha_max - alpha_min, split
+                     // plane relative to lo, bits (child / 2) << 2 | split axis; 3 = leaf)
+  const unsigned long long* nD;  // path from the root: first cut in bit 63 (1 = upper child),
+                                 // then a 1 that ends it, in bit 63 - depth
   const int* ndepth;
   const int4* nglo;  // integer box lower corner, w = split axis (-1 for a leaf)
   const int* nfirst;
@@ -57,6 +60,7 @@ struct TreeView {
   // sources sorted by the first particle of their leaf
   const float4* src;  // (y.x, y.y, y.z, L)
   const int* src_order;
+  const int* src_leaf;  // leaf cell of each sorted source
   const int* n_nodes;  // device scalar
   // several bands (trevr_build_tree_bands): up to 4 per record, unused slots 0
   int n_bands;         // 0 for a single-band tree
@@ -112,7 +116,8 @@ struct trevr_tree {
   float4* nS;
   int4* nT;
   float* nl2;
-  float2* nSP;
+  float4* nR;
+  unsigned long long* nD;
   int* ndepth;
   int* nfirst;
   int* ncount;
@@ -215,6 +220,15 @@ cudaError_t launch_walk(const TreeView& T, const long long* sink_idx, int n_sink
 cudaError_t launch_walk_bands(const TreeView& T, const long long* sink_idx, int n_sink,
                               const WalkParams& wp, float* flux_out, int* counters,
                               unsigned long long* stats, int* status, cudaStream_t s);
+
+// ---- cutwalk.cu: the warp variants (2, 3) of the flux, with every option
+cudaError_t launch_cut_walk(const TreeView& T, const long long* sink_idx, int n_sink,
+                            const WalkParams& wp, float* flux_out, int* counters,
+                            unsigned long long* stats, int* status, cudaStream_t s);
+cudaError_t launch_cut_batched(const TreeView* views, float* const* flux_out, const int2* items,
+                               int n_items, int item, unsigned* counter, const WalkParams& wp,
+                               unsigned long long* stats, int* status, int block_size, int n_sm,
+                               cudaStream_t s);
 
 // ---- adjoint.cu: from the cell accumulators to the caller's gradients
 cudaError_t adjoint_finalize(const trevr_tree* t, const AdjointArgs& J, float* grad_lum,

@@ -17,70 +17,41 @@
 // corner (planes g * h), so their fp32 rounding depends on the domain's size and not
 // on its offset from the origin.
 //
-// GPU form (sinks in Morton order, so the lanes of a warp are neighbours in space).
-//   * Variant 1 (walk_kernel): one lane per sink, a flat loop in which one
-//     iteration is a walk step or a cell clip, cells picked with selects from one
-//     per-lane list; a lane that finishes takes the next sink of its warp's chunk.
-//   * Variant 2 (walk_warp_kernel, MERGE = false): the 32 lanes walk one shared
-//     stack in shared memory with a mask of the lanes that still need each cell,
-//     and trace together the rays to a cell they accept together.
-//   * Variant 3 (MERGE = true, the default): as 2, but a lane keeps its next ray
-//     pending, and the pending rays of all lanes (to different cells) are traced
-//     together, so more lanes share each traced step.
-//   * The segment cells of a ray are known without following parent links: the
-//     sibling of a cell is its index XOR 1 (children are allocated in pairs) and
-//     the common ancestor's depth is the length of the common prefix of the
-//     sink's ancestor list and the walk path, kept as a 64-bit mask. Refined
-//     children are clipped after the ray's base segments.
-// Template options of the warp walk: ADJ (adjoint accumulation, Sec. 2.2 with the
-// decisions frozen), MOM (flux vector and pressure moments), BG (background
-// sources moved onto a sphere), STOP (early ray termination), NB (several bands)
-// and SUB (sub-bucket particle trace).
+// GPU form (sinks in Morton order, so the lanes of a warp are neighbours in space). This
+// file has the walks that clip every cell of a ray by itself:
+//   * Variant 1 (walk_kernel): one lane per sink, a flat loop in which one iteration is a
+//     walk step or a cell clip, cells picked with selects from one per-lane list; a lane
+//     that finishes takes the next sink of its warp's chunk.
+//   * walk_warp_kernel: the adjoint of variants 2 and 3, and the flux with early ray
+//     termination when counters are asked for (the segments of a ray that is cut off are
+//     counted in this walk's order). The 32 lanes walk one shared stack with a mask of the
+//     lanes that still need each cell; with MERGE a lane keeps its next ray pending, and the
+//     pending rays of all lanes (to different cells) are traced together.
+// The flux of variants 2 and 3 is in cutwalk.cu.
+//   * The segment cells of a ray are known without following parent links: the sibling of a
+//     cell is its index XOR 1 (children are allocated in pairs) and the common ancestor's
+//     depth is the length of the common prefix of the sink's ancestor list and the walk
+//     path, kept as a 64-bit mask. Refined children are clipped after the ray's base
+//     segments.
+// Template options of the warp walk: ADJ (adjoint accumulation, Sec. 2.2 with the decisions
+// frozen), BG (background sources moved onto a sphere), STOP (early ray termination).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include "trevr_internal.cuh"
+#include "walk_common.cuh"
 
 namespace trevr {
 
 namespace {
 
-constexpr int kDepth = 64;  // > max cell depth (63): lists and stacks never overflow
 constexpr int kAnc = 0;     // offsets of the three parts of the per-lane list
 constexpr int kPath = kDepth;
 constexpr int kRef = 2 * kDepth;
-constexpr float kFourPi = 12.566370614359172f;
 // refinement stack of the warp walk: refined base segments (at most 2 x 63 + 1) are
 // queued first, then each popped pair adds at most one entry per level below
 constexpr int kRayStack = 4 * kDepth;
 constexpr int kSegBuf = 64;  // segments of one ray kept for the adjoint's second pass
-
-// Neumaier-compensated fp32 sum.
-struct CSum {
-  float s = 0.0f, c = 0.0f;
-  __device__ __forceinline__ void add(float x) {
-    float t = __fadd_rn(s, x);
-    if (fabsf(s) >= fabsf(x)) c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, t), x));
-    else c = __fadd_rn(c, __fadd_rn(__fsub_rn(x, t), s));
-    s = t;
-  }
-  __device__ __forceinline__ float get() const { return __fadd_rn(s, c); }
-};
-
-// Kahan-compensated fp32 running sum (branch-free), for the optical depth of one
-// ray in the warp walks: c carries the low-order part that each addition loses,
-// so the error of the sum stays within about 2 ulp of the total however many
-// terms a refined ray has.
-struct KSum {
-  float s = 0.0f, c = 0.0f;
-  __device__ __forceinline__ void add(float x) {
-    const float y = __fsub_rn(x, c);
-    const float t = __fadd_rn(s, y);
-    c = __fsub_rn(__fsub_rn(t, s), y);
-    s = t;
-  }
-  __device__ __forceinline__ float get() const { return s; }
-};
 
 // one slab of the clip: (lo - p) * (1/d), (hi - p) * (1/d), rounded after each step;
 // along an axis the ray does not move on, the box is half-open [lo, hi), so a ray
@@ -136,25 +107,6 @@ __device__ __forceinline__ void slab_g(int k, float lo, float hi, float p, float
 }
 
 }  // namespace
-
-struct SinkCounters {
-  int rays = 0, segs = 0, visit = 0, ref = 0, clip = 0, cut = 0, sub = 0;
-};
-
-// warp-reduce the counters and add them to the device totals (all lanes call it)
-__device__ __forceinline__ void add_stats(const SinkCounters& c, unsigned long long* stats) {
-  unsigned long long v[7] = {(unsigned long long)c.rays, (unsigned long long)c.segs,
-                             (unsigned long long)c.visit, (unsigned long long)c.ref,
-                             (unsigned long long)c.clip, (unsigned long long)c.cut,
-                             (unsigned long long)c.sub};
-#pragma unroll
-  for (int q = 0; q < 7; ++q) {
-    unsigned long long x = v[q];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    if ((threadIdx.x & 31) == 0 && x) atomicAdd(&stats[q], x);
-  }
-}
 
 // Per-lane lists, kept apart from the scalar state so that the state stays in
 // registers: the ancestors of S | the depth-first path | cells to clip, and the
@@ -416,21 +368,6 @@ struct Lane {
   }
 };
 
-// Where a finished sink's results go.
-struct SinkOut {
-  float* flux;    // flux per sink (caller order), or nullptr
-  int* counters;  // 4 int per sink, or nullptr
-  float* fvec;    // flux vector, 3 x n_sink (SoA), or nullptr
-  float* press;   // second moment, 6 x n_sink (SoA: xx yy zz xy xz yz), or nullptr
-  int n_out;      // n_sink (stride of the SoA blocks)
-};
-
-// Direction moments of the intensity at one sink: sum f n and sum f n n^T, n the
-// unit vector from the pseudo-source to the sink (Eq. simpflux; Sec. 2.1).
-struct Moments {
-  CSum v[9];  // x y z | xx yy zz xy xz yz
-};
-
 // Runs the sinks [first, end) of a chunk with one warp: the lanes start on the
 // first 32 and take the next unclaimed sink of the chunk when theirs is done.
 // `map` turns a chunk position into (sorted position, output slot, dLoss/dF);
@@ -484,31 +421,6 @@ __device__ __forceinline__ void run_chunk(const TreeView& T, const WalkParams& P
     }
   }
 }
-
-// Sinks of a plain call: chunk position k is the k-th requested sink.
-template <bool ADJ>
-struct PlainMap {
-  const TreeView* T;
-  const long long* sink_idx;
-  const float* grad_flux;
-  int* status;
-  __device__ __forceinline__ bool operator()(int k, int& i, int& slot, float& g) const {
-    if (sink_idx) {
-      const long long si = sink_idx[k];
-      if (si < 0 || si >= T->n_gas) {
-        atomicOr(status, kStatusInvalid);
-        return false;
-      }
-      i = T->rank[si];
-      slot = k;
-    } else {
-      i = k;
-      slot = T->perm[k];
-    }
-    g = ADJ ? grad_flux[slot] : 0.0f;
-    return !ADJ || g != 0.0f;  // the adjoint skips sinks with dLoss/dF = 0
-  }
-};
 
 template <bool ADJ>
 __global__ void __launch_bounds__(128) walk_kernel(TreeView T, const long long* sink_idx,
@@ -610,134 +522,11 @@ __device__ __forceinline__ void warp_atomic_add(double* base, int key, float v) 
   }
 }
 
-// ---------------------------------------------------------------------------
-// Sub-bucket particle trace (Sec. 2.2.3, 3.1.3). The absorption below the bucket
-// scale is the SPH field sum_j alpha_j w_j W(|x - x_j|, h_j), W(r, h) = w(r/h)/(pi h^3)
-// the cubic spline of support 2h. Along a ray at impact parameter b from x_j, with s
-// measured from the closest approach, the column over [s0, s1] is
-// (Phi(x, s1/h) - Phi(x, s0/h)) / (pi h^2), x = b^2/h^2, where Phi(x, sigma) is the
-// integral of w(sqrt(x + t^2)) over t in [0, sigma]: odd in sigma and constant beyond
-// the support. Phi comes from the tree's pre-computed table (the paper's pre-computed
-// kernel integral), bilinear in (x, sigma).
-__device__ __forceinline__ float kint_phi(const float4* __restrict__ tab, float x, float sigma) {
-  const float a = fminf(fabsf(sigma), 2.0f);
-  const float fx = x * (0.25f * (float)kKintNX), fs = a * (0.5f * (float)kKintNS);
-  const int i = min((int)fx, kKintNX - 1), j = min((int)fs, kKintNS - 1);
-  const float u = fx - (float)i, v = fs - (float)j;
-  const float4 c = __ldg(tab + (size_t)i * kKintNS + j);  // the cell's four corners
-  const float p0 = fmaf(v, c.y - c.x, c.x);
-  const float p1 = fmaf(v, c.w - c.z, c.z);
-  const float p = fmaf(u, p1 - p0, p0);
-  return sigma < 0.0f ? -p : p;
-}
-
-// Per-warp queue of the neighbours whose support meets the chord, so that the
-// quadrature runs on full warps: (x, sigma_0, sigma_1, alpha w / (pi h^2)).
-struct SubQueue {
-  float4 g[64];
-};
-
-// Optical depth of lane src's chord p + t d, t in [t0, t1], through the particles
-// listed for its leaf, the receiving particle (sorted index si) left out. The 32
-// lanes of the warp test one neighbour each per round, with the next round's
-// entries already loading; the neighbours that reach the chord are queued in shared
-// memory and integrated 32 at a time: (Phi(x, sigma_1) - Phi(x, sigma_0)) times
-// alpha w / (pi h^2), with x = b^2 / h^2 and sigma = s / h. Every lane must call it;
-// all lanes return the sum.
-__device__ __forceinline__ float sub_bucket_tau_warp(const TreeView& T, int src, int box, int si,
-                                                     float px, float py, float pz, float dx,
-                                                     float dy, float dz, float s2, float len,
-                                                     float t0, float t1) {
-  const unsigned FULL = 0xffffffffu;
-  const unsigned lane = threadIdx.x & 31u;
-  __shared__ SubQueue queues[4];  // one per warp of a 128-thread block
-  SubQueue& Q = queues[threadIdx.x >> 5];
-  box = __shfl_sync(FULL, box, src);
-  si = __shfl_sync(FULL, si, src);
-  px = __shfl_sync(FULL, px, src);
-  py = __shfl_sync(FULL, py, src);
-  pz = __shfl_sync(FULL, pz, src);
-  dx = __shfl_sync(FULL, dx, src);
-  dy = __shfl_sync(FULL, dy, src);
-  dz = __shfl_sync(FULL, dz, src);
-  s2 = __shfl_sync(FULL, s2, src);
-  len = __shfl_sync(FULL, len, src);
-  t0 = __shfl_sync(FULL, t0, src);
-  t1 = __shfl_sync(FULL, t1, src);
-  const float inv_s2 = 1.0f / s2;
-  float part = 0.0f;
-  int qn = 0;  // queued entries (warp-uniform)
-  const unsigned k0 = __ldg(&T.nbr_first[box]), k1 = __ldg(&T.nbr_first[box + 1]);
-  int2 nja = make_int2(-1, 0);  // the next round's entries
-  float4 nq = make_float4(0.0f, 0.0f, 0.0f, 1.0f);
-  if (k0 + lane < k1) {
-    nja = __ldg(&T.nbr_ja[k0 + lane]);
-    nq = __ldg(&T.nbr_sp[k0 + lane]);
-  }
-  for (unsigned base = k0; base < k1; base += 32u) {
-    const unsigned k = base + lane;
-    const int2 ja = nja;
-    const float4 q = nq;
-    if (k + 32u < k1) {
-      nja = __ldg(&T.nbr_ja[k + 32u]);
-      nq = __ldg(&T.nbr_sp[k + 32u]);
-    }
-    const float a = __int_as_float(ja.y);
-    bool pass = false;
-    float x = 0.0f, sa = 0.0f, sb = 0.0f;
-    if (k < k1 && ja.x != si && a > 0.0f) {
-      const float ux = q.x - px, uy = q.y - py, uz = q.z - pz;
-      const float tc = (ux * dx + uy * dy + uz * dz) * inv_s2;
-      const float ex = ux - tc * dx, ey = uy - tc * dy, ez = uz - tc * dz;
-      const float b2 = ex * ex + ey * ey + ez * ez;
-      const float ih = q.w;
-      x = b2 * ih * ih;
-      sa = ((t0 - tc) * len) * ih;
-      sb = ((t1 - tc) * len) * ih;
-      if (x < 4.0f) {  // the chord [sa, sb] must meet the support |sigma| < sqrt(4 - x)
-        const float u22 = 4.0f - x;
-        pass = (sb > 0.0f || sb * sb < u22) && (sa < 0.0f || sa * sa < u22);
-      }
-    }
-    const unsigned m = __ballot_sync(FULL, pass);
-    if (pass) {
-      const float ih = q.w;
-      Q.g[qn + __popc(m & ((1u << lane) - 1u))] =
-          make_float4(x, sa, sb, a * (ih * ih * 0.318309886f));
-    }
-    qn += __popc(m);
-    __syncwarp();
-    if (qn >= 32) {
-      const float4 g = Q.g[qn - 32 + (int)lane];
-      part += g.w * (kint_phi(T.kint4, g.x, g.z) - kint_phi(T.kint4, g.x, g.y));
-      qn -= 32;
-      __syncwarp();
-    }
-  }
-  if ((int)lane < qn) {
-    const float4 g = Q.g[lane];
-    part += g.w * (kint_phi(T.kint4, g.x, g.z) - kint_phi(T.kint4, g.x, g.y));
-  }
-  __syncwarp();
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(FULL, part, o);
-  return part;
-}
-
 // Rays from the sinks of the lanes in `on` to (q, L) inside cell C; every lane
 // of the warp must call it (the loop runs while any lane has cells left).
 // STOP: early ray termination (Sec. 4): a lane whose running optical depth passes
 // P.tau_stop drops the rest of its ray, and the ray adds nothing.
-// NB > 1: several bands (2 or 4 slots of the band records): every band sums its own
-// optical depth over the shared segments, and F[b] gets band b's flux.
-// SUB: the sub-bucket particle trace for leaves whose own particles ask for
-// refinement (the sink's sorted index si is left out of the sum).
-// TD: the top-down ray walk (Sec. 3.1.3, Sec. 4): the ray's only base segment is the
-// common ancestor A = path[d*], and Eq. refcrit alone splits it through the same
-// refinement stack; without TD the base segments are C, the siblings up both paths
-// and S, as in the paper's walk.
-template <bool ADJ, bool MOM, bool STOP = false, int NB = 1, bool SUB = false, bool CNT = true,
-          bool TD = false>
+template <bool ADJ, bool STOP, bool CNT>
 __device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P, const bool on,
                                          const float px, const float py, const float pz,
                                          const int S, const int dS, const int* anc, int* rst,
@@ -746,15 +535,10 @@ __device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P,
                                          const float qy, const float qz, const float L,
                                          const int src_j, const float gk, const int stack_limit,
                                          const int box_limit, int* status, const AdjointArgs& J,
-                                         SinkCounters& cnt, CSum* F, Moments* mom,
-                                         const int si = -1) {
-  static_assert(NB == 1 || NB == 2 || NB == 4, "band slots: 1, 2 or 4");
-  static_assert(!SUB || (!ADJ && !MOM && !STOP && NB == 1), "sub-bucket trace: plain flux only");
-  static_assert(NB == 1 || !(ADJ || MOM || STOP), "bands: plain flux only");
+                                         SinkCounters& cnt, CSum* F) {
   const unsigned FULL = 0xffffffffu;
   float dx = 0.0f, dy = 0.0f, dz = 0.0f, s2 = 1.0f, len = 1.0f, ix = 0.0f, iy = 0.0f, iz = 0.0f;
   int nCs = 0, nSs = 0, nb = 0, dstar = 0;
-  int base1 = S;  // the base segment of a one-segment ray: S, or A for the top-down walk
   bool active = false;
   if (on) {
     dx = __fsub_rn(qx, px);
@@ -773,21 +557,15 @@ __device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P,
         const int mn = dC < dS ? dC : dS;
         const unsigned long long m = on_path & ((2ull << mn) - 1ull);  // mn <= 62
         dstar = __ffsll((long long)~m) - 2;
-        if (TD) {
-          nb = 1;
-          base1 = path[dstar];
-        } else {
-          nCs = dC - dstar - 1;
-          nSs = dS - dstar - 1;
-          nb = nCs + nSs + 2;
-        }
+        nCs = dC - dstar - 1;
+        nSs = dS - dstar - 1;
+        nb = nCs + nSs + 2;
       }
     }
   }
   const bool traced = active;
   const bool nz = dx != 0.0f && dy != 0.0f && dz != 0.0f;  // the ray moves along every axis
   KSum tau;
-  KSum taub[NB];  // (NB > 1) optical depth of each band
   bool cut = false;
   int b = 0, rsp = 0, boxes = 0, pass = 1;
   int slot = -1;  // the upper child of the pair popped last: clipped next
@@ -798,9 +576,6 @@ __device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P,
   int nseg = 0, kk = 0;
   bool seg_over = false;
   float gq0 = 0.0f, gq1 = 0.0f, gq2 = 0.0f, fcur = 0.0f;
-  bool need_sub = false;  // (SUB) this step's leaf is traced through its particles
-  int sub_box = 0;
-  float sub_t0 = 0.0f, sub_t1 = 0.0f;
   while (__any_sync(FULL, active)) {
     int akey = -1;
     float aval = 0.0f;
@@ -825,31 +600,7 @@ __device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P,
           if (CNT) ++cnt.rays;
           active = false;
         } else if (!ADJ) {
-          if (NB > 1) {
-            // the band luminosities of the source, or of the merged cell C
-            const float4 Lb = src_j >= 0 ? __ldg(&T.bLs[src_j]) : __ldg(&T.bLc[C]);
-            F[0].add(Lb.x * expf(-taub[0].get()) / (kFourPi * s2));
-            F[1].add(Lb.y * expf(-taub[1].get()) / (kFourPi * s2));
-            if (NB > 2) {
-              F[NB > 2 ? 2 : 0].add(Lb.z * expf(-taub[NB > 2 ? 2 : 0].get()) / (kFourPi * s2));
-              F[NB > 2 ? 3 : 0].add(Lb.w * expf(-taub[NB > 2 ? 3 : 0].get()) / (kFourPi * s2));
-            }
-          } else {
-            F[0].add(f);
-          }
-          if (MOM) {
-            const float il = 1.0f / len;
-            const float n0 = -dx * il, n1 = -dy * il, n2 = -dz * il;
-            mom->v[0].add(f * n0);
-            mom->v[1].add(f * n1);
-            mom->v[2].add(f * n2);
-            mom->v[3].add(f * n0 * n0);
-            mom->v[4].add(f * n1 * n1);
-            mom->v[5].add(f * n2 * n2);
-            mom->v[6].add(f * n0 * n1);
-            mom->v[7].add(f * n0 * n2);
-            mom->v[8].add(f * n1 * n2);
-          }
+          F[0].add(f);
           if (CNT) ++cnt.rays;
           active = false;
         } else if (pass == 1) {
@@ -887,7 +638,7 @@ __device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P,
           }
         } else {
           if (nb == 1) {
-            box = base1;
+            box = S;
           } else if (b <= nCs) {  // C = path[dC], then the siblings up C's path
             box = path[dC - max(b - 1, 0)] ^ (b > 0 ? 1 : 0);
           } else {  // the siblings down S's path, then S = anc[dS]
@@ -944,9 +695,9 @@ __device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P,
                   // (22 % fewer clips on the clumpy workload, bit-identical fluxes).
                   bool lo_t = true, hi_t = true;
                   {
-                    const float2 sp = __ldg(&T.nSP[box]);
-                    const int ax = __float_as_int(sp.y);
-                    const float Pl = sp.x;
+                    const float4 r = __ldg(&T.nR[box]);
+                    const int ax = (int)(__float_as_uint(r.w) & 3u);
+                    const float Pl = r.z;
                     const float pa = ax == 0 ? px : (ax == 1 ? py : pz);
                     const float ia = ax == 0 ? ix : (ax == 1 ? iy : iz);
                     if (ia != 0.0f) {
@@ -970,26 +721,7 @@ __device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P,
                 akey = box;
                 aval = -gk * fcur * l;
               } else {
-                if (NB > 1) {
-                  const float4 ab = __ldg(&T.bA[box]);
-                  taub[0].add(__fmul_rn(ab.x, l));
-                  taub[1].add(__fmul_rn(ab.y, l));
-                  if (NB > 2) {
-                    taub[NB > 2 ? 2 : 0].add(__fmul_rn(ab.z, l));
-                    taub[NB > 2 ? 3 : 0].add(__fmul_rn(ab.w, l));
-                  }
-                } else if (SUB && (P.tau_ref <= 0.0f ||
-                                   __fmul_rn(__ldg(&T.dbk[box]), l) > P.tau_ref)) {
-                  // a bucket that still asks for refinement: its particles are traced
-                  // by the whole warp at the end of this step
-                  need_sub = true;
-                  sub_box = box;
-                  sub_t0 = t0;
-                  sub_t1 = t1;
-                  if (CNT) ++cnt.sub;
-                } else {
-                  tau.add(__fmul_rn(a.w, l));
-                }
+                tau.add(__fmul_rn(a.w, l));
                 if (!ADJ && STOP && tau.get() > P.tau_stop) {
                   cut = true;  // the rest of the ray is not traced
                   b = nb;
@@ -1020,18 +752,6 @@ __device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P,
           }
         }
       }
-    }
-    if (SUB) {
-      // the leaves of this step that need the particle trace, one after another
-      unsigned m = __ballot_sync(FULL, need_sub);
-      while (m) {
-        const int src = __ffs(m) - 1;
-        m &= m - 1u;
-        const float t = sub_bucket_tau_warp(T, src, sub_box, si, px, py, pz, dx, dy, dz, s2, len,
-                                            sub_t0, sub_t1);
-        if ((int)(threadIdx.x & 31u) == src) tau.add(t);
-      }
-      need_sub = false;
     }
     // a retraced segment's gradient (a ray with more segments than were recorded): the
     // lanes trace different rays, so the cells differ and each lane adds its own, as the
@@ -1108,12 +828,11 @@ __device__ __forceinline__ void bg_move(const TreeView& T, const WalkParams& P, 
 // o before its ray is traced, in fp32 as d = c - o, s = sqrt((dx^2 + dy^2) + dz^2),
 // q = o + d * (R / s); the ray then ends in the leaf that holds q, whose ancestors the
 // lane finds by descending the cut planes from the root and keeps for that ray.
-template <bool ADJ, bool MERGE, bool MOM = false, bool BG = false, bool STOP = false, int NB = 1,
-          bool SUB = false, bool CNT = true, bool TD = false>
+template <bool ADJ, bool MERGE, bool BG, bool STOP, bool CNT>
 __device__ __forceinline__ void warp_walk(const TreeView& T, const WalkParams& P, const bool has,
                                           const int i, const float gk, WarpStack& ws,
                                           int* status, const AdjointArgs& J,
-                                          SinkCounters& cnt, CSum* F, Moments* mom = nullptr) {
+                                          SinkCounters& cnt, CSum* F) {
   const unsigned FULL = 0xffffffffu;
   const unsigned lane = threadIdx.x & 31u;
   const int stack_limit = P.stack_depth < kDepth ? P.stack_depth : kDepth;
@@ -1161,13 +880,11 @@ __device__ __forceinline__ void warp_walk(const TreeView& T, const WalkParams& P
         for (int d = 0; d <= mn && cpath[d] == anc[d]; ++d) onp |= 1ull << d;
         pp = cpath;
       }
-      warp_ray<ADJ, MOM, STOP, NB, SUB, CNT, TD>(T, P, pnd, px, py, pz, S, dS, anc, rst, onp, pp, pC, pdC, pqx, pqy,
-                         pqz, pL, psrc, gk, stack_limit, box_limit, status, J, cnt, F, mom,
-                         i);
+      warp_ray<ADJ, STOP, CNT>(T, P, pnd, px, py, pz, S, dS, anc, rst, onp, pp, pC, pdC, pqx, pqy,
+                         pqz, pL, psrc, gk, stack_limit, box_limit, status, J, cnt, F);
     } else {
-      warp_ray<ADJ, MOM, STOP, NB, SUB, CNT, TD>(T, P, pnd, px, py, pz, S, dS, anc, rst, on_path, ws.path, pC, pdC,
-                         pqx, pqy, pqz, pL, psrc, gk, stack_limit, box_limit, status, J, cnt, F,
-                         mom, i);
+      warp_ray<ADJ, STOP, CNT>(T, P, pnd, px, py, pz, S, dS, anc, rst, on_path, ws.path, pC, pdC,
+                         pqx, pqy, pqz, pL, psrc, gk, stack_limit, box_limit, status, J, cnt, F);
     }
     pnd = false;
     pbg = false;
@@ -1218,9 +935,8 @@ __device__ __forceinline__ void warp_walk(const TreeView& T, const WalkParams& P
         }
       }
     } else if (accM) {
-      warp_ray<ADJ, MOM, STOP, NB, SUB, CNT, TD>(T, P, acc, px, py, pz, S, dS, anc, rst, on_path, ws.path, X, dX, s.x,
-                         s.y, s.z, s.w, -1, gk, stack_limit, box_limit, status, J, cnt, F, mom,
-                         i);
+      warp_ray<ADJ, STOP, CNT>(T, P, acc, px, py, pz, S, dS, anc, rst, on_path, ws.path, X, dX, s.x,
+                         s.y, s.z, s.w, -1, gk, stack_limit, box_limit, status, J, cnt, F);
     }
     if (opnM) {
       const int4 t = __ldg(&T.nT[X]);
@@ -1241,9 +957,8 @@ __device__ __forceinline__ void warp_walk(const TreeView& T, const WalkParams& P
               psrc = jj;
             }
           } else {
-            warp_ray<ADJ, MOM, STOP, NB, SUB, CNT, TD>(T, P, opn, px, py, pz, S, dS, anc, rst, on_path, ws.path, X, dX,
-                               y.x, y.y, y.z, y.w, jj, gk, stack_limit, box_limit, status, J, cnt,
-                               F, mom, i);
+            warp_ray<ADJ, STOP, CNT>(T, P, opn, px, py, pz, S, dS, anc, rst, on_path, ws.path, X, dX,
+                               y.x, y.y, y.z, y.w, jj, gk, stack_limit, box_limit, status, J, cnt, F);
           }
         }
       } else {
@@ -1267,25 +982,14 @@ __device__ __forceinline__ void warp_walk(const TreeView& T, const WalkParams& P
   if (MERGE && __any_sync(FULL, pnd)) flush();
 }
 
-// 8 blocks of 128 per SM (at most 64 registers): measured 4% faster forward and 8%
-// faster adjoint than the compiler's own 70 registers at 7 blocks. The adjoint keeps
-// no counters (the backward call reports none) and stays at 8 blocks: 3% faster
-// than with counters; 10 and 12 blocks spilled and were 6% and 13% slower. Without
-// counters (CNT = false, the plain flux when the caller asks for no counters or
-// stats) the walk runs 12 blocks (40 registers, spilling to L1): 2.7% faster than
-// 9 blocks (56 registers) on the clumpy workload, 119.8 against 123.2 ms; 10
-// blocks were slower (141 ms).
-// CNT = false keeps no per-sink counters; the fluxes are bit-identical. The band
-// walks without counters fit 6 blocks (74 registers, no spills) instead of 4:
-// 245 ms against 262 ms for four bands on the clumpy workload. The sub-bucket walk
-// runs 8 blocks (64 registers, spilling): 325.6 ms against 343.0 ms at 4 blocks
-// (114 registers) on 2^18 particles, without counters.
-template <bool ADJ, bool MERGE, bool MOM = false, bool BG = false, bool STOP = false, int NB = 1,
-          bool SUB = false, bool CNT = true, bool TD = false>
-__global__ void __launch_bounds__(128, SUB ? 8 : ADJ ? 8 : (NB > 1 ? (CNT ? 4 : 6) : (CNT ? 8 : 12))) walk_warp_kernel(TreeView T, const long long* sink_idx,
-                                                        int n_sink, WalkParams P, SinkOut out,
-                                                        unsigned long long* stats, int* status,
-                                                        AdjointArgs J) {
+// 8 blocks of 128 per SM (at most 64 registers): measured 8% faster for the adjoint than
+// the compiler's own 70 registers at 7 blocks; 10 and 12 blocks spilled and were 6% and 13%
+// slower. The adjoint keeps no counters (the backward call reports none).
+template <bool ADJ, bool MERGE, bool BG, bool STOP, bool CNT>
+__global__ void __launch_bounds__(128, 8) walk_warp_kernel(TreeView T, const long long* sink_idx,
+                                                           int n_sink, WalkParams P, SinkOut out,
+                                                           unsigned long long* stats, int* status,
+                                                           AdjointArgs J) {
   __shared__ WarpStack stacks[4];
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   WarpStack& ws = stacks[threadIdx.x >> 5];
@@ -1297,82 +1001,20 @@ __global__ void __launch_bounds__(128, SUB ? 8 : ADJ ? 8 : (NB > 1 ? (CNT ? 4 : 
     PlainMap<ADJ> map{&T, sink_idx, J.grad_flux, status};
     has = map(k, i, slot, g);
     if (!has && !ADJ && sink_idx) {
-      if (out.flux)
-        for (int b = 0; b < (NB > 1 ? T.n_bands : 1); ++b) out.flux[(size_t)b * out.n_out + k] = 0.0f;
+      if (out.flux) out.flux[k] = 0.0f;
       if (out.counters) reinterpret_cast<int4*>(out.counters)[k] = make_int4(0, 0, 0, 0);
     }
   }
-  CSum F[NB];
-  Moments mom;
+  CSum F;
   if (__any_sync(0xffffffffu, has))
-    warp_walk<ADJ, MERGE, MOM, BG, STOP, NB, SUB, CNT, TD>(T, P, has, i, g, ws, status, J, cnt, F,
-                                                  MOM ? &mom : nullptr);
-  if (MOM && has) {
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-      if (out.fvec) out.fvec[(size_t)q * out.n_out + slot] = mom.v[q].get();
-#pragma unroll
-    for (int q = 0; q < 6; ++q)
-      if (out.press) out.press[(size_t)q * out.n_out + slot] = mom.v[3 + q].get();
-  }
+    warp_walk<ADJ, MERGE, BG, STOP, CNT>(T, P, has, i, g, ws, status, J, cnt, &F);
   if (!ADJ && has) {
-    if (NB > 1) {
-      // band-major output: band b of sink slot at b * n_out + slot
-#pragma unroll
-      for (int b = 0; b < NB; ++b)
-        if (out.flux && b < T.n_bands) out.flux[(size_t)b * out.n_out + slot] = F[b].get();
-    } else if (out.flux) {
-      out.flux[slot] = F[0].get();
-    }
+    if (out.flux) out.flux[slot] = F.get();
     if (out.counters)
-      reinterpret_cast<int4*>(out.counters)[slot] = make_int4(cnt.rays, cnt.segs, cnt.visit, cnt.ref);
+      reinterpret_cast<int4*>(out.counters)[slot] =
+          make_int4(cnt.rays, cnt.segs, cnt.visit, cnt.ref);
   }
   if (stats) add_stats(cnt, stats);
-}
-
-// Batched form of the warp-shared walk: each work item is cut into groups of 32
-// consecutive sinks, one warp walk per group.
-// CNT = false (no stats asked for): no counters, and 12 blocks-of-128 worth of
-// threads per SM instead of 8, as for the single-tree walk (2.8% faster than 9 on
-// the 64 boxes).
-template <int BS, bool MERGE, bool CNT = true>
-__global__ void __launch_bounds__(BS, CNT ? 1024 / BS : 1536 / BS) walk_warp_batched_kernel(
-    const TreeView* __restrict__ views, float* const* __restrict__ flux_out,
-    const int2* __restrict__ items, int n_items, int item, unsigned* counter, WalkParams P,
-    unsigned long long* stats, int* status) {
-  __shared__ WarpStack stacks[BS / 32];
-  WarpStack& ws = stacks[threadIdx.x >> 5];
-  const unsigned lane = threadIdx.x & 31u;
-  SinkCounters tot;
-  while (true) {
-    unsigned it = 0;
-    if (lane == 0) it = atomicAdd(counter, 1u);
-    it = __shfl_sync(0xffffffffu, it, 0);
-    if (it >= (unsigned)n_items) break;
-    const int2 w = items[it];
-    const TreeView T = views[w.x];
-    WalkParams Pt = P;  // the coincident-source cut (1e-12 side)^2 of this tree, in fp32
-    const float smin = __fmul_rn(1e-12f, T.side);
-    Pt.smin2 = __fmul_rn(smin, smin);
-    const int end = min(w.y + item, T.n_gas);
-    for (int g0 = w.y; g0 < end; g0 += 32) {
-      const int i = g0 + (int)lane;
-      const bool has = i < end;
-      SinkCounters cnt;
-      CSum F;
-      warp_walk<false, MERGE, false, false, false, 1, false, CNT>(T, Pt, has, i, 0.0f, ws, status,
-                                                                 AdjointArgs{}, cnt, &F);
-      if (has) flux_out[w.x][T.perm[i]] = F.get();
-      if (CNT) {
-        tot.rays += cnt.rays;
-        tot.segs += cnt.segs;
-        tot.visit += cnt.visit;
-        tot.ref += cnt.ref;
-        tot.clip += cnt.clip;
-      }
-    }
-  }
-  if (CNT && stats) add_stats(tot, stats);
 }
 
 cudaError_t launch_walk_batched(const TreeView* views, float* const* flux_out, const int2* items,
@@ -1383,35 +1025,10 @@ cudaError_t launch_walk_batched(const TreeView* views, float* const* flux_out, c
   cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
   if (e != cudaSuccess) return e;
   int per_sm = 1;
-  if (wp.variant >= 2) {
-    const int bs = block_size <= 64 ? 64 : (block_size <= 128 ? 128 : 256);
-    const bool merge = wp.variant == 3;
-#define TREVR_WB(BSV, MV)                                                                     \
-  do {                                                                                         \
-    if (stats) {                                                                               \
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_warp_batched_kernel<BSV, MV>, \
-                                                    BSV, 0);                                   \
-      walk_warp_batched_kernel<BSV, MV><<<n_sm * per_sm, BSV, 0, s>>>(                        \
-          views, flux_out, items, n_items, item, counter, wp, stats, status);                  \
-    } else {                                                                                   \
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(                                           \
-          &per_sm, walk_warp_batched_kernel<BSV, MV, false>, BSV, 0);                          \
-      walk_warp_batched_kernel<BSV, MV, false><<<n_sm * per_sm, BSV, 0, s>>>(                 \
-          views, flux_out, items, n_items, item, counter, wp, nullptr, status);                \
-    }                                                                                          \
-  } while (0)
-    if (bs == 64) {
-      if (merge) TREVR_WB(64, true);
-      else TREVR_WB(64, false);
-    } else if (bs == 128) {
-      if (merge) TREVR_WB(128, true);
-      else TREVR_WB(128, false);
-    } else {
-      if (merge) TREVR_WB(256, true);
-      else TREVR_WB(256, false);
-    }
-#undef TREVR_WB
-  } else if (block_size <= 64) {
+  if (wp.variant >= 2)
+    return launch_cut_batched(views, flux_out, items, n_items, item, counter, wp, stats, status,
+                              block_size, n_sm, s);
+  if (block_size <= 64) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_batched_kernel<64>, 64, 0);
     walk_batched_kernel<64><<<n_sm * per_sm, 64, 0, s>>>(views, flux_out, items, n_items, item,
                                                          counter, wp, stats, status);
@@ -1428,42 +1045,6 @@ cudaError_t launch_walk_batched(const TreeView* views, float* const* flux_out, c
   return cudaGetLastError();
 }
 
-cudaError_t launch_walk_moments(const TreeView& T, const long long* sink_idx, int n_sink,
-                                const WalkParams& wp, float* flux_out, float* fvec, float* press,
-                                int* status, cudaStream_t s) {
-  if (n_sink <= 0) return cudaSuccess;
-  walk_warp_kernel<false, true, true><<<(n_sink + 127) / 128, 128, 0, s>>>(
-      T, sink_idx, n_sink, wp, SinkOut{flux_out, nullptr, fvec, press, n_sink}, nullptr, status,
-      AdjointArgs{});
-  note_launch();
-  return cudaGetLastError();
-}
-
-// Several bands: 2 band slots for 2 bands, 4 slots for 3 or 4 (an unused slot holds
-// zeros and is not written). One band is the plain walk.
-cudaError_t launch_walk_bands(const TreeView& T, const long long* sink_idx, int n_sink,
-                              const WalkParams& wp, float* flux_out, int* counters,
-                              unsigned long long* stats, int* status, cudaStream_t s) {
-  if (n_sink <= 0) return cudaSuccess;
-  const dim3 grid((n_sink + 127) / 128);
-  const SinkOut o{flux_out, counters, nullptr, nullptr, n_sink};
-  const bool cnt = counters || stats;
-  if (T.n_bands <= 2 && cnt)
-    walk_warp_kernel<false, true, false, false, false, 2><<<grid, 128, 0, s>>>(
-        T, sink_idx, n_sink, wp, o, stats, status, AdjointArgs{});
-  else if (T.n_bands <= 2)
-    walk_warp_kernel<false, true, false, false, false, 2, false, false><<<grid, 128, 0, s>>>(
-        T, sink_idx, n_sink, wp, o, nullptr, status, AdjointArgs{});
-  else if (cnt)
-    walk_warp_kernel<false, true, false, false, false, 4><<<grid, 128, 0, s>>>(
-        T, sink_idx, n_sink, wp, o, stats, status, AdjointArgs{});
-  else
-    walk_warp_kernel<false, true, false, false, false, 4, false, false><<<grid, 128, 0, s>>>(
-        T, sink_idx, n_sink, wp, o, nullptr, status, AdjointArgs{});
-  note_launch();
-  return cudaGetLastError();
-}
-
 static int chunk_of(const WalkParams& wp) {
   return wp.sinks_per_warp > 0 ? wp.sinks_per_warp : kDefaultChunk;
 }
@@ -1474,72 +1055,21 @@ cudaError_t launch_walk(const TreeView& T, const long long* sink_idx, int n_sink
                         cudaStream_t s) {
   if (n_sink <= 0) return cudaSuccess;
   (void)block_size;
-  if (wp.sub_bucket) {
-    if (counters || stats)
-      walk_warp_kernel<false, true, false, false, false, 1, true><<<(n_sink + 127) / 128, 128, 0, s>>>(
-          T, sink_idx, n_sink, wp, SinkOut{flux_out, counters, nullptr, nullptr, n_sink}, stats,
-          status, AdjointArgs{});
-    else
-      walk_warp_kernel<false, true, false, false, false, 1, true, false><<<(n_sink + 127) / 128, 128, 0, s>>>(
-          T, sink_idx, n_sink, wp, SinkOut{flux_out, nullptr, nullptr, nullptr, n_sink}, nullptr,
-          status, AdjointArgs{});
-    note_launch();
-    return cudaGetLastError();
-  }
-  if (wp.bg_radius > 0.0f || wp.tau_stop < INFINITY) {
+  if (wp.tau_stop < INFINITY && (counters || stats)) {
+    // the counters of a cut ray depend on the order of its segments: those of this walk
     const dim3 grid((n_sink + 127) / 128);
     const SinkOut o{flux_out, counters, nullptr, nullptr, n_sink};
-    const bool bg = wp.bg_radius > 0.0f, stop = wp.tau_stop < INFINITY;
-    if (counters || stats) {
-      if (bg && stop)
-        walk_warp_kernel<false, true, false, true, true><<<grid, 128, 0, s>>>(
-            T, sink_idx, n_sink, wp, o, stats, status, AdjointArgs{});
-      else if (bg)
-        walk_warp_kernel<false, true, false, true><<<grid, 128, 0, s>>>(
-            T, sink_idx, n_sink, wp, o, stats, status, AdjointArgs{});
-      else
-        walk_warp_kernel<false, true, false, false, true><<<grid, 128, 0, s>>>(
-            T, sink_idx, n_sink, wp, o, stats, status, AdjointArgs{});
-    } else {  // no counters asked for: the walk keeps none
-      if (bg && stop)
-        walk_warp_kernel<false, true, false, true, true, 1, false, false><<<grid, 128, 0, s>>>(
-            T, sink_idx, n_sink, wp, o, nullptr, status, AdjointArgs{});
-      else if (bg)
-        walk_warp_kernel<false, true, false, true, false, 1, false, false><<<grid, 128, 0, s>>>(
-            T, sink_idx, n_sink, wp, o, nullptr, status, AdjointArgs{});
-      else
-        walk_warp_kernel<false, true, false, false, true, 1, false, false><<<grid, 128, 0, s>>>(
-            T, sink_idx, n_sink, wp, o, nullptr, status, AdjointArgs{});
-    }
-    note_launch();
-    return cudaGetLastError();
-  }
-  if (wp.topdown) {  // the top-down ray walk (merged-ray walk only)
-    const SinkOut o{flux_out, counters, nullptr, nullptr, n_sink};
-    if (counters || stats)
-      walk_warp_kernel<false, true, false, false, false, 1, false, true, true>
-          <<<(n_sink + 127) / 128, 128, 0, s>>>(T, sink_idx, n_sink, wp, o, stats, status,
-                                                AdjointArgs{});
+    if (wp.bg_radius > 0.0f)
+      walk_warp_kernel<false, true, true, true, true>
+          <<<grid, 128, 0, s>>>(T, sink_idx, n_sink, wp, o, stats, status, AdjointArgs{});
     else
-      walk_warp_kernel<false, true, false, false, false, 1, false, false, true>
-          <<<(n_sink + 127) / 128, 128, 0, s>>>(T, sink_idx, n_sink, wp, o, nullptr, status,
-                                                AdjointArgs{});
+      walk_warp_kernel<false, true, false, true, true>
+          <<<grid, 128, 0, s>>>(T, sink_idx, n_sink, wp, o, stats, status, AdjointArgs{});
     note_launch();
     return cudaGetLastError();
   }
-  if (wp.variant >= 2) {
-    if (wp.variant == 3 && (counters || stats))
-      walk_warp_kernel<false, true><<<(n_sink + 127) / 128, 128, 0, s>>>(
-          T, sink_idx, n_sink, wp, SinkOut{flux_out, counters, nullptr, nullptr, n_sink}, stats, status, AdjointArgs{});
-    else if (wp.variant == 3)  // no counters asked for: the walk keeps none
-      walk_warp_kernel<false, true, false, false, false, 1, false, false><<<(n_sink + 127) / 128, 128, 0, s>>>(
-          T, sink_idx, n_sink, wp, SinkOut{flux_out, nullptr, nullptr, nullptr, n_sink}, nullptr, status, AdjointArgs{});
-    else
-      walk_warp_kernel<false, false><<<(n_sink + 127) / 128, 128, 0, s>>>(
-          T, sink_idx, n_sink, wp, SinkOut{flux_out, counters, nullptr, nullptr, n_sink}, stats, status, AdjointArgs{});
-    note_launch();
-    return cudaGetLastError();
-  }
+  if (wp.variant >= 2)
+    return launch_cut_walk(T, sink_idx, n_sink, wp, flux_out, counters, stats, status, s);
   const int chunk = chunk_of(wp);
   const long long warps = ((long long)n_sink + chunk - 1) / chunk;
   const int blocks = (int)((warps * 32 + 127) / 128);
@@ -1556,10 +1086,10 @@ cudaError_t launch_walk_adjoint(const TreeView& T, const long long* sink_idx, in
   if (n_sink <= 0) return cudaSuccess;
   if (wp.variant >= 2) {
     if (wp.variant == 3)
-      walk_warp_kernel<true, true, false, false, false, 1, false, false><<<(n_sink + 127) / 128, 128, 0, s>>>(
+      walk_warp_kernel<true, true, false, false, false><<<(n_sink + 127) / 128, 128, 0, s>>>(
           T, sink_idx, n_sink, wp, SinkOut{nullptr, nullptr, nullptr, nullptr, n_sink}, nullptr, status, J);
     else
-      walk_warp_kernel<true, false><<<(n_sink + 127) / 128, 128, 0, s>>>(
+      walk_warp_kernel<true, false, false, false, true><<<(n_sink + 127) / 128, 128, 0, s>>>(
           T, sink_idx, n_sink, wp, SinkOut{nullptr, nullptr, nullptr, nullptr, n_sink}, nullptr, status, J);
     note_launch();
     return cudaGetLastError();

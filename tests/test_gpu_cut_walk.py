@@ -1,0 +1,73 @@
+"""The walk that cuts a ray's pieces from the common ancestor's clip, where the cuts can go
+wrong: sinks and sources on the cells' planes and one ulp to either side of them, in domains
+whose planes g * h are rounded (sides that are no power of two), rays that lie in a plane,
+several sinks at one point, and one-leaf trees. The per-lane walk (variant 1) clips every
+cell on its own: both must take the same decisions, and the oracle's.
+
+The fluxes are held to the per-lane walk's. The oracle's are no measure here: where a ray
+lies within an ulp of a plane, its FP64 lengths belong to a neighbouring cell's, and the
+per-lane walk differs from it as well (by up to 27 %). The two walks add the same fp32
+lengths in another order, both compensated, so an optical depth differs by a few ulp of
+itself: tau 4 2^-24 < 2e-5 of a flux that fp32 holds (tau < 88)."""
+import numpy as np
+import pytest
+
+import workloads
+from _parity import gpu_tree, oracle_tree
+
+pytestmark = pytest.mark.gpu
+
+
+def _plane_points(rng, n, side, level):
+    """Points on the planes of the level's grid in fp32, a third each one ulp below, on and
+    one ulp above, inside [0, side)."""
+    g = rng.integers(0, 1 << level, (3, n))
+    x = (g * (np.float64(np.float32(side)) / (1 << level))).astype(np.float32)
+    step = rng.integers(-1, 2, (3, n))
+    x = np.where(step < 0, np.nextafter(x, np.float32(-1)), x)
+    x = np.where(step > 0, np.nextafter(x, np.float32(2 * side)), x)
+    top = np.nextafter(np.float32(side), np.float32(0))
+    return np.clip(x, np.float32(0), top).astype(np.float32)
+
+
+def _problem(side, level, n=3001, s=61, seed=5):
+    rng = np.random.default_rng(seed)
+    P = workloads.uniform_box(n_gas=n, n_src=s, seed=seed)
+    P["gas_xyz"] = _plane_points(rng, n, side, level)
+    P["src_xyz"] = _plane_points(rng, s, side, level)
+    P["alpha"] = rng.lognormal(0.0, 1.5, n).astype(np.float32) / np.float32(side)
+    P["side"] = float(np.float32(side))
+    return P
+
+
+@pytest.mark.parametrize("theta,tau_ref", [(0.75, 0.1), (0.0, 0.05), (0.9, 0.0)])
+@pytest.mark.parametrize("side,level", [(1.0, 4), (0.7, 4), (0.7, 9), (0.3, 6), (3.0, 5)])
+def test_points_on_the_planes(side, level, theta, tau_ref):
+    from paper_1902_08083_gb300 import trevr
+    P = _problem(side, level)
+    G = gpu_tree(P)
+    n = P["alpha"].shape[0]
+    _, rc, _ = oracle_tree(P).flux(theta, tau_ref, with_counters=True)
+    f1, c1 = trevr.compute_flux(G, theta, tau_ref, counters=True, walk_variant=1)
+    for variant in (2, 3):
+        f, c, st = trevr.compute_flux(G, theta, tau_ref, counters=True, stats=True,
+                                      walk_variant=variant)
+        plain = trevr.compute_flux(G, theta, tau_ref, walk_variant=variant)
+        assert np.array_equal(f.cpu().numpy(), plain.cpu().numpy())
+        np.testing.assert_allclose(f.cpu().numpy(), f1.cpu().numpy(), rtol=2e-5, atol=1e-30)
+        for other in (c1.cpu().numpy(), rc):
+            mism = np.count_nonzero(np.any(c.cpu().numpy() != other, axis=1))
+            assert mism <= max(1, n // 1000), f"{mism} sinks with other decisions"
+
+
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 31, 33, 129])
+def test_few_and_equal_points(n):
+    from paper_1902_08083_gb300 import trevr
+    P = _problem(0.7, 3, n=n, s=3, seed=n)
+    P["gas_xyz"][:, : (n + 1) // 2] = P["gas_xyz"][:, :1]  # equal keys share a leaf
+    G = gpu_tree(P)
+    _, rc, _ = oracle_tree(P).flux(0.5, 0.01, with_counters=True)
+    f1 = trevr.compute_flux(G, 0.5, 0.01, walk_variant=1)
+    f, c = trevr.compute_flux(G, 0.5, 0.01, counters=True)
+    np.testing.assert_allclose(f.cpu().numpy(), f1.cpu().numpy(), rtol=2e-5, atol=1e-30)
+    np.testing.assert_array_equal(c.cpu().numpy(), rc.astype(np.int32))
