@@ -225,6 +225,9 @@ cudaError_t launch_walk_bands(const TreeView& T, const long long* sink_idx, int 
 cudaError_t launch_cut_walk(const TreeView& T, const long long* sink_idx, int n_sink,
                             const WalkParams& wp, float* flux_out, int* counters,
                             unsigned long long* stats, int* status, cudaStream_t s);
+cudaError_t launch_cut_adjoint(const TreeView& T, const long long* sink_idx, int n_sink,
+                               const WalkParams& wp, const AdjointArgs& J, int* status,
+                               cudaStream_t s);
 cudaError_t launch_cut_batched(const TreeView* views, float* const* flux_out, const int2* items,
                                int n_items, int item, unsigned* counter, const WalkParams& wp,
                                unsigned long long* stats, int* status, int block_size, int n_sm,

@@ -22,19 +22,17 @@
 //   * Variant 1 (walk_kernel): one lane per sink, a flat loop in which one iteration is a
 //     walk step or a cell clip, cells picked with selects from one per-lane list; a lane
 //     that finishes takes the next sink of its warp's chunk.
-//   * walk_warp_kernel: the adjoint of variants 2 and 3, and the flux with early ray
-//     termination when counters are asked for (the segments of a ray that is cut off are
-//     counted in this walk's order). The 32 lanes walk one shared stack with a mask of the
-//     lanes that still need each cell; with MERGE a lane keeps its next ray pending, and the
-//     pending rays of all lanes (to different cells) are traced together.
-// The flux of variants 2 and 3 is in cutwalk.cu.
+//   * walk_warp_kernel: the flux with early ray termination when counters are asked for
+//     (the segments of a ray that is cut off are counted in this walk's order). The 32 lanes
+//     walk one shared stack with a mask of the lanes that still need each cell; a lane keeps
+//     its next ray pending, and the pending rays of all lanes (to different cells) are traced
+//     together.
+// Everything else of variants 2 and 3 is in cutwalk.cu.
 //   * The segment cells of a ray are known without following parent links: the sibling of a
 //     cell is its index XOR 1 (children are allocated in pairs) and the common ancestor's
 //     depth is the length of the common prefix of the sink's ancestor list and the walk
 //     path, kept as a 64-bit mask. Refined children are clipped after the ray's base
 //     segments.
-// Template options of the warp walk: ADJ (adjoint accumulation, Sec. 2.2 with the decisions
-// frozen), BG (background sources moved onto a sphere), STOP (early ray termination).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -51,7 +49,6 @@ constexpr int kRef = 2 * kDepth;
 // refinement stack of the warp walk: refined base segments (at most 2 x 63 + 1) are
 // queued first, then each popped pair adds at most one entry per level below
 constexpr int kRayStack = 4 * kDepth;
-constexpr int kSegBuf = 64;  // segments of one ray kept for the adjoint's second pass
 
 // one slab of the clip: (lo - p) * (1/d), (hi - p) * (1/d), rounded after each step;
 // along an axis the ray does not move on, the box is half-open [lo, hi), so a ray
@@ -75,15 +72,6 @@ __device__ __forceinline__ void slab_nz(float lo, float hi, float p, float inv, 
   const float tb = __fmul_rn(__fsub_rn(hi, p), inv);
   t0 = fmaxf(t0, fminf(ta, tb));
   t1 = fminf(t1, fmaxf(ta, tb));
-}
-
-__device__ __forceinline__ void slab_g_nz(int k, float lo, float hi, float p, float inv,
-                                          float& t0, float& t1, int& k0, int& k1) {
-  const float ta = __fmul_rn(__fsub_rn(lo, p), inv);
-  const float tb = __fmul_rn(__fsub_rn(hi, p), inv);
-  const float tn = fminf(ta, tb), tx = fmaxf(ta, tb);
-  if (tn > t0) { t0 = tn; k0 = k; }
-  if (tx < t1) { t1 = tx; k1 = k; }
 }
 
 // gradient-carrying slab: remembers which axis sets t0 / t1
@@ -505,37 +493,18 @@ struct WarpStack {
   int path[kDepth];  // the walk's depth-first path
 };
 
-// Sum of v over the lanes that asked (key >= 0) when they all name the same cell,
-// else one atomic per lane. Every lane of the warp must call it.
-__device__ __forceinline__ void warp_atomic_add(double* base, int key, float v) {
-  const unsigned FULL = 0xffffffffu;
-  const unsigned want = __ballot_sync(FULL, key >= 0);
-  if (!want) return;
-  const int k0 = __shfl_sync(FULL, key, __ffs(want) - 1);
-  if (__all_sync(FULL, key < 0 || key == k0)) {
-    float x = key >= 0 ? v : 0.0f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(&base[k0], (double)x);
-  } else if (key >= 0) {
-    atomicAdd(&base[key], (double)v);
-  }
-}
-
 // Rays from the sinks of the lanes in `on` to (q, L) inside cell C; every lane
 // of the warp must call it (the loop runs while any lane has cells left).
-// STOP: early ray termination (Sec. 4): a lane whose running optical depth passes
-// P.tau_stop drops the rest of its ray, and the ray adds nothing.
-template <bool ADJ, bool STOP, bool CNT>
+// Early ray termination (Sec. 4): a lane whose running optical depth passes P.tau_stop
+// drops the rest of its ray, and the ray adds nothing.
 __device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P, const bool on,
                                          const float px, const float py, const float pz,
                                          const int S, const int dS, const int* anc, int* rst,
                                          const unsigned long long on_path, const int* path,
                                          const int C, const int dC, const float qx,
                                          const float qy, const float qz, const float L,
-                                         const int src_j, const float gk, const int stack_limit,
-                                         const int box_limit, int* status, const AdjointArgs& J,
-                                         SinkCounters& cnt, CSum* F) {
+                                         const int box_limit, int* status, SinkCounters& cnt,
+                                         CSum& F) {
   const unsigned FULL = 0xffffffffu;
   float dx = 0.0f, dy = 0.0f, dz = 0.0f, s2 = 1.0f, len = 1.0f, ix = 0.0f, iy = 0.0f, iz = 0.0f;
   int nCs = 0, nSs = 0, nb = 0, dstar = 0;
@@ -563,62 +532,19 @@ __device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P,
       }
     }
   }
-  const bool traced = active;
   const bool nz = dx != 0.0f && dy != 0.0f && dz != 0.0f;  // the ray moves along every axis
   KSum tau;
   bool cut = false;
-  int b = 0, rsp = 0, boxes = 0, pass = 1;
+  int b = 0, rsp = 0, boxes = 0;
   int slot = -1;  // the upper child of the pair popped last: clipped next
-  // adjoint: the first pass records its segment cells and lengths (up to kSegBuf),
-  // so the second pass replays them instead of tracing the ray again
-  int segb[ADJ ? kSegBuf : 1];
-  float segl[ADJ ? kSegBuf : 1];
-  int nseg = 0, kk = 0;
-  bool seg_over = false;
-  float gq0 = 0.0f, gq1 = 0.0f, gq2 = 0.0f, fcur = 0.0f;
   while (__any_sync(FULL, active)) {
-    int akey = -1;
-    float aval = 0.0f;
-    if (ADJ && active && pass == 3) {
-      if (kk < nseg) {
-        // four recorded segments per iteration: 2.2 % faster backward than one
-        // (145.5 against 148.8 ms at 2^21), eight were slower (154 ms)
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (kk + u < nseg) atomicAdd(&J.G[segb[kk + u]], (double)(-gk * fcur * segl[kk + u]));
-        kk += 4;
-      } else {
-        if (CNT) ++cnt.rays;
-        active = false;
-      }
-    } else if (active) {
+    if (active) {
       const bool from_stack = b >= nb && (rsp > 0 || slot >= 0);  // base segments first
       if (!from_stack && b >= nb) {
-        const float f = L * expf(-tau.get()) / (kFourPi * s2);
-        if (!ADJ && STOP && cut) {
-          if (CNT) ++cnt.cut;
-          if (CNT) ++cnt.rays;
-          active = false;
-        } else if (!ADJ) {
-          F[0].add(f);
-          if (CNT) ++cnt.rays;
-          active = false;
-        } else if (pass == 1) {
-          fcur = f;  // second pass over the same cells, now that f is known
-          if (!seg_over) {
-            pass = 3;  // replay the recorded segments
-            kk = 0;
-          } else {
-            pass = 2;  // too many segments to record: trace the ray again
-            b = 0;
-            rsp = 0;
-            slot = -1;
-            boxes = 0;
-          }
-        } else {
-          if (CNT) ++cnt.rays;
-          active = false;
-        }
+        if (cut) ++cnt.cut;
+        else F.add(L * expf(-tau.get()) / (kFourPi * s2));
+        ++cnt.rays;
+        active = false;
       } else {
         int box;
         if (from_stack) {
@@ -653,19 +579,9 @@ __device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P,
         {
           const float4 a = __ldg(&T.nA[box]);
           const float4 bb = __ldg(&T.nB[box]);
-          const bool want_grad = ADJ && pass == 1 && src_j < 0;
           float t0 = 0.0f, t1 = 1.0f;
           bool miss = false;
-          int k0 = -1, k1 = -1;
-          if (want_grad && nz) {
-            slab_g_nz(0, a.x, bb.x, px, ix, t0, t1, k0, k1);
-            slab_g_nz(1, a.y, bb.y, py, iy, t0, t1, k0, k1);
-            slab_g_nz(2, a.z, bb.z, pz, iz, t0, t1, k0, k1);
-          } else if (want_grad) {
-            slab_g(0, a.x, bb.x, px, dx, ix, t0, t1, k0, k1, miss);
-            slab_g(1, a.y, bb.y, py, dy, iy, t0, t1, k0, k1, miss);
-            slab_g(2, a.z, bb.z, pz, dz, iz, t0, t1, k0, k1, miss);
-          } else if (nz) {  // no axis along which the ray stays still: no face tests
+          if (nz) {  // no axis along which the ray stays still: no face tests
             slab_nz(a.x, bb.x, px, ix, t0, t1);
             slab_nz(a.y, bb.y, py, iy, t0, t1);
             slab_nz(a.z, bb.z, pz, iz, t0, t1);
@@ -675,7 +591,7 @@ __device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P,
             slab(a.z, bb.z, pz, dz, iz, t0, t1, miss);
           }
           const float l = (!miss && t1 > t0) ? __fmul_rn(__fsub_rn(t1, t0), len) : 0.0f;
-          if (CNT) ++cnt.clip;
+          ++cnt.clip;
           if (l > 0.0f) {
             bool pushed = false;
             if (P.tau_ref <= 0.0f || __fmul_rn(bb.w, l) > P.tau_ref) {
@@ -688,7 +604,7 @@ __device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P,
                   atomicOr(status, kStatusIterationLimit);
                   active = false;
                 } else {
-                  if (CNT) ++cnt.ref;
+                  ++cnt.ref;
                   // The children's intervals are this cell's cut at the split plane,
                   // whose t is the one their clips would compute ((P - p) * (1/d),
                   // with min / max exact), so a child the ray misses is not queued
@@ -717,59 +633,19 @@ __device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P,
               }
             }
             if (!pushed) {
-              if (ADJ && pass == 2) {
-                akey = box;
-                aval = -gk * fcur * l;
-              } else {
-                tau.add(__fmul_rn(a.w, l));
-                if (!ADJ && STOP && tau.get() > P.tau_stop) {
-                  cut = true;  // the rest of the ray is not traced
-                  b = nb;
-                  rsp = 0;
-                  slot = -1;
-                }
-                if (ADJ) {
-                  if (nseg < kSegBuf) {
-                    segb[nseg] = box;
-                    segl[nseg] = l;
-                    ++nseg;
-                  } else {
-                    seg_over = true;
-                  }
-                }
-                if (want_grad) {
-                  const float w = (t1 - t0) / len;
-                  const float g0 = (k1 == 0 ? -t1 * ix : 0.0f) + (k0 == 0 ? t0 * ix : 0.0f);
-                  const float g1 = (k1 == 1 ? -t1 * iy : 0.0f) + (k0 == 1 ? t0 * iy : 0.0f);
-                  const float g2 = (k1 == 2 ? -t1 * iz : 0.0f) + (k0 == 2 ? t0 * iz : 0.0f);
-                  gq0 = fmaf(a.w, g0 * len + w * dx, gq0);
-                  gq1 = fmaf(a.w, g1 * len + w * dy, gq1);
-                  gq2 = fmaf(a.w, g2 * len + w * dz, gq2);
-                }
-                if (CNT) ++cnt.segs;
+              tau.add(__fmul_rn(a.w, l));
+              if (tau.get() > P.tau_stop) {
+                cut = true;  // the rest of the ray is not traced
+                b = nb;
+                rsp = 0;
+                slot = -1;
               }
+              ++cnt.segs;
             }
           }
         }
       }
     }
-    // a retraced segment's gradient (a ray with more segments than were recorded): the
-    // lanes trace different rays, so the cells differ and each lane adds its own, as the
-    // replay does (1.4 % faster than trying a warp-wide sum first)
-    if (ADJ && akey >= 0) atomicAdd(&J.G[akey], (double)aval);
-  }
-  if (ADJ) {
-    // the pseudo-source's terms. The lanes of one call may mix single sources and
-    // merged cells (merged pending rays), so every lane takes part in every
-    // warp-wide sum, naming no key (-1) for a term that is not its own.
-    const bool single = traced && src_j >= 0, merged = traced && src_j < 0;
-    const float gf = traced ? gk * fcur : 0.0f;
-    const float c = traced ? gf / L : 0.0f, inv_s2 = 2.0f / s2;
-    warp_atomic_add(J.e, single ? src_j : -1, c);
-    warp_atomic_add(J.a, merged ? C : -1, c);
-    warp_atomic_add(J.b + 0, merged ? 3 * C : -1, c * (-dx * inv_s2 - gq0));
-    warp_atomic_add(J.b + 1, merged ? 3 * C : -1, c * (-dy * inv_s2 - gq1));
-    warp_atomic_add(J.b + 2, merged ? 3 * C : -1, c * (-dz * inv_s2 - gq2));
   }
 }
 
@@ -818,21 +694,19 @@ __device__ __forceinline__ void bg_move(const TreeView& T, const WalkParams& P, 
 
 // The hot path for the 32 sinks of one warp (lane holds sorted position i if
 // `has`); every lane of the warp must call it. Accumulates the lane's flux in F.
-// MERGE = true: a lane that accepts a cell (or reaches a single source) does not
-// trace the ray at once; it keeps it pending, and the pending rays of all lanes are
-// traced together (each lane to its own cell) when a lane needs its slot again or
-// when the walk is about to overwrite the part of the path a pending ray uses. More
-// lanes then share each traced batch; every lane still gets the same rays.
-// BG = true (with MERGE): background sources (Sec. 2.2.4). A merged cell's centre of
+// A lane that accepts a cell (or reaches a single source) does not trace the ray at once;
+// it keeps it pending, and the pending rays of all lanes are traced together (each lane to
+// its own cell) when a lane needs its slot again or when the walk is about to overwrite the
+// part of the path a pending ray uses.
+// BG: background sources (Sec. 2.2.4). A merged cell's centre of
 // luminosity c is moved radially onto the sphere of radius R around the domain centre
 // o before its ray is traced, in fp32 as d = c - o, s = sqrt((dx^2 + dy^2) + dz^2),
 // q = o + d * (R / s); the ray then ends in the leaf that holds q, whose ancestors the
 // lane finds by descending the cut planes from the root and keeps for that ray.
-template <bool ADJ, bool MERGE, bool BG, bool STOP, bool CNT>
+template <bool BG>
 __device__ __forceinline__ void warp_walk(const TreeView& T, const WalkParams& P, const bool has,
-                                          const int i, const float gk, WarpStack& ws,
-                                          int* status, const AdjointArgs& J,
-                                          SinkCounters& cnt, CSum* F) {
+                                          const int i, WarpStack& ws, int* status,
+                                          SinkCounters& cnt, CSum& F) {
   const unsigned FULL = 0xffffffffu;
   const unsigned lane = threadIdx.x & 31u;
   const int stack_limit = P.stack_depth < kDepth ? P.stack_depth : kDepth;
@@ -862,11 +736,11 @@ __device__ __forceinline__ void warp_walk(const TreeView& T, const WalkParams& P
     ws.mask[0] = live;
   }
   int sp = live ? 1 : 0;
-  // this lane's pending ray (MERGE)
+  // this lane's pending ray
   bool pnd = false;
   bool pbg = false;          // (BG) the pending ray ends at a moved source: path in cpath
   int cpath[BG ? kDepth : 1] = {};  // (BG) ancestors of the leaf holding the moved source
-  int pC = 0, pdC = 0, psrc = -1;
+  int pC = 0, pdC = 0;
   float pqx = 0.0f, pqy = 0.0f, pqz = 0.0f, pL = 0.0f;
   auto flush = [&]() {
     if (BG) {
@@ -880,11 +754,11 @@ __device__ __forceinline__ void warp_walk(const TreeView& T, const WalkParams& P
         for (int d = 0; d <= mn && cpath[d] == anc[d]; ++d) onp |= 1ull << d;
         pp = cpath;
       }
-      warp_ray<ADJ, STOP, CNT>(T, P, pnd, px, py, pz, S, dS, anc, rst, onp, pp, pC, pdC, pqx, pqy,
-                         pqz, pL, psrc, gk, stack_limit, box_limit, status, J, cnt, F);
+      warp_ray(T, P, pnd, px, py, pz, S, dS, anc, rst, onp, pp, pC, pdC, pqx, pqy, pqz, pL,
+               box_limit, status, cnt, F);
     } else {
-      warp_ray<ADJ, STOP, CNT>(T, P, pnd, px, py, pz, S, dS, anc, rst, on_path, ws.path, pC, pdC,
-                         pqx, pqy, pqz, pL, psrc, gk, stack_limit, box_limit, status, J, cnt, F);
+      warp_ray(T, P, pnd, px, py, pz, S, dS, anc, rst, on_path, ws.path, pC, pdC, pqx, pqy, pqz,
+               pL, box_limit, status, cnt, F);
     }
     pnd = false;
     pbg = false;
@@ -896,7 +770,7 @@ __device__ __forceinline__ void warp_walk(const TreeView& T, const WalkParams& P
     const unsigned M = ws.mask[sp];
     __syncwarp();
     // a pending ray reads the path up to its cell's depth: trace it before that changes
-    if (MERGE && __any_sync(FULL, pnd && !pbg && pdC >= dX)) flush();
+    if (__any_sync(FULL, pnd && !pbg && pdC >= dX)) flush();
     if (lane == 0) ws.path[dX] = X;
     const unsigned long long bit = 1ull << dX;
     if (has) on_path = (dX <= dS && anc[dX] == X) ? (on_path | bit) : (on_path & ~bit);
@@ -905,7 +779,7 @@ __device__ __forceinline__ void warp_walk(const TreeView& T, const WalkParams& P
     if (!(s.w > 0.0f)) continue;
     bool acc = false, opn = false;
     if ((M >> lane) & 1u) {
-      if (CNT) ++cnt.visit;
+      ++cnt.visit;
       const float4 a = __ldg(&T.nA[X]);
       const float4 bb = __ldg(&T.nB[X]);
       const float ex = fmaxf(fmaxf(__fsub_rn(a.x, px), __fsub_rn(px, bb.x)), 0.0f);
@@ -916,27 +790,20 @@ __device__ __forceinline__ void warp_walk(const TreeView& T, const WalkParams& P
       acc = __ldg(&T.nl2[X]) < __fmul_rn(P.theta2, r2);
       opn = !acc;
     }
-    const unsigned accM = __ballot_sync(FULL, acc);
     const unsigned opnM = __ballot_sync(FULL, opn);
-    if (MERGE) {
-      if (__any_sync(FULL, acc && pnd)) flush();
-      if (acc) {
-        pnd = true;
-        pC = X;
-        pdC = dX;
-        pqx = s.x;
-        pqy = s.y;
-        pqz = s.z;
-        pL = s.w;
-        psrc = -1;
-        if (BG) {
-          bg_move(T, P, s, pqx, pqy, pqz, pC, pdC, cpath);
-          pbg = true;
-        }
+    if (__any_sync(FULL, acc && pnd)) flush();
+    if (acc) {
+      pnd = true;
+      pC = X;
+      pdC = dX;
+      pqx = s.x;
+      pqy = s.y;
+      pqz = s.z;
+      pL = s.w;
+      if (BG) {
+        bg_move(T, P, s, pqx, pqy, pqz, pC, pdC, cpath);
+        pbg = true;
       }
-    } else if (accM) {
-      warp_ray<ADJ, STOP, CNT>(T, P, acc, px, py, pz, S, dS, anc, rst, on_path, ws.path, X, dX, s.x,
-                         s.y, s.z, s.w, -1, gk, stack_limit, box_limit, status, J, cnt, F);
     }
     if (opnM) {
       const int4 t = __ldg(&T.nT[X]);
@@ -944,21 +811,15 @@ __device__ __forceinline__ void warp_walk(const TreeView& T, const WalkParams& P
         for (int jj = t.z; jj < t.z + t.w; ++jj) {
           const float4 y = __ldg(&T.src[jj]);
           if (!(y.w > 0.0f)) continue;
-          if (MERGE) {
-            if (__any_sync(FULL, opn && pnd)) flush();
-            if (opn) {
-              pnd = true;
-              pC = X;
-              pdC = dX;
-              pqx = y.x;
-              pqy = y.y;
-              pqz = y.z;
-              pL = y.w;
-              psrc = jj;
-            }
-          } else {
-            warp_ray<ADJ, STOP, CNT>(T, P, opn, px, py, pz, S, dS, anc, rst, on_path, ws.path, X, dX,
-                               y.x, y.y, y.z, y.w, jj, gk, stack_limit, box_limit, status, J, cnt, F);
+          if (__any_sync(FULL, opn && pnd)) flush();
+          if (opn) {
+            pnd = true;
+            pC = X;
+            pdC = dX;
+            pqx = y.x;
+            pqy = y.y;
+            pqz = y.z;
+            pL = y.w;
           }
         }
       } else {
@@ -979,17 +840,14 @@ __device__ __forceinline__ void warp_walk(const TreeView& T, const WalkParams& P
       }
     }
   }
-  if (MERGE && __any_sync(FULL, pnd)) flush();
+  if (__any_sync(FULL, pnd)) flush();
 }
 
-// 8 blocks of 128 per SM (at most 64 registers): measured 8% faster for the adjoint than
-// the compiler's own 70 registers at 7 blocks; 10 and 12 blocks spilled and were 6% and 13%
-// slower. The adjoint keeps no counters (the backward call reports none).
-template <bool ADJ, bool MERGE, bool BG, bool STOP, bool CNT>
+template <bool BG>
 __global__ void __launch_bounds__(128, 8) walk_warp_kernel(TreeView T, const long long* sink_idx,
                                                            int n_sink, WalkParams P, SinkOut out,
-                                                           unsigned long long* stats, int* status,
-                                                           AdjointArgs J) {
+                                                           unsigned long long* stats,
+                                                           int* status) {
   __shared__ WarpStack stacks[4];
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   WarpStack& ws = stacks[threadIdx.x >> 5];
@@ -998,17 +856,16 @@ __global__ void __launch_bounds__(128, 8) walk_warp_kernel(TreeView T, const lon
   float g = 0.0f;
   bool has = false;
   if (k < n_sink) {
-    PlainMap<ADJ> map{&T, sink_idx, J.grad_flux, status};
+    PlainMap<false> map{&T, sink_idx, nullptr, status};
     has = map(k, i, slot, g);
-    if (!has && !ADJ && sink_idx) {
+    if (!has && sink_idx) {
       if (out.flux) out.flux[k] = 0.0f;
       if (out.counters) reinterpret_cast<int4*>(out.counters)[k] = make_int4(0, 0, 0, 0);
     }
   }
   CSum F;
-  if (__any_sync(0xffffffffu, has))
-    warp_walk<ADJ, MERGE, BG, STOP, CNT>(T, P, has, i, g, ws, status, J, cnt, &F);
-  if (!ADJ && has) {
+  if (__any_sync(0xffffffffu, has)) warp_walk<BG>(T, P, has, i, ws, status, cnt, F);
+  if (has) {
     if (out.flux) out.flux[slot] = F.get();
     if (out.counters)
       reinterpret_cast<int4*>(out.counters)[slot] =
@@ -1060,11 +917,9 @@ cudaError_t launch_walk(const TreeView& T, const long long* sink_idx, int n_sink
     const dim3 grid((n_sink + 127) / 128);
     const SinkOut o{flux_out, counters, nullptr, nullptr, n_sink};
     if (wp.bg_radius > 0.0f)
-      walk_warp_kernel<false, true, true, true, true>
-          <<<grid, 128, 0, s>>>(T, sink_idx, n_sink, wp, o, stats, status, AdjointArgs{});
+      walk_warp_kernel<true><<<grid, 128, 0, s>>>(T, sink_idx, n_sink, wp, o, stats, status);
     else
-      walk_warp_kernel<false, true, false, true, true>
-          <<<grid, 128, 0, s>>>(T, sink_idx, n_sink, wp, o, stats, status, AdjointArgs{});
+      walk_warp_kernel<false><<<grid, 128, 0, s>>>(T, sink_idx, n_sink, wp, o, stats, status);
     note_launch();
     return cudaGetLastError();
   }
@@ -1084,16 +939,7 @@ cudaError_t launch_walk_adjoint(const TreeView& T, const long long* sink_idx, in
                                 const WalkParams& wp, const AdjointArgs& J, int* status,
                                 cudaStream_t s) {
   if (n_sink <= 0) return cudaSuccess;
-  if (wp.variant >= 2) {
-    if (wp.variant == 3)
-      walk_warp_kernel<true, true, false, false, false><<<(n_sink + 127) / 128, 128, 0, s>>>(
-          T, sink_idx, n_sink, wp, SinkOut{nullptr, nullptr, nullptr, nullptr, n_sink}, nullptr, status, J);
-    else
-      walk_warp_kernel<true, false, false, false, true><<<(n_sink + 127) / 128, 128, 0, s>>>(
-          T, sink_idx, n_sink, wp, SinkOut{nullptr, nullptr, nullptr, nullptr, n_sink}, nullptr, status, J);
-    note_launch();
-    return cudaGetLastError();
-  }
+  if (wp.variant >= 2) return launch_cut_adjoint(T, sink_idx, n_sink, wp, J, status, s);
   const int chunk = chunk_of(wp);
   const long long warps = ((long long)n_sink + chunk - 1) / chunk;
   const int blocks = (int)((warps * 32 + 127) / 128);
