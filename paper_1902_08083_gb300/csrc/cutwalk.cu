@@ -5,6 +5,12 @@
 // that accepts a cell, or reaches a source of an opened leaf, keeps that ray waiting; when a
 // lane with a waiting ray gets another, the waiting rays of all lanes are traced together.
 //
+// Where a call has too few sinks to fill the GPU with a warp per 32, a block of several warps
+// takes the same 32 sinks: each walks the source tree, and the takings (a cell accepted by some
+// lanes, a source reached) go to the warps in turn. A sink's flux is summed in kSlots
+// compensated parts, the takings in turn to each, whether or not the warps share a group, so
+// that the result does not depend on it.
+//
 // A ray is a list of pieces along [0, 1] (p + t d). All of them are cut from the clip of
 // the common ancestor A of the sink's leaf S and the source's cell C: a cell's interval
 // at its split plane, at t = (plane - p) * (1/d), gives the intervals of its children. On
@@ -45,10 +51,40 @@ constexpr int kSpare = 20;
 static_assert(3 * kDepth + 3 + 2 * kSpare <= kPieces, "the list holds every piece of a ray");
 constexpr int kSegBuf = 64;  // segments of one ray kept for the adjoint's replay
 
+constexpr int kSlots = 8;    // parts of a sink's flux; at most as many warps per group
+
 struct CutStack {
   int node[kDepth + 2];
   unsigned mask[kDepth + 2];
 };
+
+// A warp's share of a group's takings: those with (number & (parts - 1)) == part. parts is a
+// power of two, at most kSlots.
+struct Share {
+  int part, parts;
+};
+
+// Compensated sums of one lane's takings, one per slot.
+struct Slots {
+  float2 v[kSlots];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int k = 0; k < kSlots; ++k) v[k] = make_float2(0.0f, 0.0f);
+  }
+  __device__ __forceinline__ void add(int k, float f) {
+    CSum t;
+    t.s = v[k].x;
+    t.c = v[k].y;
+    t.add(f);
+    v[k] = make_float2(t.s, t.c);
+  }
+};
+
+// s + c of a part joins the sum
+__device__ __forceinline__ void join(CSum& sum, float2 part) {
+  sum.add(part.x);
+  sum.c = __fadd_rn(sum.c, part.y);
+}
 
 // ---------------------------------------------------------------------------
 // Sub-bucket particle trace (Sec. 2.2.3, 3.1.3). The absorption below the bucket
@@ -90,7 +126,7 @@ __device__ __forceinline__ float sub_bucket_tau_warp(const TreeView& T, int src,
                                                      float t0, float t1) {
   const unsigned FULL = 0xffffffffu;
   const unsigned lane = threadIdx.x & 31u;
-  __shared__ SubQueue queues[4];  // one per warp of a 128-thread block
+  __shared__ SubQueue queues[kSlots];  // one per warp of a block
   SubQueue& Q = queues[threadIdx.x >> 5];
   box = __shfl_sync(FULL, box, src);
   si = __shfl_sync(FULL, si, src);
@@ -339,7 +375,7 @@ template <bool ADJ, bool MOM, bool BG, bool STOP, int NB, bool SUB, bool CNT, bo
 __device__ __forceinline__ void cut_ray(const TreeView& T, const WalkParams& P, const float tref,
                                         const bool on, const int ent, const Sink& K, Line& ray,
                                         Pieces<ADJ>& W, const AdjointArgs& J, SinkCounters& cnt,
-                                        CSum* F, Moments* mom) {
+                                        const int slot, Slots& flux, CSum* F, Moments* mom) {
   const unsigned FULL = 0xffffffffu;
   float L = 0.0f;
   int C = kRoot;
@@ -617,7 +653,7 @@ __device__ __forceinline__ void cut_ray(const TreeView& T, const WalkParams& P, 
     return;
   }
   f = L * expf(-tau.get()) / (kFourPi * ray.s2);
-  F[0].add(f);
+  flux.add(slot, f);
   if (MOM) {
     const float il = 1.0f / ray.len;
     const float n0 = -ray.dx * il, n1 = -ray.dy * il, n2 = -ray.dz * il;
@@ -638,9 +674,9 @@ __device__ __forceinline__ void cut_ray(const TreeView& T, const WalkParams& P, 
 // another; without it (variant 2) the rays to a cell are traced as soon as it is accepted.
 template <bool ADJ, bool MERGE, bool MOM, bool BG, bool STOP, int NB, bool SUB, bool CNT, bool TD>
 __device__ __forceinline__ void cut_walk(const TreeView& T, const WalkParams& P, const bool has,
-                                         const int i, const float grad, CutStack& ws, int* status,
-                                         const AdjointArgs& J, SinkCounters& cnt, CSum* F,
-                                         Moments* mom) {
+                                         const int i, const float grad, const Share share,
+                                         CutStack& ws, int* status, const AdjointArgs& J,
+                                         SinkCounters& cnt, Slots& flux, CSum* F, Moments* mom) {
   const unsigned FULL = 0xffffffffu;
   const unsigned lane = threadIdx.x & 31u;
   const int stack_limit = P.stack_depth < kDepth ? P.stack_depth : kDepth;
@@ -667,6 +703,8 @@ __device__ __forceinline__ void cut_walk(const TreeView& T, const WalkParams& P,
   int w_ent = 0;          // (a cell, or ~source)
   int j = 0, j_end = 0;   // sources of the opened leaf still to be taken
   unsigned opened = 0;    // the lanes that opened it
+  int taken = 0, w_slot = 0;  // takings so far; the slot of the waiting ray
+  if (!ADJ && NB == 1) flux.clear();
   __syncwarp();
   while (true) {
     bool take = false;
@@ -686,7 +724,7 @@ __device__ __forceinline__ void cut_walk(const TreeView& T, const WalkParams& P,
       const float4 s = __ldg(&T.nS[X]);
       bool open = false;
       if (s.w > 0.0f && ((M >> lane) & 1u)) {
-        if (CNT) ++cnt.visit;
+        if (CNT && share.part == 0) ++cnt.visit;
         const float4 a = __ldg(&T.nA[X]);
         const float4 bb = __ldg(&T.nB[X]);
         const float ex = fmaxf(fmaxf(__fsub_rn(a.x, ray.px), __fsub_rn(ray.px, bb.x)), 0.0f);
@@ -720,15 +758,21 @@ __device__ __forceinline__ void cut_walk(const TreeView& T, const WalkParams& P,
         }
       }
     }
+    if (!done) {
+      if (!__any_sync(FULL, take)) continue;
+      const int turn = taken++;
+      if ((turn & (share.parts - 1)) != share.part) continue;
+    }
     if (__any_sync(FULL, wait && (done || take || !MERGE))) {
-      cut_ray<ADJ, MOM, BG, STOP, NB, SUB, CNT, TD>(T, P, tref, wait, w_ent, K, ray, W, J, cnt, F,
-                                                    mom);
+      cut_ray<ADJ, MOM, BG, STOP, NB, SUB, CNT, TD>(T, P, tref, wait, w_ent, K, ray, W, J, cnt,
+                                                    w_slot, flux, F, mom);
       wait = false;
     }
     if (done) break;
     if (take) {
       wait = true;
       w_ent = ent;
+      w_slot = (taken - 1) & (kSlots - 1);
     }
   }
 }
@@ -745,12 +789,18 @@ __device__ __forceinline__ void cut_walk(const TreeView& T, const WalkParams& P,
 // 9.2 at 8).
 constexpr int cut_blocks(bool SUB, int NB) { return SUB ? 4 : NB > 1 ? 6 : 8; }
 
-template <bool MERGE, bool MOM, bool BG, bool STOP, int NB, bool SUB, bool CNT, bool TD>
-__global__ void __launch_bounds__(128, cut_blocks(SUB, NB))
+// SHARED: the block's warps (a power of two, at most kSlots) share one group of 32 sinks.
+template <bool SHARED, bool MERGE, bool MOM, bool BG, bool STOP, int NB, bool SUB, bool CNT,
+          bool TD>
+__global__ void __launch_bounds__(SHARED ? 32 * kSlots : 128,
+                                  SHARED ? cut_blocks(SUB, NB) / 2 : cut_blocks(SUB, NB))
     cut_walk_kernel(TreeView T, const long long* sink_idx, int n_sink, WalkParams P, SinkOut out,
                     unsigned long long* stats, int* status) {
-  __shared__ CutStack stacks[4];
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ CutStack stacks[SHARED ? kSlots : 4];
+  __shared__ float2 parts[SHARED ? kSlots : 1][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const Share share = SHARED ? Share{warp, (int)(blockDim.x >> 5)} : Share{0, 1};
+  const int k = SHARED ? blockIdx.x * 32 + lane : blockIdx.x * 128 + threadIdx.x;
   SinkCounters cnt;
   int i = 0, slot = 0;
   float g = 0.0f;
@@ -758,20 +808,63 @@ __global__ void __launch_bounds__(128, cut_blocks(SUB, NB))
   if (k < n_sink) {
     PlainMap<false> map{&T, sink_idx, nullptr, status};
     has = map(k, i, slot, g);
-    if (!has && sink_idx) {
+    if (!has && sink_idx && share.part == 0) {
       if (out.flux)
         for (int b = 0; b < (NB > 1 ? T.n_bands : 1); ++b)
           out.flux[(size_t)b * out.n_out + k] = 0.0f;
       if (out.counters) reinterpret_cast<int4*>(out.counters)[k] = make_int4(0, 0, 0, 0);
     }
   }
+  Slots flux;
   CSum F[NB];
   Moments mom;
   if (__any_sync(0xffffffffu, has))
     cut_walk<false, MERGE, MOM, BG, STOP, NB, SUB, CNT, TD>(
-        T, P, has, i, 0.0f, stacks[threadIdx.x >> 5], status, AdjointArgs{}, cnt, F,
+        T, P, has, i, 0.0f, share, stacks[warp], status, AdjointArgs{}, cnt, flux, F,
         MOM ? &mom : nullptr);
-  if (MOM && has) {
+  else if (NB == 1)
+    flux.clear();
+  if (CNT && stats) add_stats(cnt, stats);
+  // the group's sums, in warp 0 (every warp of the block comes here)
+  auto gather = [&](CSum& v) {
+    parts[SHARED ? warp : 0][lane] = make_float2(v.s, v.c);
+    __syncthreads();
+    if (warp == 0)
+      for (int w = 1; w < share.parts; ++w) join(v, parts[SHARED ? w : 0][lane]);
+    __syncthreads();
+  };
+  if (NB == 1) {
+    if (SHARED) {
+#pragma unroll
+      for (int q = 0; q < kSlots; ++q)
+        if ((q & (share.parts - 1)) == share.part) parts[SHARED ? q : 0][lane] = flux.v[q];
+      __syncthreads();
+    }
+#pragma unroll
+    for (int q = 0; q < kSlots; ++q) join(F[0], SHARED ? parts[SHARED ? q : 0][lane] : flux.v[q]);
+    if (SHARED) __syncthreads();
+  } else if (SHARED) {
+#pragma unroll
+    for (int b = 0; b < NB; ++b) gather(F[b]);
+  }
+  if (MOM && SHARED) {
+#pragma unroll
+    for (int q = 0; q < 9; ++q) gather(mom.v[q]);
+  }
+  if (CNT && SHARED && out.counters) {
+    __shared__ int counted[3][32];
+    if (warp == 0) counted[0][lane] = counted[1][lane] = counted[2][lane] = 0;
+    __syncthreads();
+    atomicAdd(&counted[0][lane], cnt.rays);
+    atomicAdd(&counted[1][lane], cnt.segs);
+    atomicAdd(&counted[2][lane], cnt.ref);
+    __syncthreads();
+    cnt.rays = counted[0][lane];
+    cnt.segs = counted[1][lane];
+    cnt.ref = counted[2][lane];
+  }
+  if (!has || warp >= (SHARED ? 1 : 4)) return;
+  if (MOM) {
 #pragma unroll
     for (int q = 0; q < 3; ++q)
       if (out.fvec) out.fvec[(size_t)q * out.n_out + slot] = mom.v[q].get();
@@ -779,20 +872,16 @@ __global__ void __launch_bounds__(128, cut_blocks(SUB, NB))
     for (int q = 0; q < 6; ++q)
       if (out.press) out.press[(size_t)q * out.n_out + slot] = mom.v[3 + q].get();
   }
-  if (has) {
-    if (NB > 1) {
-      // band-major output: band b of sink slot at b * n_out + slot
+  if (NB > 1) {
+    // band-major output: band b of sink slot at b * n_out + slot
 #pragma unroll
-      for (int b = 0; b < NB; ++b)
-        if (out.flux && b < T.n_bands) out.flux[(size_t)b * out.n_out + slot] = F[b].get();
-    } else if (out.flux) {
-      out.flux[slot] = F[0].get();
-    }
-    if (out.counters)
-      reinterpret_cast<int4*>(out.counters)[slot] =
-          make_int4(cnt.rays, cnt.segs, cnt.visit, cnt.ref);
+    for (int b = 0; b < NB; ++b)
+      if (out.flux && b < T.n_bands) out.flux[(size_t)b * out.n_out + slot] = F[b].get();
+  } else if (out.flux) {
+    out.flux[slot] = F[0].get();
   }
-  if (CNT && stats) add_stats(cnt, stats);
+  if (out.counters)
+    reinterpret_cast<int4*>(out.counters)[slot] = make_int4(cnt.rays, cnt.segs, cnt.visit, cnt.ref);
 }
 
 // Batched form: each work item is cut into groups of 32 consecutive sinks, one warp walk
@@ -820,9 +909,12 @@ __global__ void __launch_bounds__(BS, 1024 / BS) cut_walk_batched_kernel(
     for (int g0 = w.y; g0 < end; g0 += 32) {
       const int i = g0 + (int)lane;
       const bool has = i < end;
+      Slots flux;
       CSum F;
       cut_walk<false, MERGE, false, false, false, 1, false, CNT, false>(
-          T, Pt, has, i, 0.0f, ws, status, AdjointArgs{}, tot, &F, nullptr);
+          T, Pt, has, i, 0.0f, Share{0, 1}, ws, status, AdjointArgs{}, tot, flux, &F, nullptr);
+#pragma unroll
+      for (int q = 0; q < kSlots; ++q) join(F, flux.v[q]);
       if (has) flux_out[w.x][T.perm[i]] = F.get();
     }
   }
@@ -832,12 +924,14 @@ __global__ void __launch_bounds__(BS, 1024 / BS) cut_walk_batched_kernel(
 // The adjoint walk; a sink with dLoss/dF = 0 is left out. Flux and gradients of 2^20 sinks
 // and 1024 sources take 59.9 ms (119 when each cell was clipped and its bounding planes
 // tracked), 25 of them the flux; 4 to 10 blocks per SM lie within 9%, 8 is the fastest.
-template <bool MERGE>
-__global__ void __launch_bounds__(128, 8)
+template <bool SHARED, bool MERGE>
+__global__ void __launch_bounds__(SHARED ? 32 * kSlots : 128, SHARED ? 4 : 8)
     cut_adjoint_kernel(TreeView T, const long long* sink_idx, int n_sink, WalkParams P, int* status,
                        AdjointArgs J) {
-  __shared__ CutStack stacks[4];
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ CutStack stacks[SHARED ? kSlots : 4];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const Share share = SHARED ? Share{warp, (int)(blockDim.x >> 5)} : Share{0, 1};
+  const int k = SHARED ? blockIdx.x * 32 + lane : blockIdx.x * 128 + threadIdx.x;
   SinkCounters cnt;
   int i = 0, slot = 0;
   float g = 0.0f;
@@ -846,21 +940,39 @@ __global__ void __launch_bounds__(128, 8)
     PlainMap<true> map{&T, sink_idx, J.grad_flux, status};
     has = map(k, i, slot, g);
   }
+  Slots none;
   if (__any_sync(0xffffffffu, has))
     cut_walk<true, MERGE, false, false, false, 1, false, false, false>(
-        T, P, has, i, g, stacks[threadIdx.x >> 5], status, J, cnt, nullptr, nullptr);
+        T, P, has, i, g, share, stacks[warp], status, J, cnt, none, nullptr, nullptr);
+}
+
+// Warps per group of 32 sinks: doubled while the call then has at most 64 warps on each of the
+// 152 SMs. At 32768 sinks of a background field 8 take 11.8 ms (1: 29.6, 4: 12.3); at 100003
+// sinks 2 take 7.80 (1: 8.31, 4: 7.83, 8: 7.99); at 65536 sinks with the particle trace 4 take
+// 39.7 (1: 59.0, 2: 50.2, 8: 43.5); at 262144 sinks one warp takes 7.5 and 2 take 8.5, since
+// every warp of a group walks the whole source tree.
+int group_warps(int n_sink) {
+  const int groups = (n_sink + 31) / 32;
+  int w = 1;
+  while (w < kSlots && 2 * w * groups <= 64 * 152) w *= 2;
+  return w;
 }
 
 template <bool MERGE, bool MOM, bool BG, bool STOP, int NB, bool SUB, bool TD>
 cudaError_t launch(const TreeView& T, const long long* sink_idx, int n_sink, const WalkParams& wp,
                    const SinkOut& out, unsigned long long* stats, int* status, cudaStream_t s) {
-  const int grid = (n_sink + 127) / 128;
-  if (!MOM && (out.counters || stats))
-    cut_walk_kernel<MERGE, MOM, BG, STOP, NB, SUB, !MOM, TD>
-        <<<grid, 128, 0, s>>>(T, sink_idx, n_sink, wp, out, stats, status);
-  else  // no counters asked for: the walk keeps none
-    cut_walk_kernel<MERGE, MOM, BG, STOP, NB, SUB, false, TD>
-        <<<grid, 128, 0, s>>>(T, sink_idx, n_sink, wp, out, nullptr, status);
+  const int w = group_warps(n_sink);
+  const int grid = w > 1 ? (n_sink + 31) / 32 : (n_sink + 127) / 128, threads = w > 1 ? 32 * w : 128;
+  auto go = [&](auto kernel, unsigned long long* st) {
+    kernel<<<grid, threads, 0, s>>>(T, sink_idx, n_sink, wp, out, st, status);
+  };
+  if (!MOM && (out.counters || stats)) {
+    if (w > 1) go(cut_walk_kernel<true, MERGE, MOM, BG, STOP, NB, SUB, !MOM, TD>, stats);
+    else go(cut_walk_kernel<false, MERGE, MOM, BG, STOP, NB, SUB, !MOM, TD>, stats);
+  } else {  // no counters asked for: the walk keeps none
+    if (w > 1) go(cut_walk_kernel<true, MERGE, MOM, BG, STOP, NB, SUB, false, TD>, nullptr);
+    else go(cut_walk_kernel<false, MERGE, MOM, BG, STOP, NB, SUB, false, TD>, nullptr);
+  }
   note_launch();
   return cudaGetLastError();
 }
@@ -910,11 +1022,18 @@ cudaError_t launch_cut_batched(const TreeView* views, float* const* flux_out, co
 cudaError_t launch_cut_adjoint(const TreeView& T, const long long* sink_idx, int n_sink,
                                const WalkParams& wp, const AdjointArgs& J, int* status,
                                cudaStream_t s) {
-  const int grid = (n_sink + 127) / 128;
-  if (wp.variant == 3)
-    cut_adjoint_kernel<true><<<grid, 128, 0, s>>>(T, sink_idx, n_sink, wp, status, J);
-  else
-    cut_adjoint_kernel<false><<<grid, 128, 0, s>>>(T, sink_idx, n_sink, wp, status, J);
+  const int w = group_warps(n_sink);
+  const int grid = w > 1 ? (n_sink + 31) / 32 : (n_sink + 127) / 128, threads = w > 1 ? 32 * w : 128;
+  auto go = [&](auto kernel) {
+    kernel<<<grid, threads, 0, s>>>(T, sink_idx, n_sink, wp, status, J);
+  };
+  if (wp.variant == 3) {
+    if (w > 1) go(cut_adjoint_kernel<true, true>);
+    else go(cut_adjoint_kernel<false, true>);
+  } else {
+    if (w > 1) go(cut_adjoint_kernel<true, false>);
+    else go(cut_adjoint_kernel<false, false>);
+  }
   note_launch();
   return cudaGetLastError();
 }
