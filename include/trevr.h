@@ -344,7 +344,7 @@ void trevr_tree_free(trevr_tree* t);
  * that reserves its device memory up front and forbids allocation inside its
  * time-step loop, or a plug-in that only receives buffers from the application
  * that owns the GPU. Its scratch memory is a fixed file-scope device array
- * sized for TREVR_NOALLOC_MAX_N particles (about 12.3 MiB, held on every GPU
+ * sized for TREVR_NOALLOC_MAX_N particles (about 12.5 MiB, held on every GPU
  * that loads the library until the process exits).
  *
  * The result is the same as the keys and the permutation of trevr_build_tree

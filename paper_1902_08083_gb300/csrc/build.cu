@@ -49,159 +49,6 @@ __global__ void keys_kernel(const float* __restrict__ xyz, const float* __restri
 }
 
 // ------------------------------------------------------------------------------------
-// Device-wide exclusive scan (unsigned, in place)
-// ------------------------------------------------------------------------------------
-__global__ void scan_tile_kernel(unsigned* data, int n, unsigned* tile_sums) {
-  __shared__ unsigned smem[32];
-  const int base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
-  unsigned v[kScanItems];
-  unsigned s = 0;
-#pragma unroll
-  for (int j = 0; j < kScanItems; ++j) {
-    v[j] = (base + j < n) ? data[base + j] : 0u;
-    s += v[j];
-  }
-  unsigned total;
-  unsigned off = block_exclusive_scan(s, smem, &total);
-#pragma unroll
-  for (int j = 0; j < kScanItems; ++j) {
-    if (base + j < n) data[base + j] = off;
-    off += v[j];
-  }
-  if (threadIdx.x == 0) tile_sums[blockIdx.x] = total;
-}
-
-__global__ void scan_add_kernel(unsigned* data, int n, const unsigned* tile_offsets) {
-  const int base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
-  const unsigned o = tile_offsets[blockIdx.x];
-#pragma unroll
-  for (int j = 0; j < kScanItems; ++j)
-    if (base + j < n) data[base + j] += o;
-}
-
-int scan_tiles(int n) { return (n + kScanTile - 1) / kScanTile; }
-
-// scratch must hold scan_scratch_words(n) unsigned
-size_t scan_scratch_words(int n) {
-  size_t w = 0;
-  while (n > 1) {
-    n = scan_tiles(n);
-    w += (size_t)n;
-  }
-  return w + 1;
-}
-
-static void exclusive_scan(unsigned* data, int n, unsigned* scratch, cudaStream_t s) {
-  if (n <= 0) return;
-  int tiles = scan_tiles(n);
-  scan_tile_kernel<<<tiles, kScanThreads, 0, s>>>(data, n, scratch);
-  note_launch();
-  if (tiles > 1) {
-    exclusive_scan(scratch, tiles, scratch + tiles, s);
-    scan_add_kernel<<<tiles, kScanThreads, 0, s>>>(data, n, scratch);
-    note_launch();
-  }
-}
-
-void exclusive_scan_u32(unsigned* data, int n, unsigned* scratch, cudaStream_t s) {
-  exclusive_scan(data, n, scratch, s);
-}
-
-// ------------------------------------------------------------------------------------
-// Stable LSD radix sort, 8-bit digits. counts layout: [digit][tile].
-// ------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSortThreads) radix_hist_kernel(
-    const unsigned long long* __restrict__ keys, int n, int shift, unsigned* __restrict__ counts,
-    int n_tiles) {
-  __shared__ unsigned hist[256];
-  for (int d = threadIdx.x; d < 256; d += blockDim.x) hist[d] = 0;
-  __syncthreads();
-  const int base = blockIdx.x * kSortTile;
-  for (int r = 0; r < kSortItems; ++r) {
-    int i = base + r * kSortThreads + threadIdx.x;
-    if (i < n) atomicAdd(&hist[(unsigned)(keys[i] >> shift) & 255u], 1u);
-  }
-  __syncthreads();
-  for (int d = threadIdx.x; d < 256; d += blockDim.x)
-    counts[(size_t)d * n_tiles + blockIdx.x] = hist[d];
-}
-
-__global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(
-    const unsigned long long* __restrict__ kin, const unsigned* __restrict__ vin,
-    unsigned long long* __restrict__ kout, unsigned* __restrict__ vout, int n, int shift,
-    const unsigned* __restrict__ offsets, int n_tiles) {
-  constexpr int kWarps = kSortThreads / 32;
-  __shared__ unsigned base_off[256];
-  __shared__ unsigned wcnt[kWarps][256];
-  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
-  for (int d = threadIdx.x; d < 256; d += blockDim.x)
-    base_off[d] = offsets[(size_t)d * n_tiles + blockIdx.x];
-  const unsigned lt_mask = (1u << lane) - 1u;
-  const int base = blockIdx.x * kSortTile;
-  for (int r = 0; r < kSortItems; ++r) {
-    for (int d = lane; d < 256; d += 32) wcnt[warp][d] = 0;
-    __syncthreads();
-    const int i = base + r * kSortThreads + threadIdx.x;
-    const bool valid = i < n;
-    unsigned long long k = valid ? kin[i] : 0ull;
-    unsigned v = valid ? vin[i] : 0u;
-    unsigned digit = valid ? ((unsigned)(k >> shift) & 255u) : 256u;
-    unsigned peers = __match_any_sync(0xffffffffu, digit);
-    unsigned rank = __popc(peers & lt_mask);
-    if (valid && rank == 0) wcnt[warp][digit] = __popc(peers);
-    __syncthreads();
-    if (valid) {
-      unsigned pos = base_off[digit] + rank;
-      for (unsigned w = 0; w < warp; ++w) pos += wcnt[w][digit];
-      kout[pos] = k;
-      vout[pos] = v;
-    }
-    __syncthreads();
-    for (int d = threadIdx.x; d < 256; d += blockDim.x) {
-      unsigned t = 0;
-#pragma unroll
-      for (int w = 0; w < kWarps; ++w) t += wcnt[w][d];
-      base_off[d] += t;
-    }
-    __syncthreads();
-  }
-}
-
-size_t sort_count_words(int n) {
-  int tiles = (n + kSortTile - 1) / kSortTile;
-  return (size_t)256 * (size_t)(tiles > 0 ? tiles : 1);
-}
-
-// Sorts (k, v) by bits [0, bits) of k; result ends in (k, v). Uses the scratch buffers.
-void radix_sort(unsigned long long* k, unsigned* v, int n, int bits, const SortScratch& S,
-                       cudaStream_t s) {
-  if (n <= 1) return;
-  const int tiles = (n + kSortTile - 1) / kSortTile;
-  const int nc = 256 * tiles;
-  unsigned long long *ka = k, *kb = S.k2;
-  unsigned *va = v, *vb = S.v2;
-  int passes = (bits + 7) / 8;
-  for (int p = 0; p < passes; ++p) {
-    int shift = 8 * p;
-    radix_hist_kernel<<<tiles, kSortThreads, 0, s>>>(ka, n, shift, S.counts, tiles);
-    note_launch();
-    exclusive_scan(S.counts, nc, S.scan_scratch, s);
-    radix_scatter_kernel<<<tiles, kSortThreads, 0, s>>>(ka, va, kb, vb, n, shift, S.counts, tiles);
-    note_launch();
-    unsigned long long* tk = ka;
-    ka = kb;
-    kb = tk;
-    unsigned* tv = va;
-    va = vb;
-    vb = tv;
-  }
-  if (ka != k) {
-    cudaMemcpyAsync(k, ka, (size_t)n * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s);
-    cudaMemcpyAsync(v, va, (size_t)n * sizeof(unsigned), cudaMemcpyDeviceToDevice, s);
-  }
-}
-
-// ------------------------------------------------------------------------------------
 // Particle gather into Morton order
 // ------------------------------------------------------------------------------------
 // Sorted particles: position relative to the domain's lower corner (u = x - lo, one
@@ -214,7 +61,7 @@ __global__ void gather_particles_kernel(const float* __restrict__ xyz,
                                         int* perm, int* rank) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  int o = (int)order[i];
+  const int o = (int)min(order[i], (unsigned)(n - 1));  // any number if the sort gave up
   pos[i] = make_float4(__fsub_rn(xyz[o], D.lo[0]), __fsub_rn(xyz[(size_t)n + o], D.lo[1]),
                        __fsub_rn(xyz[2 * (size_t)n + o], D.lo[2]), alpha[o]);
   w[i] = weight ? weight[o] : 1.0f;
@@ -245,12 +92,13 @@ struct TopoArrays {
   int bucket;
 };
 
-__global__ void topo_init_kernel(TopoArrays A, int n) {
+// After a sort that gave up there is no level at all, and the build ends with its status.
+__global__ void topo_init_kernel(TopoArrays A, int n, const int* status) {
   for (int l = threadIdx.x; l < 2 * kMaxLevels; l += blockDim.x) A.levels[l] = 0;
   __syncthreads();
   if (threadIdx.x == 0) {
     A.levels[0] = kRoot;
-    A.levels[1] = kRoot + 1;
+    A.levels[1] = (*status & kStatusIterationLimit) ? kRoot : kRoot + 1;
     A.nfirst[kRoot] = 0;
     A.ncount[kRoot] = n;
     A.nglo[kRoot] = make_int4(0, 0, 0, -1);
@@ -433,17 +281,19 @@ __global__ void src_leaf_kernel(const float* __restrict__ xyz, const float* __re
 
 // sources sorted by leaf, positions relative to the domain's lower corner
 __global__ void gather_sources_kernel(const float* __restrict__ xyz, const float* __restrict__ lum,
-                                      int n_src, Domain32 D, const unsigned* __restrict__ order,
+                                      int n_src, int n_gas, Domain32 D,
+                                      const unsigned* __restrict__ order,
                                       const unsigned long long* __restrict__ leaf_first,
                                       const int* __restrict__ leaf_of, float4* src, int* src_order,
                                       int* src_leaf) {
   int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n_src) return;
-  int o = (int)order[k];
+  const int o = (int)min(order[k], (unsigned)(n_src - 1));  // any number if the sort gave up
   src[k] = make_float4(__fsub_rn(xyz[o], D.lo[0]), __fsub_rn(xyz[(size_t)n_src + o], D.lo[1]),
                        __fsub_rn(xyz[2 * (size_t)n_src + o], D.lo[2]), lum[o]);
   src_order[k] = o;
-  src_leaf[k] = leaf_of[(int)leaf_first[k]];  // the leaf that starts at that particle
+  // the leaf that starts at that particle
+  src_leaf[k] = leaf_of[min(leaf_first[k], (unsigned long long)(n_gas - 1))];
 }
 
 __device__ __forceinline__ int lower_bound_u64(const unsigned long long* a, int n,
@@ -726,8 +576,7 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   SortScratch SS;
   SS.k2 = tmp.get<unsigned long long>(nmax);
   SS.v2 = tmp.get<unsigned>(nmax);
-  SS.counts = tmp.get<unsigned>(sort_count_words(nmax));
-  SS.scan_scratch = tmp.get<unsigned>(scan_scratch_words((int)sort_count_words(nmax)));
+  SS.work = tmp.get<unsigned>(sort_work_words(nmax));
   int* nsplit = tmp.get<int>(cap);
   int* nbit = tmp.get<int>(cap);
   unsigned* bcount = tmp.get<unsigned>(kTopoBlocks);
@@ -766,7 +615,7 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   keys_kernel<<<grid_for(n, 256), 256, 0, s>>>(gas_xyz, alpha, weight, n, D, t->key, vals,
                                                  t->status);
   note_launch();
-  radix_sort(t->key, vals, n, 63, SS, s);
+  radix_sort(t->key, vals, n, 63, SS, t->status, s);
   gather_particles_kernel<<<grid_for(n, 256), 256, 0, s>>>(gas_xyz, alpha, weight, n, D, vals,
                                                             t->pos, t->w, t->perm, t->rank);
   note_launch();
@@ -786,7 +635,7 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   TA.levels = t->levels;
   TA.bcount = bcount;
   TA.bucket = bucket;
-  topo_init_kernel<<<1, 128, 0, s>>>(TA, n);
+  topo_init_kernel<<<1, 128, 0, s>>>(TA, n, t->status);
   note_launch();
   if (!launch_topology_cooperative(TA, s)) {
     for (int L = 0; L < kMaxLevels - 1; ++L) {
@@ -802,6 +651,7 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   cudaMemcpyAsync(levels, t->levels, sizeof(levels), cudaMemcpyDeviceToHost, s);
   err = cudaStreamSynchronize(s);
   if (err != cudaSuccess) return fail(cuda_to_error(err));
+  if (levels[1] <= levels[0]) return fail(TREVR_ERR_ITERATION_LIMIT);
   int max_depth = 0;
   for (int L = 0; L < kMaxLevels; ++L)
     if (levels[2 * L + 1] > levels[2 * L]) max_depth = L;
@@ -815,8 +665,10 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
     src_leaf_kernel<<<grid_for(ns, 256), 256, 0, s>>>(src_xyz, src_lum, ns, D, t->nT, t->nglo,
                                                        t->nfirst, skeys, svals, t->status);
     note_launch();
-    radix_sort(skeys, svals, ns, 32, SS, s);
-    gather_sources_kernel<<<grid_for(ns, 256), 256, 0, s>>>(src_xyz, src_lum, ns, D, svals, skeys,
+    int bits = 1;  // keys are particle numbers
+    while (bits < 31 && ((n - 1) >> bits)) ++bits;
+    radix_sort(skeys, svals, ns, bits, SS, t->status, s);
+    gather_sources_kernel<<<grid_for(ns, 256), 256, 0, s>>>(src_xyz, src_lum, ns, n, D, svals, skeys,
                                                              t->leaf_of, t->src, t->src_order,
                                                              t->src_leaf);
     note_launch();

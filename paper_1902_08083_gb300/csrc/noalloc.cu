@@ -8,7 +8,7 @@
 // so the call itself never allocates or frees anything.
 //
 // The array is sized for at most TREVR_NOALLOC_MAX_N particles. Every GPU that
-// loads this library holds it (about 12.3 MiB) until the process exits. All
+// loads this library holds it (about 12.5 MiB) until the process exits. All
 // calls share it, and each call overwrites it: two calls whose work overlaps on
 // the GPU (other streams, other host threads) race on the same scratch.
 #include <cuda_runtime.h>
@@ -29,11 +29,10 @@ constexpr size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 // layout of the scratch array
 constexpr size_t kOffK2 = 0;
 constexpr size_t kOffV2 = kOffK2 + align256((size_t)kMaxN * sizeof(unsigned long long));
-constexpr size_t kOffCounts = kOffV2 + align256((size_t)kMaxN * sizeof(unsigned));
-constexpr size_t kCountWords = (size_t)256 * ((kMaxN + kSortTile - 1) / kSortTile);
-constexpr size_t kOffScan = kOffCounts + align256(kCountWords * sizeof(unsigned));
-constexpr size_t kScanWords = 4096;  // >= scan_scratch_words(kCountWords), checked at set-up
-constexpr size_t kOffStatus = kOffScan + align256(kScanWords * sizeof(unsigned));
+constexpr size_t kOffWork = kOffV2 + align256((size_t)kMaxN * sizeof(unsigned));
+constexpr size_t kWorkWords =
+    (size_t)kSortHead + 2 * 256 * (size_t)((kMaxN + kSortTile - 1) / kSortTile);
+constexpr size_t kOffStatus = kOffWork + align256(kWorkWords * sizeof(unsigned));
 constexpr size_t kScratchBytes = kOffStatus + 256;
 
 static __device__ __align__(256) unsigned char g_sort_scratch[kScratchBytes];
@@ -94,8 +93,7 @@ extern "C" int trevr_morton_sort_noalloc(const float* gas_xyz, long long n_gas,
   for (int d = 0; d < 3; ++d)
     if (!std::isfinite(dom->lo[d]) || !std::isfinite(dom->lo[d] + dom->side))
       return TREVR_ERR_INVALID_ARGUMENT;
-  if (scan_scratch_words((int)sort_count_words((int)n_gas)) > kScanWords)
-    return TREVR_ERR_INVALID_ARGUMENT;
+  if (sort_work_words((int)n_gas) > kWorkWords) return TREVR_ERR_INVALID_ARGUMENT;
   unsigned char* base = nullptr;
   cudaError_t err = scratch_on_current_device(&base);
   if (err != cudaSuccess) return cuda_to_error(err);
@@ -104,8 +102,7 @@ extern "C" int trevr_morton_sort_noalloc(const float* gas_xyz, long long n_gas,
   SortScratch S;
   S.k2 = reinterpret_cast<unsigned long long*>(base + kOffK2);
   S.v2 = reinterpret_cast<unsigned*>(base + kOffV2);
-  S.counts = reinterpret_cast<unsigned*>(base + kOffCounts);
-  S.scan_scratch = reinterpret_cast<unsigned*>(base + kOffScan);
+  S.work = reinterpret_cast<unsigned*>(base + kOffWork);
   int* status = reinterpret_cast<int*>(base + kOffStatus);
   // the status word must start at zero; the rest of the scratch is fully
   // overwritten before it is read
@@ -126,7 +123,7 @@ extern "C" int trevr_morton_sort_noalloc(const float* gas_xyz, long long n_gas,
                                                        reinterpret_cast<unsigned*>(perm_out),
                                                        status);
   note_launch();
-  radix_sort(keys_out, reinterpret_cast<unsigned*>(perm_out), n, 63, S, s);
+  radix_sort(keys_out, reinterpret_cast<unsigned*>(perm_out), n, 63, S, status, s);
   int h_status = 0;
   err = cudaMemcpyAsync(&h_status, status, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);

@@ -52,14 +52,11 @@ __device__ __forceinline__ unsigned long long block_reduce_add(unsigned long lon
   return s;  // valid in thread 0
 }
 
-// ---- device-wide exclusive scan of unsigned (in place), host driver in build.cu
-constexpr int kScanThreads = 256;
-constexpr int kScanItems = 4;
-constexpr int kScanTile = kScanThreads * kScanItems;
-
-// ---- LSD radix sort of (uint64 key, uint32 value), stable, 8-bit digits
+// ---- LSD radix sort of (uint64 key, uint32 value), stable, 8-bit digits (sort.cu)
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 16;
 constexpr int kSortTile = kSortThreads * kSortItems;
+constexpr int kSmallSort = 4096;         // at most so many pairs are sorted by one block
+constexpr int kSortHead = 8 * 256 + 64;  // words of the digit counts and tickets
 
 }  // namespace trevr

@@ -164,19 +164,18 @@ int build_tree_bands_impl(const float* gas_xyz, const float* alpha_bands, const 
                           long long n_src, int n_bands, const trevr_domain* dom, int bucket,
                           cudaStream_t s, trevr_tree** out, float* build_ms);
 
-// ---- build.cu: stable LSD radix sort of (uint64 key, uint32 value) pairs
+// ---- sort.cu: stable LSD radix sort of (uint64 key, uint32 value) pairs
 struct SortScratch {
   unsigned long long* k2;  // n keys
   unsigned* v2;            // n values
-  unsigned* counts;        // sort_count_words(n)
-  unsigned* scan_scratch;  // scan_scratch_words(sort_count_words(n))
+  unsigned* work;          // sort_work_words(n)
 };
-size_t sort_count_words(int n);
-size_t scan_scratch_words(int n);
-int scan_tiles(int n);
-// sorts (k, v) in place by bits [0, bits) of k
+size_t sort_work_words(int n);
+// sorts (k, v) in place by bits [0, bits) of k, with every key < 2^bits; a look-back that does
+// not end in time sets kStatusIterationLimit in *status
 void radix_sort(unsigned long long* k, unsigned* v, int n, int bits, const SortScratch& S,
-                cudaStream_t s);
+                int* status, cudaStream_t s);
+size_t scan_scratch_words(int n);
 // exclusive prefix sum of n words in place; scratch holds scan_scratch_words(n) words
 void exclusive_scan_u32(unsigned* data, int n, unsigned* scratch, cudaStream_t s);
 // ---- subbucket.cu
