@@ -80,12 +80,46 @@ static WalkParams walk_params(const trevr_tree* t, const trevr_params* prm) {
   wp.tau_stop = prm->tau_stop > 0.0f ? prm->tau_stop : INFINITY;
   wp.sub_bucket = prm->sub_bucket;
   wp.topdown = prm->ray_walk;
+  wp.order = nullptr;
   // background sources, early termination, the sub-bucket trace and the top-down ray
   // walk are built into the merged-ray walk only
   if (wp.bg_radius > 0.0f || prm->tau_stop > 0.0f || prm->sub_bucket || prm->ray_walk)
     wp.variant = 3;
   return wp;
 }
+
+// The order in which a call's listed sinks are walked: Morton order, so that the sinks of a
+// warp are neighbours. In the caller's order, one particle in ten of 2^20 (4096 sources) took
+// 31.2 ms, longer than all of them: 8 of 32 lanes ran at a time. Up to 32 sinks share a warp
+// in any order. The order costs a sort by rank; while a stream is being captured nothing is
+// allocated and the caller's order stays, as it does when there is no memory for it. A sink's
+// results do not depend on the order.
+struct SinkOrder {
+  void* buf = nullptr;
+  cudaStream_t s;
+  SinkOrder(const trevr_tree* t, const long long* sink_idx, long long n, WalkParams& wp,
+            cudaStream_t stream)
+      : s(stream) {
+    if (!sink_idx || n <= 32 || t->n_src < 4) return;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) {
+      cudaGetLastError();
+      return;
+    }
+    const size_t bytes = sink_order_bytes((int)n), own = ((size_t)n * 4 + 255) & ~(size_t)255;
+    if (pool_malloc_async(&buf, bytes + own, s) != cudaSuccess) {
+      cudaGetLastError();
+      buf = nullptr;
+      return;
+    }
+    unsigned* order = static_cast<unsigned*>(buf);
+    sink_order(t, sink_idx, (int)n, static_cast<unsigned char*>(buf) + own, order, s);
+    wp.order = order;
+  }
+  ~SinkOrder() {
+    if (buf) cudaFreeAsync(buf, s);
+  }
+};
 
 static bool params_ok(const trevr_params* prm) {
   if (!prm) return false;
@@ -216,6 +250,7 @@ int trevr_compute_flux_bands(const trevr_tree* t, const long long* sink_idx, lon
   if (!sink_idx && n_sink != t->n_gas) return TREVR_ERR_INVALID_ARGUMENT;
   cudaStream_t s = (cudaStream_t)stream;
   WalkParams wp = walk_params(t, prm);
+  const SinkOrder sorted(t, sink_idx, n_sink, wp, s);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (stats) {
     cudaMemsetAsync(t->d_stats, 0, 7 * sizeof(unsigned long long), s);
@@ -274,6 +309,7 @@ int trevr_compute_flux(const trevr_tree* t, const long long* sink_idx, long long
   if (!sink_idx && n_sink != t->n_gas) return TREVR_ERR_INVALID_ARGUMENT;
   cudaStream_t s = (cudaStream_t)stream;
   WalkParams wp = walk_params(t, prm);
+  const SinkOrder sorted(t, sink_idx, n_sink, wp, s);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (stats) {
     cudaMemsetAsync(t->d_stats, 0, 7 * sizeof(unsigned long long), s);
@@ -328,6 +364,7 @@ int trevr_compute_flux_moments(const trevr_tree* t, const long long* sink_idx, l
   if (!sink_idx && n_sink != t->n_gas) return TREVR_ERR_INVALID_ARGUMENT;
   cudaStream_t s = (cudaStream_t)stream;
   WalkParams wp = walk_params(t, prm);
+  const SinkOrder sorted(t, sink_idx, n_sink, wp, s);
   cudaError_t err = launch_walk_moments(t->view(), sink_idx, (int)n_sink, wp, flux_out, fvec_out,
                                         press_out, t->status, s);
   if (err != cudaSuccess) return cuda_to_error(err);
@@ -372,6 +409,7 @@ int trevr_compute_flux_backward(const trevr_tree* t, const long long* sink_idx, 
   J.e = buf + 5 * nc;
   double* H = buf + 5 * nc + ns;
   WalkParams wp = walk_params(t, prm);
+  const SinkOrder sorted(t, sink_idx, n_sink, wp, s);
   err = launch_walk_adjoint(t->view(), sink_idx, (int)n_sink, wp, J, t->status, s);
   if (err == cudaSuccess) err = adjoint_finalize(t, J, grad_lum, grad_alpha, H, s);
   cudaFreeAsync(buf, s);
@@ -468,6 +506,7 @@ int trevr_compute_flux_batched(trevr_batch* B, const trevr_params* prm, float* c
   wp.tau_stop = INFINITY;
   wp.sub_bucket = 0;
   wp.topdown = 0;
+  wp.order = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (stats) {
     std::memset(stats, 0, sizeof(*stats));

@@ -49,6 +49,48 @@ __global__ void keys_kernel(const float* __restrict__ xyz, const float* __restri
 }
 
 // ------------------------------------------------------------------------------------
+// Sinks of a call in Morton order
+// ------------------------------------------------------------------------------------
+__global__ void sink_keys_kernel(const long long* __restrict__ sink_idx, int n, int n_gas,
+                                 const int* __restrict__ rank,
+                                 unsigned long long* __restrict__ keys, unsigned* __restrict__ vals) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= n) return;
+  const long long si = sink_idx[k];
+  keys[k] = si >= 0 && si < n_gas ? (unsigned long long)rank[si] : (unsigned long long)n_gas;
+  vals[k] = (unsigned)k;
+}
+
+namespace {
+constexpr size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
+}
+
+size_t sink_order_bytes(int n) {
+  return 2 * align256((size_t)n * 8) + align256((size_t)n * 4) + align256(sort_work_words(n) * 4);
+}
+
+void sink_order(const trevr_tree* t, const long long* sink_idx, int n, void* scratch,
+                unsigned* order, cudaStream_t s) {
+  unsigned char* p = static_cast<unsigned char*>(scratch);
+  auto take = [&](size_t bytes) {
+    void* q = p;
+    p += align256(bytes);
+    return q;
+  };
+  unsigned long long* keys = static_cast<unsigned long long*>(take((size_t)n * 8));
+  SortScratch S;
+  S.k2 = static_cast<unsigned long long*>(take((size_t)n * 8));
+  S.v2 = static_cast<unsigned*>(take((size_t)n * 4));
+  S.work = static_cast<unsigned*>(take(sort_work_words(n) * 4));
+  const int n_gas = (int)t->n_gas;
+  sink_keys_kernel<<<(n + 255) / 256, 256, 0, s>>>(sink_idx, n, n_gas, t->rank, keys, order);
+  note_launch();
+  int bits = 1;  // keys are ranks, and n_gas itself
+  while (bits < 31 && (n_gas >> bits)) ++bits;
+  radix_sort(keys, order, n, bits, S, t->status, s);
+}
+
+// ------------------------------------------------------------------------------------
 // Particle gather into Morton order
 // ------------------------------------------------------------------------------------
 // Sorted particles: position relative to the domain's lower corner (u = x - lo, one

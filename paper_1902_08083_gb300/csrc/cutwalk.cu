@@ -806,13 +806,13 @@ __global__ void __launch_bounds__(SHARED ? 32 * kSlots : 128,
   float g = 0.0f;
   bool has = false;
   if (k < n_sink) {
-    PlainMap<false> map{&T, sink_idx, nullptr, status};
+    PlainMap<false> map{&T, sink_idx, nullptr, status, P.order, n_sink};
     has = map(k, i, slot, g);
-    if (!has && sink_idx && share.part == 0) {
+    if (!has && sink_idx && slot >= 0 && share.part == 0) {
       if (out.flux)
         for (int b = 0; b < (NB > 1 ? T.n_bands : 1); ++b)
-          out.flux[(size_t)b * out.n_out + k] = 0.0f;
-      if (out.counters) reinterpret_cast<int4*>(out.counters)[k] = make_int4(0, 0, 0, 0);
+          out.flux[(size_t)b * out.n_out + slot] = 0.0f;
+      if (out.counters) reinterpret_cast<int4*>(out.counters)[slot] = make_int4(0, 0, 0, 0);
     }
   }
   Slots flux;
@@ -937,7 +937,7 @@ __global__ void __launch_bounds__(SHARED ? 32 * kSlots : 128, SHARED ? 4 : 8)
   float g = 0.0f;
   bool has = false;
   if (k < n_sink) {
-    PlainMap<true> map{&T, sink_idx, J.grad_flux, status};
+    PlainMap<true> map{&T, sink_idx, J.grad_flux, status, P.order, n_sink};
     has = map(k, i, slot, g);
   }
   Slots none;

@@ -181,6 +181,12 @@ void exclusive_scan_u32(unsigned* data, int n, unsigned* scratch, cudaStream_t s
 // ---- subbucket.cu
 int set_smoothing_impl(trevr_tree* t, const float* h, cudaStream_t s);
 
+// ---- build.cu: the positions [0, n) of sink_idx in Morton order of their particles (those
+// out of range last) in `order`; `scratch` holds sink_order_bytes(n)
+size_t sink_order_bytes(int n);
+void sink_order(const trevr_tree* t, const long long* sink_idx, int n, void* scratch,
+                unsigned* order, cudaStream_t s);
+
 // ---- walk.cu
 struct WalkParams {
   float theta2;  // theta_open^2 (fp32)
@@ -193,6 +199,7 @@ struct WalkParams {
   float tau_stop;      // early ray termination threshold (+inf = off)
   int sub_bucket;      // sub-bucket particle trace (the tree has smoothing lengths)
   int topdown;         // 1: top-down ray walk (a ray starts as its common ancestor cell)
+  const unsigned* order;  // the order in which the sinks of sink_idx are walked, or nullptr
 };
 // accumulators of the adjoint (FP64, zeroed by the caller)
 struct AdjointArgs {

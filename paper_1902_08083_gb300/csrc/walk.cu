@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(128) walk_kernel(TreeView T, const long long* 
         }
       }
     }
-    PlainMap<ADJ> map{&T, sink_idx, J.grad_flux, status};
+    PlainMap<ADJ> map{&T, sink_idx, J.grad_flux, status, P.order, n_sink};
     run_chunk<ADJ>(T, P, (int)first, end, map, out, status, J, tot);
   }
   if (stats) add_stats(tot, stats);
@@ -856,11 +856,11 @@ __global__ void __launch_bounds__(128, 8) walk_warp_kernel(TreeView T, const lon
   float g = 0.0f;
   bool has = false;
   if (k < n_sink) {
-    PlainMap<false> map{&T, sink_idx, nullptr, status};
+    PlainMap<false> map{&T, sink_idx, nullptr, status, P.order, n_sink};
     has = map(k, i, slot, g);
-    if (!has && sink_idx) {
-      if (out.flux) out.flux[k] = 0.0f;
-      if (out.counters) reinterpret_cast<int4*>(out.counters)[k] = make_int4(0, 0, 0, 0);
+    if (!has && sink_idx && slot >= 0) {
+      if (out.flux) out.flux[slot] = 0.0f;
+      if (out.counters) reinterpret_cast<int4*>(out.counters)[slot] = make_int4(0, 0, 0, 0);
     }
   }
   CSum F;

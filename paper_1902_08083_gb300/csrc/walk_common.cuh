@@ -74,22 +74,29 @@ struct Moments {
   CSum v[9];  // x y z | xx yy zz xy xz yz
 };
 
-// Sinks of a plain call: chunk position k is the k-th requested sink.
+// Sinks of a plain call: chunk position k is the k-th requested sink, or the one that
+// `order` puts there.
 template <bool ADJ>
 struct PlainMap {
   const TreeView* T;
   const long long* sink_idx;
   const float* grad_flux;
   int* status;
+  const unsigned* order;
+  int n_sink;
   __device__ __forceinline__ bool operator()(int k, int& i, int& slot, float& g) const {
     if (sink_idx) {
-      const long long si = sink_idx[k];
+      slot = order ? (int)order[k] : k;
+      if ((unsigned)slot >= (unsigned)n_sink) {  // the order's sort gave up (status is set)
+        slot = -1;
+        return false;
+      }
+      const long long si = sink_idx[slot];
       if (si < 0 || si >= T->n_gas) {
         atomicOr(status, kStatusInvalid);
         return false;
       }
       i = T->rank[si];
-      slot = k;
     } else {
       i = k;
       slot = T->perm[k];
