@@ -1,12 +1,7 @@
 // Radiation-tree build on the GPU (Grond et al. 2019, Sec. 2.2 and 2.3):
-// Morton keys -> stable radix sort -> top-down binary tree of Morton prefixes,
-// level by level -> source deposit -> bottom-up cell moments, level by level.
-//
-// The topology pass is one cooperative launch that walks the levels with grid-wide
-// barriers (or, where that is not possible, a pair of fixed-grid launches per level
-// that read the extent of their level from device memory), so it runs without host
-// round trips; the host synchronises once, after the topology, to size the moment pass.
-#include <cooperative_groups.h>
+// Morton keys -> stable radix sort (sort.cu) -> binary tree of Morton prefixes (topology.cu) ->
+// source deposit -> bottom-up cell moments. The host synchronises once, after the topology, to
+// size the moment pass.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -15,6 +10,7 @@
 
 #include "morton.cuh"
 #include "primitives.cuh"
+#include "topology.cuh"
 #include "trevr_internal.cuh"
 
 namespace trevr {
@@ -109,182 +105,6 @@ __global__ void gather_particles_kernel(const float* __restrict__ xyz,
   w[i] = weight ? weight[o] : 1.0f;
   perm[i] = o;
   rank[o] = i;
-}
-
-// ------------------------------------------------------------------------------------
-// Topology: top-down, one level per pair of launches
-// ------------------------------------------------------------------------------------
-constexpr int kTopoBlocks = 512;
-constexpr int kTopoThreads = 256;
-
-struct TopoArrays {
-  const unsigned long long* key;
-  int* nfirst;
-  int* ncount;
-  int4* nglo;  // w = split axis (-1 leaf)
-  int4* nghi;
-  int4* nT;    // x child, y parent, z src_first, w src_count
-  int* ndepth;
-  unsigned long long* nD;  // path from the root (TreeView::nD)
-  int* nsplit;  // first particle of the upper child, -1 for a leaf
-  int* nbit;    // split key bit
-  int* leaf_of;
-  int* levels;  // [kMaxLevels][2]
-  unsigned* bcount;  // [kTopoBlocks]
-  int bucket;
-};
-
-// After a sort that gave up there is no level at all, and the build ends with its status.
-__global__ void topo_init_kernel(TopoArrays A, int n, const int* status) {
-  for (int l = threadIdx.x; l < 2 * kMaxLevels; l += blockDim.x) A.levels[l] = 0;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    A.levels[0] = kRoot;
-    A.levels[1] = (*status & kStatusIterationLimit) ? kRoot : kRoot + 1;
-    A.nfirst[kRoot] = 0;
-    A.ncount[kRoot] = n;
-    A.nglo[kRoot] = make_int4(0, 0, 0, -1);
-    A.nghi[kRoot] = make_int4(kGridMax, kGridMax, kGridMax, 0);
-    A.nT[kRoot] = make_int4(-1, 0, 0, 0);
-    A.ndepth[kRoot] = 0;
-    A.nD[kRoot] = A.nD[0] = 1ull << 63;
-    // entry 0 is unused: make it an inert leaf
-    A.nT[0] = make_int4(-1, 0, 0, 0);
-  }
-}
-
-// Values that other blocks wrote earlier in the same launch (the one-launch topology
-// below) are read through L2 (ld.global.cg): L1 is not coherent across SMs.
-__device__ __forceinline__ void level_chunk(const int* levels, int L, int* begin, int* end,
-                                            int* c0, int* c1) {
-  *begin = __ldcg(&levels[2 * L]);
-  *end = __ldcg(&levels[2 * L + 1]);
-  int m = *end - *begin;
-  int chunk = (m + gridDim.x - 1) / gridDim.x;
-  *c0 = *begin + blockIdx.x * chunk;
-  *c1 = min(*c0 + chunk, *end);
-}
-
-// Decide leaf / split for every cell of level L; count internal cells per block.
-__device__ __forceinline__ void topo_split_level(const TopoArrays& A, int L) {
-  __shared__ unsigned long long red[32];
-  int begin, end, c0, c1;
-  level_chunk(A.levels, L, &begin, &end, &c0, &c1);
-  unsigned long long cnt = 0;
-  for (int X = c0 + threadIdx.x; X < c1; X += blockDim.x) {
-    const int f = __ldcg(&A.nfirst[X]), c = __ldcg(&A.ncount[X]);
-    const unsigned long long kf = A.key[f], kl = A.key[f + c - 1];
-    if (c <= A.bucket || kf == kl) {
-      A.nsplit[X] = -1;
-      A.nT[X].x = -1;
-      A.nglo[X].w = -1;
-      for (int i = f; i < f + c; ++i) A.leaf_of[i] = X;
-    } else {
-      const int b = 63 - __clzll((long long)(kf ^ kl));
-      // first index in [f, f+c) whose key has bit b set (bit b is monotone in the range)
-      int lo = f, hi = f + c - 1;
-      while (lo < hi) {
-        int mid = lo + ((hi - lo) >> 1);
-        if ((A.key[mid] >> b) & 1ull) hi = mid;
-        else lo = mid + 1;
-      }
-      A.nsplit[X] = lo;
-      A.nbit[X] = b;
-      ++cnt;
-    }
-  }
-  unsigned long long tot = block_reduce_add(cnt, red);
-  if (threadIdx.x == 0) A.bcount[blockIdx.x] = (unsigned)tot;
-}
-
-// Allocate the children of the internal cells of level L (in cell order, two
-// consecutive slots each) and write their ranges and boxes.
-__device__ __forceinline__ void topo_emit_level(const TopoArrays& A, int L) {
-  __shared__ unsigned scan_smem[32];
-  __shared__ unsigned long long red[32];
-  int begin, end, c0, c1;
-  level_chunk(A.levels, L, &begin, &end, &c0, &c1);
-  // offset of this block = sum of the counts of the blocks before it
-  unsigned long long pre = 0, all = 0;
-  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
-    unsigned v = __ldcg(&A.bcount[b]);
-    all += v;
-    if (b < (int)blockIdx.x) pre += v;
-  }
-  pre = block_reduce_add(pre, red);
-  all = block_reduce_add(all, red);
-  __shared__ unsigned s_pre;
-  if (threadIdx.x == 0) {
-    s_pre = (unsigned)pre;
-    if (blockIdx.x == 0) {
-      A.levels[2 * (L + 1)] = end;
-      A.levels[2 * (L + 1) + 1] = end + 2 * (int)all;
-    }
-  }
-  __syncthreads();
-  unsigned running = s_pre;
-  for (int base = c0; base < c1; base += blockDim.x) {
-    const int X = base + threadIdx.x;
-    const bool internal = X < c1 && A.nsplit[X] >= 0;
-    unsigned total;
-    unsigned off = block_exclusive_scan(internal ? 1u : 0u, scan_smem, &total);
-    if (internal) {
-      const int child = end + 2 * (int)(running + off);
-      const int f = __ldcg(&A.nfirst[X]), c = __ldcg(&A.ncount[X]), k = A.nsplit[X],
-                b = A.nbit[X];
-      const int axis = (62 - b) % 3;
-      const int shift = kGridBits - 1 - (62 - b) / 3;
-      const unsigned g = key_coord(A.key[f], axis);
-      const int plane = (int)(((g >> shift) | 1u) << shift);
-      int4 lo = __ldcg(&A.nglo[X]), hi = __ldcg(&A.nghi[X]);
-      A.nT[X].x = child;
-      A.nglo[X].w = axis;
-      int4 lo1 = make_int4(lo.x, lo.y, lo.z, 0), hi1 = make_int4(hi.x, hi.y, hi.z, 0);
-      int4 lo2 = lo1, hi2 = hi1;
-      if (axis == 0) { hi1.x = plane; lo2.x = plane; }
-      else if (axis == 1) { hi1.y = plane; lo2.y = plane; }
-      else { hi1.z = plane; lo2.z = plane; }
-      A.nfirst[child] = f;
-      A.ncount[child] = k - f;
-      A.nfirst[child + 1] = k;
-      A.ncount[child + 1] = f + c - k;
-      A.nglo[child] = lo1;
-      A.nghi[child] = hi1;
-      A.nglo[child + 1] = lo2;
-      A.nghi[child + 1] = hi2;
-      A.nT[child] = make_int4(-1, X, 0, 0);
-      A.nT[child + 1] = make_int4(-1, X, 0, 0);
-      A.ndepth[child] = L + 1;
-      A.ndepth[child + 1] = L + 1;
-      const unsigned long long way = __ldcg(&A.nD[X]), end = 1ull << (62 - L);
-      A.nD[child] = way ^ (3ull * end);
-      A.nD[child + 1] = way | end;
-    }
-    running += total;
-  }
-}
-
-__global__ void __launch_bounds__(kTopoThreads) topo_split_kernel(TopoArrays A, int L) {
-  topo_split_level(A, L);
-}
-
-__global__ void __launch_bounds__(kTopoThreads) topo_emit_kernel(TopoArrays A, int L) {
-  topo_emit_level(A, L);
-}
-
-// Every level in one cooperative launch: split, grid-wide barrier, emit, barrier, until
-// a level has no cells (every block reads the same level extent after a barrier, so
-// all leave the loop together). The per-level pair of launches is the fallback when
-// a cooperative launch is not possible.
-__global__ void __launch_bounds__(kTopoThreads) topo_levels_kernel(TopoArrays A) {
-  cooperative_groups::grid_group grid = cooperative_groups::this_grid();
-  for (int L = 0; L < kMaxLevels - 1; ++L) {
-    if (__ldcg(&A.levels[2 * L + 1]) <= __ldcg(&A.levels[2 * L])) break;
-    topo_split_level(A, L);
-    grid.sync();
-    topo_emit_level(A, L);
-    grid.sync();
-  }
 }
 
 // ------------------------------------------------------------------------------------
@@ -513,31 +333,6 @@ __global__ void moments_level_kernel(MomentArrays A, int L) {
 // ------------------------------------------------------------------------------------
 namespace {
 
-// One cooperative launch of the whole topology pass, with as many blocks (at most
-// kTopoBlocks, the size of the per-block count array) as can be resident together.
-// Returns false, leaving no error behind, when the device cannot run it.
-bool launch_topology_cooperative(TopoArrays& TA, cudaStream_t s) {
-  int dev = 0, coop = 0, n_sm = 0, per_sm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, topo_levels_kernel, kTopoThreads,
-                                                    0) != cudaSuccess ||
-      !coop || per_sm < 1) {
-    cudaGetLastError();
-    return false;
-  }
-  const int grid = per_sm * n_sm < kTopoBlocks ? per_sm * n_sm : kTopoBlocks;
-  void* args[] = {&TA};
-  if (cudaLaunchCooperativeKernel((void*)topo_levels_kernel, dim3(grid), dim3(kTopoThreads), args,
-                                  0, s) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  note_launch();
-  return true;
-}
-
 struct Allocs {
   std::vector<void*> ptrs;
   cudaStream_t s;
@@ -562,7 +357,6 @@ inline int grid_for(long long n, int threads) { return (int)((n + threads - 1) /
 
 }  // namespace
 
-TreeView trevr_tree_view(const trevr_tree* t);
 
 int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weight, long long n_gas_ll,
                     const float* src_xyz, const float* src_lum, long long n_src_ll,
@@ -619,9 +413,15 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   SS.k2 = tmp.get<unsigned long long>(nmax);
   SS.v2 = tmp.get<unsigned>(nmax);
   SS.work = tmp.get<unsigned>(sort_work_words(nmax));
-  int* nsplit = tmp.get<int>(cap);
-  int* nbit = tmp.get<int>(cap);
-  unsigned* bcount = tmp.get<unsigned>(kTopoBlocks);
+  TopoArrays TA;
+  TA.up = tmp.get<int>(n);
+  TA.range = tmp.get<int2>(n);
+  TA.bit = tmp.get<unsigned char>(n);
+  TA.depth = tmp.get<unsigned char>(n);
+  TA.place = tmp.get<int>(n);
+  TA.list = tmp.get<int>(n);
+  TA.counts = tmp.get<unsigned>(topo_count_words(n));
+  unsigned* topo_scan = tmp.get<unsigned>(scan_scratch_words((int)topo_count_words(n)));
   unsigned long long* skeys = tmp.get<unsigned long long>(ns);
   unsigned* svals = tmp.get<unsigned>(ns);
 
@@ -661,9 +461,11 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   gather_particles_kernel<<<grid_for(n, 256), 256, 0, s>>>(gas_xyz, alpha, weight, n, D, vals,
                                                             t->pos, t->w, t->perm, t->rank);
   note_launch();
-  // 2. topology, top-down
-  TopoArrays TA;
+  // 2. topology
+  TA.n = n;
+  TA.bucket = bucket;
   TA.key = t->key;
+  TA.status = t->status;
   TA.nfirst = t->nfirst;
   TA.ncount = t->ncount;
   TA.nglo = t->nglo;
@@ -671,22 +473,9 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   TA.nT = t->nT;
   TA.ndepth = t->ndepth;
   TA.nD = t->nD;
-  TA.nsplit = nsplit;
-  TA.nbit = nbit;
   TA.leaf_of = t->leaf_of;
   TA.levels = t->levels;
-  TA.bcount = bcount;
-  TA.bucket = bucket;
-  topo_init_kernel<<<1, 128, 0, s>>>(TA, n, t->status);
-  note_launch();
-  if (!launch_topology_cooperative(TA, s)) {
-    for (int L = 0; L < kMaxLevels - 1; ++L) {
-      topo_split_kernel<<<kTopoBlocks, kTopoThreads, 0, s>>>(TA, L);
-      note_launch();
-      topo_emit_kernel<<<kTopoBlocks, kTopoThreads, 0, s>>>(TA, L);
-      note_launch();
-    }
-  }
+  launch_topology(TA, topo_scan, s);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return fail(cuda_to_error(err));
   int levels[2 * kMaxLevels];
@@ -755,8 +544,7 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   MA.nl2 = t->nl2;
   MA.nR = t->nR;
   MA.h = t->h;
-  // one launch per level, sized to the level (measured faster than one cooperative
-  // launch over all levels: 0.26 against 0.66 ms per build at 2^22)
+  // one launch per level, sized to the level
   for (int L = max_depth; L >= 0; --L) {
     int m = levels[2 * L + 1] - levels[2 * L];
     int blocks = grid_for(m, 128);
