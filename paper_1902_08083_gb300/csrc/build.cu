@@ -207,6 +207,7 @@ struct MomentArrays {
   float4* nS;
   float* nl2;
   float4* nR;
+  float4* nV;
   float h;
 };
 
@@ -305,12 +306,16 @@ __device__ __forceinline__ void cell_records(const MomentArrays& A, int X, const
   A.nl2[X] = l2;
   const int child = A.nT[X].x, ax = gl.w;
   float plane = 0.0f;
-  unsigned link = 3u;  // a leaf
+  unsigned link = 3u, below = 0u;  // a leaf
   if (child >= 0) {
     const int4 u = A.nglo[child + 1];
     plane = rel_plane(A.h, ax == 0 ? u.x : (ax == 1 ? u.y : u.z));
     link = ((unsigned)child >> 1) << 2 | (unsigned)ax;  // children are the pair (2k, 2k + 1)
+    below = (unsigned)child | (__double2float_rn(__ldcg(&A.mom[child].L)) > 0.0f ? 1u << 31 : 0u) |
+            (__double2float_rn(__ldcg(&A.mom[child + 1].L)) > 0.0f ? 1u : 0u);
   }
+  A.nV[2 * (size_t)X] = make_float4(blo[0], blo[1], blo[2], l2);
+  A.nV[2 * (size_t)X + 1] = make_float4(bhi[0], bhi[1], bhi[2], __uint_as_float(below));
   A.nR[X] = make_float4(abar, dal, plane, __uint_as_float(link));
   // entry 0: an empty leaf
   if (X == kRoot) A.nR[0] = make_float4(0.0f, 0.0f, 0.0f, __uint_as_float(3u));
@@ -540,6 +545,7 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   t->nS = keep.get<float4>(ncell);
   t->nl2 = keep.get<float>(ncell);
   t->nR = keep.get<float4>(ncell);
+  t->nV = keep.get<float4>(2 * ncell);
   t->nW = keep.get<double>(ncell);
   Moments* mom = tmp.get<Moments>(ncell);
   unsigned* arrived = tmp.get<unsigned>(ncell);
@@ -570,6 +576,7 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   MA.nS = t->nS;
   MA.nl2 = t->nl2;
   MA.nR = t->nR;
+  MA.nV = t->nV;
   MA.h = t->h;
   int climb = 0;  // the lowest level of the climbing launch
   while (climb < max_depth && levels[2 * climb + 3] <= kClimbCells) ++climb;

@@ -53,9 +53,14 @@ constexpr int kSegBuf = 64;  // segments of one ray kept for the adjoint's repla
 
 constexpr int kSlots = 8;    // parts of a sink's flux; at most as many warps per group
 
-struct CutStack {
-  int node[kDepth + 2];
-  unsigned mask[kDepth + 2];
+// A warp's shared memory: the walk's stack, (cell, mask of the lanes that need it) and the
+// place in a stack that holds dark cells too (stack_depth limits that one), and the queue of
+// the particle trace.
+template <bool SUB>
+struct __align__(16) CutStack {
+  float4 queue[SUB ? 64 : 1];
+  int2 e[kDepth + 2];
+  unsigned char place[kDepth + 2];
 };
 
 // A warp's share of a group's takings: those with (number & (parts - 1)) == part. parts is a
@@ -107,27 +112,20 @@ __device__ __forceinline__ float kint_phi(const float4* __restrict__ tab, float 
   return sigma < 0.0f ? -p : p;
 }
 
-// Per-warp queue of the neighbours whose support meets the chord, so that the
-// quadrature runs on full warps: (x, sigma_0, sigma_1, alpha w / (pi h^2)).
-struct SubQueue {
-  float4 g[64];
-};
-
 // Optical depth of lane src's chord p + t d, t in [t0, t1], through the particles
 // listed for its leaf, the receiving particle (sorted index si) left out. The 32
 // lanes of the warp test one neighbour each per round, with the next round's
 // entries already loading; the neighbours that reach the chord are queued in shared
-// memory and integrated 32 at a time: (Phi(x, sigma_1) - Phi(x, sigma_0)) times
+// memory, as (x, sigma_0, sigma_1, alpha w / (pi h^2)), and integrated 32 at a time: (Phi(x, sigma_1) - Phi(x, sigma_0)) times
 // alpha w / (pi h^2), with x = b^2 / h^2 and sigma = s / h. Every lane must call it;
 // all lanes return the sum.
 __device__ __forceinline__ float sub_bucket_tau_warp(const TreeView& T, int src, int box, int si,
                                                      float px, float py, float pz, float dx,
                                                      float dy, float dz, float s2, float len,
-                                                     float t0, float t1) {
+                                                     float t0, float t1,
+                                                     float4* __restrict__ queue) {
   const unsigned FULL = 0xffffffffu;
   const unsigned lane = threadIdx.x & 31u;
-  __shared__ SubQueue queues[kSlots];  // one per warp of a block
-  SubQueue& Q = queues[threadIdx.x >> 5];
   box = __shfl_sync(FULL, box, src);
   si = __shfl_sync(FULL, si, src);
   px = __shfl_sync(FULL, px, src);
@@ -178,20 +176,20 @@ __device__ __forceinline__ float sub_bucket_tau_warp(const TreeView& T, int src,
     const unsigned m = __ballot_sync(FULL, pass);
     if (pass) {
       const float ih = q.w;
-      Q.g[qn + __popc(m & ((1u << lane) - 1u))] =
+      queue[qn + __popc(m & ((1u << lane) - 1u))] =
           make_float4(x, sa, sb, a * (ih * ih * 0.318309886f));
     }
     qn += __popc(m);
     __syncwarp();
     if (qn >= 32) {
-      const float4 g = Q.g[qn - 32 + (int)lane];
+      const float4 g = queue[qn - 32 + (int)lane];
       part += g.w * (kint_phi(T.kint4, g.x, g.z) - kint_phi(T.kint4, g.x, g.y));
       qn -= 32;
       __syncwarp();
     }
   }
   if ((int)lane < qn) {
-    const float4 g = Q.g[lane];
+    const float4 g = queue[lane];
     part += g.w * (kint_phi(T.kint4, g.x, g.z) - kint_phi(T.kint4, g.x, g.y));
   }
   __syncwarp();
@@ -375,7 +373,8 @@ template <bool ADJ, bool MOM, bool BG, bool STOP, int NB, bool SUB, bool CNT, bo
 __device__ __forceinline__ void cut_ray(const TreeView& T, const WalkParams& P, const float tref,
                                         const bool on, const int ent, const Sink& K, Line& ray,
                                         Pieces<ADJ>& W, const AdjointArgs& J, SinkCounters& cnt,
-                                        const int slot, Slots& flux, CSum* F, Moments* mom) {
+                                        const int slot, Slots& flux, CSum* F, Moments* mom,
+                                        float4* queue) {
   const unsigned FULL = 0xffffffffu;
   float L = 0.0f;
   int C = kRoot;
@@ -431,7 +430,7 @@ __device__ __forceinline__ void cut_ray(const TreeView& T, const WalkParams& P, 
         r = __ldg(&T.nR[cell]);
       }
       float a, b;
-      ray.clip(__ldg(&T.nA[cell]), __ldg(&T.nB[cell]), a, b);
+      ray.clip(__ldg(&T.nV[2 * (size_t)cell]), __ldg(&T.nV[2 * (size_t)cell + 1]), a, b);
       if (TD || ds == dS || ds == dC) {  // one piece: A, or S = C
         if (CNT) ++cnt.clip;
         if (a < b) {
@@ -602,7 +601,7 @@ __device__ __forceinline__ void cut_ray(const TreeView& T, const WalkParams& P, 
           const int src = __ffs(m) - 1;
           m &= m - 1u;
           const float t = sub_bucket_tau_warp(T, src, sub_box, K.i, ray.px, ray.py, ray.pz, ray.dx,
-                                              ray.dy, ray.dz, ray.s2, ray.len, sub_t0, sub_t1);
+                                              ray.dy, ray.dz, ray.s2, ray.len, sub_t0, sub_t1, queue);
           if ((int)(threadIdx.x & 31u) == src) tau.add(t);
         }
       }
@@ -672,10 +671,15 @@ __device__ __forceinline__ void cut_ray(const TreeView& T, const WalkParams& P, 
 // The walk of the 32 sinks of one warp (a lane holds the sorted position i if `has`);
 // every lane of the warp must call it. MERGE: a ray waits until its lane gets
 // another; without it (variant 2) the rays to a cell are traced as soon as it is accepted.
+// A step of the walk is a chain of loads for all lanes, and below some 10^5 sinks that chain is
+// what it takes. So a cell is two 16-byte loads that are on their way together (they were five
+// in three arrays, one behind another), dark children are never pushed, and an opened leaf's
+// sources are looked at 32 at a time: 7.35 -> 7.05 ms at 100003 sinks, 10.8 -> 9.6 for a
+// background field at 32768, 0.52 -> 0.48 for a step of 4096, 54.1 -> 53.2 at 2^22.
 template <bool ADJ, bool MERGE, bool MOM, bool BG, bool STOP, int NB, bool SUB, bool CNT, bool TD>
 __device__ __forceinline__ void cut_walk(const TreeView& T, const WalkParams& P, const bool has,
                                          const int i, const float grad, const Share share,
-                                         CutStack& ws, int* status, const AdjointArgs& J,
+                                         CutStack<SUB>& ws, int* status, const AdjointArgs& J,
                                          SinkCounters& cnt, Slots& flux, CSum* F, Moments* mom) {
   const unsigned FULL = 0xffffffffu;
   const unsigned lane = threadIdx.x & 31u;
@@ -694,85 +698,106 @@ __device__ __forceinline__ void cut_walk(const TreeView& T, const WalkParams& P,
     K.way = __ldg(&T.nD[T.leaf_of[i]]);
   }
   const unsigned live = __ballot_sync(FULL, has);
-  if (lane == 0) {
-    ws.node[0] = kRoot;
-    ws.mask[0] = live;
+  int sp = 0;
+  if (live && __ldg(&T.nS[kRoot].w) > 0.0f) {
+    if (lane == 0) {
+      ws.e[0] = make_int2(kRoot, (int)live);
+      ws.place[0] = 0;
+    }
+    sp = 1;
   }
-  int sp = live ? 1 : 0;
   bool wait = false;      // this lane has a ray that waits to be traced, to w_ent
   int w_ent = 0;          // (a cell, or ~source)
-  int j = 0, j_end = 0;   // sources of the opened leaf still to be taken
+  int j = 0, j_end = 0;   // sources of the opened leaf from j on are still to be looked at
   unsigned opened = 0;    // the lanes that opened it
+  unsigned lit = 0, own = 0;  // of the 32 sources before j: those with light, this warp's of them
+  int first = 0;              // number of the takings before the first of `lit`
   int taken = 0, w_slot = 0;  // takings so far; the slot of the waiting ray
   if (!ADJ && NB == 1) flux.clear();
   __syncwarp();
   while (true) {
-    bool take = false;
-    int ent = 0;
-    const bool done = j >= j_end && sp == 0;
-    if (j < j_end) {
-      if (__ldg(&T.src[j].w) > 0.0f) {
-        take = (opened >> lane) & 1u;
-        ent = ~j;
-      }
-      ++j;
-    } else if (!done) {
+    bool take = false, done = false;
+    int ent = 0, turn = 0;
+    if (own) {
+      const int q = __ffs(own) - 1;
+      own &= own - 1u;
+      ent = ~(j - 32 + q);
+      turn = first + __popc(lit & ((1u << q) - 1u));
+      take = (opened >> lane) & 1u;
+    } else if (j < j_end) {
+      const int mine = j + (int)lane;
+      const bool light = mine < j_end && __ldg(&T.src[mine].w) > 0.0f;
+      lit = __ballot_sync(FULL, light);
+      first = taken;
+      const int number = first + __popc(lit & ((1u << lane) - 1u));
+      own = __ballot_sync(FULL, light && (number & (share.parts - 1)) == share.part);
+      taken += __popc(lit);
+      j += 32;
+      continue;
+    } else if (sp > 0) {
       --sp;
-      const int X = ws.node[sp];
-      const unsigned M = ws.mask[sp];
+      const int2 top = ws.e[sp];
+      const int X = top.x, place = ws.place[sp];
       __syncwarp();
-      const float4 s = __ldg(&T.nS[X]);
+      const float4 lo = __ldg(&T.nV[2 * (size_t)X]), hi = __ldg(&T.nV[2 * (size_t)X + 1]);
+      const unsigned below = __float_as_uint(hi.w);
       bool open = false;
-      if (s.w > 0.0f && ((M >> lane) & 1u)) {
+      if (((unsigned)top.y >> lane) & 1u) {
         if (CNT && share.part == 0) ++cnt.visit;
-        const float4 a = __ldg(&T.nA[X]);
-        const float4 bb = __ldg(&T.nB[X]);
-        const float ex = fmaxf(fmaxf(__fsub_rn(a.x, ray.px), __fsub_rn(ray.px, bb.x)), 0.0f);
-        const float ey = fmaxf(fmaxf(__fsub_rn(a.y, ray.py), __fsub_rn(ray.py, bb.y)), 0.0f);
-        const float ez = fmaxf(fmaxf(__fsub_rn(a.z, ray.pz), __fsub_rn(ray.pz, bb.z)), 0.0f);
+        const float ex = fmaxf(fmaxf(__fsub_rn(lo.x, ray.px), __fsub_rn(ray.px, hi.x)), 0.0f);
+        const float ey = fmaxf(fmaxf(__fsub_rn(lo.y, ray.py), __fsub_rn(ray.py, hi.y)), 0.0f);
+        const float ez = fmaxf(fmaxf(__fsub_rn(lo.z, ray.pz), __fsub_rn(ray.pz, hi.z)), 0.0f);
         const float r2 =
             __fadd_rn(__fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey)), __fmul_rn(ez, ez));
-        take = __ldg(&T.nl2[X]) < __fmul_rn(P.theta2, r2);
+        take = lo.w < __fmul_rn(P.theta2, r2);
         open = !take;
       }
       ent = X;
       const unsigned openM = __ballot_sync(FULL, open);
       if (openM) {
-        const int4 t = __ldg(&T.nT[X]);
-        if (t.x < 0) {
+        const int child = (int)(below & 0x7ffffffeu);
+        if (child == 0) {
+          const int4 t = __ldg(&T.nT[X]);
           j = t.z;
           j_end = t.z + t.w;
           opened = openM;
-        } else if (sp + 2 > stack_limit) {
+        } else if (place + 2 > stack_limit) {
           if (lane == 0) atomicOr(status, kStatusStackOverflow);
           sp = 0;
-        } else {
-          if (lane == 0) {
-            ws.node[sp] = t.x + 1;
-            ws.mask[sp] = openM;
-            ws.node[sp + 1] = t.x;
-            ws.mask[sp + 1] = openM;
+        } else {  // the children with light, the lower one on top
+          if (below & 1u) {
+            if (lane == 0) {
+              ws.e[sp] = make_int2(child + 1, (int)openM);
+              ws.place[sp] = (unsigned char)place;
+            }
+            ++sp;
           }
-          sp += 2;
+          if (below >> 31) {
+            if (lane == 0) {
+              ws.e[sp] = make_int2(child, (int)openM);
+              ws.place[sp] = (unsigned char)(place + 1);
+            }
+            ++sp;
+          }
           __syncwarp();
         }
       }
-    }
-    if (!done) {
       if (!__any_sync(FULL, take)) continue;
-      const int turn = taken++;
+      turn = taken++;
       if ((turn & (share.parts - 1)) != share.part) continue;
+    } else {
+      done = true;
     }
     if (__any_sync(FULL, wait && (done || take || !MERGE))) {
       cut_ray<ADJ, MOM, BG, STOP, NB, SUB, CNT, TD>(T, P, tref, wait, w_ent, K, ray, W, J, cnt,
-                                                    w_slot, flux, F, mom);
+                                                    w_slot, flux, F, mom, ws.queue);
       wait = false;
     }
     if (done) break;
     if (take) {
       wait = true;
       w_ent = ent;
-      w_slot = (taken - 1) & (kSlots - 1);
+      w_slot = turn & (kSlots - 1);
     }
   }
 }
@@ -784,20 +809,24 @@ __device__ __forceinline__ void cut_walk(const TreeView& T, const WalkParams& P,
 // 56.7 ms (21.4 and 8.3 ms at 100003 sinks, tau_ref = 0.01).
 // Blocks of 128 per SM: 8 leave the plain walk its registers (61, no spills); 12 and 16 (40
 // and 32 registers) gave 58.9 and 55.9 ms at 2^22 but 9.5 and 10.1 ms at 100003 sinks, where
-// a warp's own speed counts and 8 took 8.4. The particle trace needs 4 (57.2 ms at 2^16
+// a warp's own speed counts and 8 took 8.4. The particle trace needs 4 or 5 (57.2 ms at 2^16
 // sinks, against 66.9 at 6 and 72.4 at 8), the bands 6 (8.95 ms for three at 200003 sinks,
 // 9.2 at 8).
-constexpr int cut_blocks(bool SUB, int NB) { return SUB ? 4 : NB > 1 ? 6 : 8; }
+constexpr int cut_blocks(bool SUB, int NB) { return SUB ? 5 : NB > 1 ? 6 : 8; }
+// warps per group at most: the particle trace keeps 5 blocks of 4
+constexpr int most_warps(bool SUB) { return SUB ? 4 : kSlots; }
 
 // SHARED: the block's warps (a power of two, at most kSlots) share one group of 32 sinks.
 template <bool SHARED, bool MERGE, bool MOM, bool BG, bool STOP, int NB, bool SUB, bool CNT,
           bool TD>
-__global__ void __launch_bounds__(SHARED ? 32 * kSlots : 128,
-                                  SHARED ? cut_blocks(SUB, NB) / 2 : cut_blocks(SUB, NB))
+__global__ void __launch_bounds__(SHARED && !SUB ? 32 * kSlots : 128,
+                                  SHARED && !SUB ? cut_blocks(SUB, NB) / 2 : cut_blocks(SUB, NB))
     cut_walk_kernel(TreeView T, const long long* sink_idx, int n_sink, WalkParams P, SinkOut out,
                     unsigned long long* stats, int* status) {
-  __shared__ CutStack stacks[SHARED ? kSlots : 4];
-  __shared__ float2 parts[SHARED ? kSlots : 1][32];
+  // the warps' stacks, and after the walk the parts of the group's sums
+  extern __shared__ float4 block_memory[];
+  CutStack<SUB>* stacks = reinterpret_cast<CutStack<SUB>*>(block_memory);
+  float2(*parts)[32] = reinterpret_cast<float2(*)[32]>(block_memory);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Share share = SHARED ? Share{warp, (int)(blockDim.x >> 5)} : Share{0, 1};
   const int k = SHARED ? blockIdx.x * 32 + lane : blockIdx.x * 128 + threadIdx.x;
@@ -825,6 +854,7 @@ __global__ void __launch_bounds__(SHARED ? 32 * kSlots : 128,
   else if (NB == 1)
     flux.clear();
   if (CNT && stats) add_stats(cnt, stats);
+  if (SHARED) __syncthreads();
   // the group's sums, in warp 0 (every warp of the block comes here)
   auto gather = [&](CSum& v) {
     parts[SHARED ? warp : 0][lane] = make_float2(v.s, v.c);
@@ -891,8 +921,8 @@ __global__ void __launch_bounds__(BS, 1024 / BS) cut_walk_batched_kernel(
     const TreeView* __restrict__ views, float* const* __restrict__ flux_out,
     const int2* __restrict__ items, int n_items, int item, unsigned* counter, WalkParams P,
     unsigned long long* stats, int* status) {
-  __shared__ CutStack stacks[BS / 32];
-  CutStack& ws = stacks[threadIdx.x >> 5];
+  __shared__ CutStack<false> stacks[BS / 32];
+  CutStack<false>& ws = stacks[threadIdx.x >> 5];
   const unsigned lane = threadIdx.x & 31u;
   SinkCounters tot;
   while (true) {
@@ -928,7 +958,8 @@ template <bool SHARED, bool MERGE>
 __global__ void __launch_bounds__(SHARED ? 32 * kSlots : 128, SHARED ? 4 : 8)
     cut_adjoint_kernel(TreeView T, const long long* sink_idx, int n_sink, WalkParams P, int* status,
                        AdjointArgs J) {
-  __shared__ CutStack stacks[SHARED ? kSlots : 4];
+  extern __shared__ float4 block_memory[];
+  CutStack<false>* stacks = reinterpret_cast<CutStack<false>*>(block_memory);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Share share = SHARED ? Share{warp, (int)(blockDim.x >> 5)} : Share{0, 1};
   const int k = SHARED ? blockIdx.x * 32 + lane : blockIdx.x * 128 + threadIdx.x;
@@ -951,20 +982,28 @@ __global__ void __launch_bounds__(SHARED ? 32 * kSlots : 128, SHARED ? 4 : 8)
 // sinks 2 take 7.80 (1: 8.31, 4: 7.83, 8: 7.99); at 65536 sinks with the particle trace 4 take
 // 39.7 (1: 59.0, 2: 50.2, 8: 43.5); at 262144 sinks one warp takes 7.5 and 2 take 8.5, since
 // every warp of a group walks the whole source tree.
-int group_warps(int n_sink) {
+int group_warps(int n_sink, int most) {
   const int groups = (n_sink + 31) / 32;
   int w = 1;
-  while (w < kSlots && 2 * w * groups <= 64 * 152) w *= 2;
+  while (w < most && 2 * w * groups <= 64 * 152) w *= 2;
   return w;
+}
+
+// Shared memory of a block, for the warps that it has: blocks of two warps with room for eight
+// took 9.9 ms for 100003 sinks instead of 7.3, since what they hold is taken from L1.
+template <bool SUB>
+size_t block_bytes(int w) {
+  const size_t stacks = (w > 1 ? w : 4) * sizeof(CutStack<SUB>), sums = kSlots * 32 * sizeof(float2);
+  return w > 1 && stacks < sums ? sums : stacks;
 }
 
 template <bool MERGE, bool MOM, bool BG, bool STOP, int NB, bool SUB, bool TD>
 cudaError_t launch(const TreeView& T, const long long* sink_idx, int n_sink, const WalkParams& wp,
                    const SinkOut& out, unsigned long long* stats, int* status, cudaStream_t s) {
-  const int w = group_warps(n_sink);
+  const int w = group_warps(n_sink, most_warps(SUB));
   const int grid = w > 1 ? (n_sink + 31) / 32 : (n_sink + 127) / 128, threads = w > 1 ? 32 * w : 128;
   auto go = [&](auto kernel, unsigned long long* st) {
-    kernel<<<grid, threads, 0, s>>>(T, sink_idx, n_sink, wp, out, st, status);
+    kernel<<<grid, threads, block_bytes<SUB>(w), s>>>(T, sink_idx, n_sink, wp, out, st, status);
   };
   if (!MOM && (out.counters || stats)) {
     if (w > 1) go(cut_walk_kernel<true, MERGE, MOM, BG, STOP, NB, SUB, !MOM, TD>, stats);
@@ -1022,10 +1061,10 @@ cudaError_t launch_cut_batched(const TreeView* views, float* const* flux_out, co
 cudaError_t launch_cut_adjoint(const TreeView& T, const long long* sink_idx, int n_sink,
                                const WalkParams& wp, const AdjointArgs& J, int* status,
                                cudaStream_t s) {
-  const int w = group_warps(n_sink);
+  const int w = group_warps(n_sink, kSlots);
   const int grid = w > 1 ? (n_sink + 31) / 32 : (n_sink + 127) / 128, threads = w > 1 ? 32 * w : 128;
   auto go = [&](auto kernel) {
-    kernel<<<grid, threads, 0, s>>>(T, sink_idx, n_sink, wp, status, J);
+    kernel<<<grid, threads, block_bytes<false>(w), s>>>(T, sink_idx, n_sink, wp, status, J);
   };
   if (wp.variant == 3) {
     if (w > 1) go(cut_adjoint_kernel<true, true>);

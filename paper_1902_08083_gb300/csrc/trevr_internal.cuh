@@ -51,6 +51,8 @@ struct TreeView {
   const float* nl2;  // l^2 (furthest vertex from the centre of luminosity)
   const float4* nR;  // what a ray needs of a cell it cuts: (abar, alpha_max - alpha_min, split
                      // plane relative to lo, bits (child / 2) << 2 | split axis; 3 = leaf)
+  const float4* nV;  // what the source walk needs of a cell, two per cell: (lo, l^2) and (hi,
+                     // bits child | lower child lit << 31 | upper child lit); child 0 = leaf
   const unsigned long long* nD;  // path from the root: first cut in bit 63 (1 = upper child),
                                  // then a 1 that ends it, in bit 63 - depth
   const int* ndepth;
@@ -117,6 +119,7 @@ struct trevr_tree {
   int4* nT;
   float* nl2;
   float4* nR;
+  float4* nV;
   unsigned long long* nD;
   int* ndepth;
   int* nfirst;

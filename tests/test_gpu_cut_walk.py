@@ -71,3 +71,33 @@ def test_few_and_equal_points(n):
     f, c = trevr.compute_flux(G, 0.5, 0.01, counters=True)
     np.testing.assert_allclose(f.cpu().numpy(), f1.cpu().numpy(), rtol=2e-5, atol=1e-30)
     np.testing.assert_array_equal(c.cpu().numpy(), rc.astype(np.int32))
+
+
+@pytest.mark.parametrize("n_src", [1, 31, 32, 33, 64, 65, 100])
+@pytest.mark.parametrize("n_gas", [5, 600])
+def test_many_sources_in_a_leaf(n_gas, n_src):
+    # every other source dark, all within one leaf's cell
+    from paper_1902_08083_gb300 import trevr
+    rng = np.random.default_rng(n_src)
+    P = workloads.uniform_box(n_gas=n_gas, n_src=n_src, seed=n_src)
+    P["src_xyz"] = (0.3 + 0.004 * rng.random((3, n_src))).astype(np.float32)
+    P["src_lum"][1::2] = 0.0
+    P["alpha"] = rng.lognormal(0.0, 1.0, n_gas).astype(np.float32)
+    G = gpu_tree(P)
+    ref, rc, _ = oracle_tree(P).flux(0.3, 0.1, with_counters=True)
+    f, c = trevr.compute_flux(G, 0.3, 0.1, counters=True)
+    np.testing.assert_array_equal(c.cpu().numpy(), rc.astype(np.int32))
+    np.testing.assert_allclose(f.cpu().numpy(), ref, rtol=1e-3)  # the parity tests' bound
+
+
+def test_stack_limit_counts_dark_cells():
+    # sources in one corner: a stack of two entries has no room below the root's children,
+    # whether or not their siblings hold light
+    from paper_1902_08083_gb300 import trevr
+    P = workloads.uniform_box(n_gas=4096, n_src=40, seed=3)
+    P["src_xyz"] = (P["src_xyz"] * np.float32(0.1)).astype(np.float32)
+    G = gpu_tree(P)
+    with pytest.raises(trevr.TrevrError) as ei:
+        trevr.compute_flux(G, 0.1, 0.1, stats=True, stack_depth=2)
+    assert ei.value.code == 3
+    trevr.compute_flux(G, 0.1, 0.1, stats=True)
