@@ -170,7 +170,6 @@ TreeView trevr_tree::view() const {
   v.src = src;
   v.src_order = src_order;
   v.src_leaf = src_leaf;
-  v.n_nodes = d_n_nodes;
   v.n_bands = n_bands;
   v.bA = bA;
   v.bLc = bLc;
@@ -202,9 +201,8 @@ int trevr_build_tree(const float* gas_xyz, const float* alpha, const float* weig
   for (int d = 0; d < 3; ++d)
     if (!std::isfinite(dom->lo[d]) || !std::isfinite(dom->lo[d] + dom->side))
       return TREVR_ERR_INVALID_ARGUMENT;
-  float ms = 0.0f;
   return build_tree_impl(gas_xyz, alpha, weight, n_gas, src_xyz, src_lum, n_src, dom,
-                         prm->bucket, (cudaStream_t)stream, out, &ms);
+                         prm->bucket, (cudaStream_t)stream, out);
 }
 
 int trevr_build_tree_bands(const float* gas_xyz, const float* alpha_bands, const float* weight,
@@ -225,9 +223,8 @@ int trevr_build_tree_bands(const float* gas_xyz, const float* alpha_bands, const
   for (int d = 0; d < 3; ++d)
     if (!std::isfinite(dom->lo[d]) || !std::isfinite(dom->lo[d] + dom->side))
       return TREVR_ERR_INVALID_ARGUMENT;
-  float ms = 0.0f;
   return build_tree_bands_impl(gas_xyz, alpha_bands, weight, n_gas, src_xyz, lum_bands, n_src,
-                               n_bands, dom, prm->bucket, (cudaStream_t)stream, out, &ms);
+                               n_bands, dom, prm->bucket, (cudaStream_t)stream, out);
 }
 
 int trevr_tree_set_smoothing(trevr_tree* t, const float* hsml, void* stream) {
@@ -672,11 +669,8 @@ void trevr_tree_free(trevr_tree* t) {
   cudaGetDevice(&cur);
   cudaSetDevice(t->device);
   cudaDeviceSynchronize();
-  void* ptrs[] = {t->nR, t->nV, t->nD, t->key, t->perm,   t->rank,   t->leaf_of, t->pos,    t->w,      t->nA,
-                  t->nB,  t->nS,     t->nT,     t->nl2,     t->ndepth, t->nfirst, t->ncount,
-                  t->nglo, t->nghi,  t->src,    t->src_order, t->levels, t->d_n_nodes,
-                  t->status, t->d_stats, t->src_leaf, t->nW, t->bA, t->bLc, t->bLs, t->sp, t->aw,
-                  t->dbk, t->nbr_first, t->nbr_ja, t->nbr_sp, t->kint4};
+  void* ptrs[] = {t->mem[0], t->mem[1], t->bA,        t->bLc,    t->bLs,    t->sp,
+                  t->aw,     t->dbk,    t->nbr_first, t->nbr_ja, t->nbr_sp, t->kint4};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   cudaSetDevice(cur);

@@ -140,7 +140,7 @@ inline int grid_of(long long n, int threads) {
 int build_tree_bands_impl(const float* gas_xyz, const float* alpha_bands, const float* weight,
                           long long n_gas, const float* src_xyz, const float* lum_bands,
                           long long n_src, int n_bands, const trevr_domain* dom, int bucket,
-                          cudaStream_t s, trevr_tree** out, float* build_ms) {
+                          cudaStream_t s, trevr_tree** out) {
   const int n = (int)n_gas, ns = (int)n_src, nb = n_bands;
   float* lsum = nullptr;
   int* st = nullptr;
@@ -165,18 +165,13 @@ int build_tree_bands_impl(const float* gas_xyz, const float* alpha_bands, const 
     return e != cudaSuccess ? cuda_to_error(e) : status_to_error(bad);
   }
   trevr_tree* t = nullptr;
-  float ms = 0.0f;
   int rc = build_tree_impl(gas_xyz, alpha_bands, weight, n_gas, src_xyz, lsum, n_src, dom, bucket,
-                           s, &t, &ms);
+                           s, &t);
   cudaFreeAsync(lsum, s);
   if (rc != TREVR_OK) {
     cudaFreeAsync(st, s);
     return rc;
   }
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  cudaEventCreate(&e0);
-  cudaEventCreate(&e1);
-  cudaEventRecord(e0, s);
   const size_t ncell = (size_t)t->n_nodes + kRoot;
   float* as = nullptr;
   BandMom* mom = nullptr;
@@ -226,21 +221,15 @@ int build_tree_bands_impl(const float* gas_xyz, const float* alpha_bands, const 
   }
   if (as) cudaFreeAsync(as, s);
   if (mom) cudaFreeAsync(mom, s);
-  cudaEventRecord(e1, s);
   bad = 0;
   cudaMemcpyAsync(&bad, st, sizeof(int), cudaMemcpyDeviceToHost, s);
   const cudaError_t e2 = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = e2;
-  float ms2 = 0.0f;
-  if (e == cudaSuccess) cudaEventElapsedTime(&ms2, e0, e1);
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
   cudaFree(st);
   if (e != cudaSuccess || bad) {
     trevr_tree_free(t);
     return e != cudaSuccess ? cuda_to_error(e) : status_to_error(bad);
   }
-  if (build_ms) *build_ms = ms + ms2;
   *out = t;
   return TREVR_OK;
 }

@@ -6,7 +6,6 @@
 #include <stdint.h>
 
 #include <cstring>
-#include <vector>
 
 #include "morton.cuh"
 #include "primitives.cuh"
@@ -172,13 +171,14 @@ __device__ __forceinline__ int lower_bound_u64(const unsigned long long* a, int 
 __global__ void node_src_range_kernel(int n_cells_end, const int* __restrict__ nfirst,
                                       const int* __restrict__ ncount,
                                       const unsigned long long* __restrict__ src_keys, int n_src,
-                                      int4* nT) {
+                                      int4* nT, unsigned* arrived) {
   int X = blockIdx.x * blockDim.x + threadIdx.x + kRoot;
   if (X >= n_cells_end) return;
   int a = lower_bound_u64(src_keys, n_src, (unsigned long long)nfirst[X]);
   int b = lower_bound_u64(src_keys, n_src, (unsigned long long)(nfirst[X] + ncount[X]));
   nT[X].z = a;
   nT[X].w = b - a;
+  arrived[X] = 0;  // for the climb of the moments
 }
 
 // ------------------------------------------------------------------------------------
@@ -317,8 +317,13 @@ __device__ __forceinline__ void cell_records(const MomentArrays& A, int X, const
   A.nV[2 * (size_t)X] = make_float4(blo[0], blo[1], blo[2], l2);
   A.nV[2 * (size_t)X + 1] = make_float4(bhi[0], bhi[1], bhi[2], __uint_as_float(below));
   A.nR[X] = make_float4(abar, dal, plane, __uint_as_float(link));
-  // entry 0: an empty leaf
-  if (X == kRoot) A.nR[0] = make_float4(0.0f, 0.0f, 0.0f, __uint_as_float(3u));
+  if (X == kRoot) {  // entry 0: an empty leaf without light
+    const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    A.nA[0] = A.nB[0] = A.nS[0] = A.nV[0] = A.nV[1] = zero;
+    A.nR[0] = make_float4(0.0f, 0.0f, 0.0f, __uint_as_float(3u));
+    A.nl2[0] = 0.0f;
+    A.nW[0] = 0.0;
+  }
 }
 
 // The moments of the levels up to the one that ends at `end`, whose lower levels are done: a
@@ -359,25 +364,33 @@ __global__ void moments_level_kernel(MomentArrays A, int L) {
 // ------------------------------------------------------------------------------------
 namespace {
 
-struct Allocs {
-  std::vector<void*> ptrs;
-  cudaStream_t s;
-  bool ok = true;
+// Arrays laid out one behind another, 256 bytes apart, in one block of the pool: a first pass
+// over the layout adds up the sizes, a second hands out the addresses. A build made 35
+// allocations and its tree's end 36 frees, about 100 us of host time, on the way of the next
+// step's first launch.
+struct Layout {
+  char* base;
+  size_t at;
   template <class T>
-  T* get(size_t n) {
-    void* p = nullptr;
-    if (pool_malloc_async(&p, (n ? n : 1) * sizeof(T), s) != cudaSuccess) {
-      ok = false;
-      return nullptr;
-    }
-    ptrs.push_back(p);
-    return (T*)p;
-  }
-  void release() {
-    for (void* p : ptrs) cudaFreeAsync(p, s);
-    ptrs.clear();
+  void get(T*& p, size_t n) {
+    p = base ? reinterpret_cast<T*>(base + at) : nullptr;
+    at += ((n ? n : 1) * sizeof(T) + 255) & ~(size_t)255;
   }
 };
+
+template <class F>
+void* allocate(const F& arrays, cudaStream_t s) {
+  Layout sizes{nullptr, 0};
+  arrays(sizes);
+  void* p = nullptr;
+  if (pool_malloc_async(&p, sizes.at, s) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  Layout places{static_cast<char*>(p), 0};
+  arrays(places);
+  return p;
+}
 
 inline int grid_for(long long n, int threads) { return (int)((n + threads - 1) / threads); }
 
@@ -391,15 +404,9 @@ constexpr int kClimbCells = 131072;
 
 int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weight, long long n_gas_ll,
                     const float* src_xyz, const float* src_lum, long long n_src_ll,
-                    const trevr_domain* dom, int bucket, cudaStream_t s, trevr_tree** out,
-                    float* build_ms) {
+                    const trevr_domain* dom, int bucket, cudaStream_t s, trevr_tree** out) {
   const int n = (int)n_gas_ll;
   const int ns = (int)n_src_ll;
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  cudaEventCreate(&e0);
-  cudaEventCreate(&e1);
-  cudaEventRecord(e0, s);
-
   trevr_tree* t = new trevr_tree();
   std::memset(t, 0, sizeof(*t));
   cudaGetDevice(&t->device);
@@ -415,62 +422,69 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   const size_t cap = 2 * (size_t)n + 2;
   t->cap_nodes = cap;
 
-  Allocs keep{{}, s}, tmp{{}, s};
-  // persistent
-  t->key = keep.get<unsigned long long>(n);
-  t->perm = keep.get<int>(n);
-  t->rank = keep.get<int>(n);
-  t->leaf_of = keep.get<int>(n);
-  t->pos = keep.get<float4>(n);
-  t->w = keep.get<float>(n);
-  t->nfirst = keep.get<int>(cap);
-  t->ncount = keep.get<int>(cap);
-  t->nglo = keep.get<int4>(cap);
-  t->nghi = keep.get<int4>(cap);
-  t->nT = keep.get<int4>(cap);
-  t->ndepth = keep.get<int>(cap);
-  t->nD = keep.get<unsigned long long>(cap);
-  t->src = keep.get<float4>(ns);
-  t->src_order = keep.get<int>(ns);
-  t->src_leaf = keep.get<int>(ns);
-  t->levels = keep.get<int>(2 * kMaxLevels);
-  t->d_n_nodes = keep.get<int>(1);
-  t->status = keep.get<int>(1);
-  t->d_stats = keep.get<unsigned long long>(8);
-  // scratch
-  unsigned* vals = tmp.get<unsigned>(n);
   const int nmax = n > ns ? n : ns;
+  unsigned *vals, *topo_scan, *svals;
+  unsigned long long* skeys;
   SortScratch SS;
-  SS.k2 = tmp.get<unsigned long long>(nmax);
-  SS.v2 = tmp.get<unsigned>(nmax);
-  SS.work = tmp.get<unsigned>(sort_work_words(nmax));
   TopoArrays TA;
-  TA.up = tmp.get<int>(n);
-  TA.range = tmp.get<int2>(n);
-  TA.bit = tmp.get<unsigned char>(n);
-  TA.depth = tmp.get<unsigned char>(n);
-  TA.place = tmp.get<int>(n);
-  TA.list = tmp.get<int>(n);
-  TA.counts = tmp.get<unsigned>(topo_count_words(n));
-  unsigned* topo_scan = tmp.get<unsigned>(scan_scratch_words((int)topo_count_words(n)));
-  unsigned long long* skeys = tmp.get<unsigned long long>(ns);
-  unsigned* svals = tmp.get<unsigned>(ns);
+  t->mem[0] = allocate(
+      [&](Layout& a) {
+        a.get(t->key, n);
+        a.get(t->perm, n);
+        a.get(t->rank, n);
+        a.get(t->leaf_of, n);
+        a.get(t->pos, n);
+        a.get(t->w, n);
+        a.get(t->nfirst, cap);
+        a.get(t->ncount, cap);
+        a.get(t->nglo, cap);
+        a.get(t->nghi, cap);
+        a.get(t->nT, cap);
+        a.get(t->ndepth, cap);
+        a.get(t->nD, cap);
+        a.get(t->src, ns);
+        a.get(t->src_order, ns);
+        a.get(t->src_leaf, ns);
+        a.get(t->levels, 2 * kMaxLevels);
+        a.get(t->d_stats, 9);  // and the status word
+      },
+      s);
+  void* scratch = allocate(
+      [&](Layout& a) {
+        a.get(vals, n);
+        a.get(SS.k2, nmax);
+        a.get(SS.v2, nmax);
+        a.get(SS.work, sort_work_words(nmax));
+        a.get(TA.up, n);
+        a.get(TA.range, n);
+        a.get(TA.bit, n);
+        a.get(TA.depth, n);
+        a.get(TA.place, n);
+        a.get(TA.list, n);
+        a.get(TA.counts, topo_count_words(n));
+        a.get(topo_scan, scan_scratch_words((int)topo_count_words(n)));
+        a.get(skeys, ns);
+        a.get(svals, ns);
+      },
+      s);
+  void* sums = nullptr;  // the moments, later
 
+  auto release = [&]() {  // the scratch blocks
+    if (scratch) cudaFreeAsync(scratch, s);
+    if (sums) cudaFreeAsync(sums, s);
+    scratch = sums = nullptr;
+  };
   auto fail = [&](int code) {
-    tmp.release();
-    keep.release();
+    release();
+    for (void* p : t->mem)
+      if (p) cudaFreeAsync(p, s);
     cudaStreamSynchronize(s);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
     delete t;
     return code;
   };
-  if (!keep.ok || !tmp.ok) {
-    cudaGetLastError();
-    return fail(TREVR_ERR_OUT_OF_MEMORY);
-  }
-  cudaMemsetAsync(t->status, 0, sizeof(int), s);
-  cudaMemsetAsync(t->d_stats, 0, 8 * sizeof(unsigned long long), s);
+  if (!t->mem[0] || !scratch) return fail(TREVR_ERR_OUT_OF_MEMORY);
+  t->status = reinterpret_cast<int*>(t->d_stats + 8);
+  cudaMemsetAsync(t->d_stats, 0, 9 * sizeof(unsigned long long), s);
 
   Domain32 D;
   for (int d = 0; d < 3; ++d) {
@@ -522,6 +536,28 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   t->max_depth = max_depth;
   for (int l = 0; l < 2 * kMaxLevels; ++l) t->h_levels[l] = levels[l];
 
+  const size_t ncell = (size_t)end_cells;
+  Moments* mom;
+  unsigned* arrived;
+  t->mem[1] = allocate(
+      [&](Layout& a) {
+        a.get(t->nA, ncell);
+        a.get(t->nB, ncell);
+        a.get(t->nS, ncell);
+        a.get(t->nl2, ncell);
+        a.get(t->nR, ncell);
+        a.get(t->nV, 2 * ncell);
+        a.get(t->nW, ncell);
+      },
+      s);
+  sums = allocate(
+      [&](Layout& a) {
+        a.get(mom, ncell);
+        a.get(arrived, ncell);
+      },
+      s);
+  if (!t->mem[1] || !sums) return fail(TREVR_ERR_OUT_OF_MEMORY);
+
   // 3. sources
   if (ns > 0) {
     src_leaf_kernel<<<grid_for(ns, 256), 256, 0, s>>>(src_xyz, src_lum, ns, D, t->nT, t->nglo,
@@ -530,35 +566,15 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
     int bits = 1;  // keys are particle numbers
     while (bits < 31 && ((n - 1) >> bits)) ++bits;
     radix_sort(skeys, svals, ns, bits, SS, t->status, s);
-    gather_sources_kernel<<<grid_for(ns, 256), 256, 0, s>>>(src_xyz, src_lum, ns, n, D, svals, skeys,
-                                                             t->leaf_of, t->src, t->src_order,
-                                                             t->src_leaf);
-    note_launch();
-    node_src_range_kernel<<<grid_for(end_cells - kRoot, 256), 256, 0, s>>>(
-        end_cells, t->nfirst, t->ncount, skeys, ns, t->nT);
+    gather_sources_kernel<<<grid_for(ns, 256), 256, 0, s>>>(src_xyz, src_lum, ns, n, D, svals,
+                                                             skeys, t->leaf_of, t->src,
+                                                             t->src_order, t->src_leaf);
     note_launch();
   }
+  node_src_range_kernel<<<grid_for(end_cells - kRoot, 256), 256, 0, s>>>(
+      end_cells, t->nfirst, t->ncount, skeys, ns, t->nT, arrived);
+  note_launch();
   // 4. moments, bottom-up
-  const size_t ncell = (size_t)end_cells;
-  t->nA = keep.get<float4>(ncell);
-  t->nB = keep.get<float4>(ncell);
-  t->nS = keep.get<float4>(ncell);
-  t->nl2 = keep.get<float>(ncell);
-  t->nR = keep.get<float4>(ncell);
-  t->nV = keep.get<float4>(2 * ncell);
-  t->nW = keep.get<double>(ncell);
-  Moments* mom = tmp.get<Moments>(ncell);
-  unsigned* arrived = tmp.get<unsigned>(ncell);
-  if (!keep.ok || !tmp.ok) {
-    cudaGetLastError();
-    return fail(TREVR_ERR_OUT_OF_MEMORY);
-  }
-  // entry 0: an inert cell (no luminosity)
-  cudaMemsetAsync(t->nA, 0, sizeof(float4), s);
-  cudaMemsetAsync(t->nB, 0, sizeof(float4), s);
-  cudaMemsetAsync(t->nS, 0, sizeof(float4), s);
-  cudaMemsetAsync(t->nl2, 0, sizeof(float), s);
-  cudaMemsetAsync(t->nW, 0, sizeof(double), s);
   MomentArrays MA;
   MA.nT = t->nT;
   MA.nglo = t->nglo;
@@ -587,38 +603,18 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
     moments_level_kernel<<<blocks, 128, 0, s>>>(MA, L);
     note_launch();
   }
-  cudaMemsetAsync(arrived, 0, (size_t)levels[2 * climb + 1] * sizeof(unsigned), s);
   moments_climb_kernel<<<grid_for(levels[2 * climb + 1] - kRoot, 64), 64, 0, s>>>(
       MA, levels[2 * climb], levels[2 * climb + 1], arrived);
   records_kernel<<<grid_for(levels[2 * climb + 1] - kRoot, 128), 128, 0, s>>>(
       MA, levels[2 * climb + 1]);
   note_launch(2);
-  cudaMemcpyAsync(t->d_n_nodes, &levels[2 * max_depth + 1], sizeof(int), cudaMemcpyHostToDevice, s);
-  tmp.release();
-  cudaEventRecord(e1, s);
+  release();
   int status = 0;
   cudaMemcpyAsync(&status, t->status, sizeof(int), cudaMemcpyDeviceToHost, s);
   err = cudaStreamSynchronize(s);
   if (err == cudaSuccess) err = cudaGetLastError();
-  if (err != cudaSuccess) {
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    keep.release();
-    delete t;
-    return cuda_to_error(err);
-  }
-  float ms = 0.0f;
-  cudaEventElapsedTime(&ms, e0, e1);
-  if (build_ms) *build_ms = ms;
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  if (status) {
-    keep.release();
-    cudaStreamSynchronize(s);
-    delete t;
-    return status_to_error(status);
-  }
-  // keep.ptrs is dropped: the tree owns those buffers now
+  if (err != cudaSuccess) return fail(cuda_to_error(err));
+  if (status) return fail(status_to_error(status));
   *out = t;
   return TREVR_OK;
 }

@@ -63,7 +63,6 @@ struct TreeView {
   const float4* src;  // (y.x, y.y, y.z, L)
   const int* src_order;
   const int* src_leaf;  // leaf cell of each sorted source
-  const int* n_nodes;  // device scalar
   // several bands (trevr_build_tree_bands): up to 4 per record, unused slots 0
   int n_bands;         // 0 for a single-band tree
   const float4* bA;    // per cell: mean absorption of each band
@@ -148,9 +147,10 @@ struct trevr_tree {
   int h_levels[2 * trevr::kMaxLevels];  // host copy of the level ranges
   // bookkeeping
   int* levels;    // kMaxLevels x 2 (begin, end)
-  int* d_n_nodes;
   int* status;    // device status word
   unsigned long long* d_stats;  // 4 counters
+  void* mem[2];   // the blocks that hold the arrays of the build: those sized by the particles, and
+                  // those sized by the cells (the bands' and the particle trace's are their own)
   trevr::TreeView view() const;
 };
 
@@ -159,13 +159,12 @@ namespace trevr {
 // ---- build.cu
 int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weight, long long n_gas,
                     const float* src_xyz, const float* src_lum, long long n_src,
-                    const trevr_domain* dom, int bucket, cudaStream_t s, trevr_tree** out,
-                    float* build_ms);
+                    const trevr_domain* dom, int bucket, cudaStream_t s, trevr_tree** out);
 // ---- bands.cu
 int build_tree_bands_impl(const float* gas_xyz, const float* alpha_bands, const float* weight,
                           long long n_gas, const float* src_xyz, const float* lum_bands,
                           long long n_src, int n_bands, const trevr_domain* dom, int bucket,
-                          cudaStream_t s, trevr_tree** out, float* build_ms);
+                          cudaStream_t s, trevr_tree** out);
 
 // ---- sort.cu: stable LSD radix sort of (uint64 key, uint32 value) pairs
 struct SortScratch {
