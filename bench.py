@@ -367,7 +367,7 @@ def _bench_batched(args, sm_mhz):
                         "cells_visited": st["src_nodes_visited"] / n,
                         "cells_clipped": st["cells_clipped"] / n},
            "roofline": _issue_roofline(prof, n, t_rep, sm_mhz, dev_sm, alg_bytes, peak,
-                                       peak_kind, "walk_warp_batched_kernel (persistent, "
+                                       peak_kind, "cut_walk_batched_kernel (persistent, "
                                        "graph replay)")}
     if prof is not None:
         res["roofline"]["captured_launch_shape"] = prof.get("launch_shape")
@@ -698,7 +698,7 @@ def run_ours(args):
     prof = (_kernel_profile("walk_warp_kernel_issue.json")
             if shape["walk_variant"] in (0, 3) else None)
     roofline = _issue_roofline(prof, n, t_walk, sm_mhz, n_sm, alg_bytes, peak, peak_kind,
-                               "walk_warp_kernel, variant 3 (warp-shared walk, merged rays, "
+                               "cut_walk_kernel, variant 3 (warp-shared walk, merged rays, "
                                "flux, no counters)")
 
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world,
@@ -749,7 +749,7 @@ def run_profile(args):
     """A short program for ncu: one tree build, then on a contiguous Morton-ordered run
     of --sink-sample sinks the walk with counters (launch 0, whose counters are
     printed) and the walk the benchmark times, without counters (launch 1, the one
-    to capture: -k regex:walk_warp_kernel -s 1 -c 1)."""
+    to capture: -k regex:cut_walk_kernel -s 1 -c 1)."""
     import torch
     from paper_1902_08083_gb300 import trevr
     torch.cuda.set_device(0)
@@ -779,7 +779,7 @@ def run_profile_sub(args):
     """A short program for ncu on the sub-bucket walk: the 2^18-particle sub-bucket
     workload, its neighbour lists, one walk with counters (launch 0, counters
     printed) and one without (launch 1, the one to capture:
-    -k regex:walk_warp_kernel -s 1 -c 1)."""
+    -k regex:cut_walk_kernel -s 1 -c 1)."""
     import torch
     from paper_1902_08083_gb300 import trevr
     torch.cuda.set_device(0)
@@ -805,7 +805,7 @@ def run_profile_sub(args):
 def run_profile_batched(args):
     """A short program for ncu on the batched walk: the 64 boxes, the autotuned launch
     shape, one batched call with counters (launch 0, counters printed) and one without
-    (launch 1, the one to capture: -k regex:walk_warp_batched_kernel -s 1 -c 1)."""
+    (launch 1, the one to capture: -k regex:cut_walk_batched_kernel -s 1 -c 1)."""
     import torch
     from paper_1902_08083_gb300 import autotune, trevr
     torch.cuda.set_device(0)

@@ -117,7 +117,8 @@ typedef struct {
     long long segments;          /* ray segments summed (cells whose mean absorption was used) */
     long long src_nodes_visited; /* source-tree cells tested against the opening angle */
     long long refine_expansions; /* cells replaced by their two children (Eq. refcrit) */
-    long long cells_clipped;     /* ray/cell intersection tests (every cell record a ray read) */
+    long long cells_clipped;     /* cells that a ray is cut with: its base cells, and the
+                                    children that it crosses of the cells it refines */
     float build_ms;
     float walk_ms;
     long long rays_terminated;   /* rays cut off by tau_stop (of the interactions) */
@@ -156,12 +157,14 @@ int trevr_build_tree(const float* gas_xyz, const float* alpha, const float* weig
 /*
  * Flux at the sinks (Eq. simpint summed over the pseudo-sources of the
  * opening-angle walk, Sec. 2.2.1-2.2.3), in fp32. Each sink's flux is a
- * compensated sum. The warp-shared walks (variants 2 and 3) sum a ray's optical
- * depth plainly, and the per-lane walk (variant 1) sums it with compensation.
+ * compensated sum, and so is a ray's optical depth.
  *
  *   t         tree from trevr_build_tree.
  *   sink_idx  n_sink int64 caller indices of gas particles, or NULL = all
  *             gas particles in the caller's order (then n_sink must be n_gas).
+ *             They are walked in Morton order, whatever their own: the call
+ *             sorts them in stream-ordered memory (24 bytes a sink), except
+ *             while the stream is being captured.
  *   prm       host pointer: theta_open, tau_ref, tuning fields.
  *   flux_out  n_sink floats: flux_out[k] is the flux at sink k.
  *   sink_counters  NULL, or 4*n_sink int32: per sink the number of rays,

@@ -116,8 +116,9 @@ __device__ __forceinline__ float kint_phi(const float4* __restrict__ tab, float 
 // listed for its leaf, the receiving particle (sorted index si) left out. The 32
 // lanes of the warp test one neighbour each per round, with the next round's
 // entries already loading; the neighbours that reach the chord are queued in shared
-// memory, as (x, sigma_0, sigma_1, alpha w / (pi h^2)), and integrated 32 at a time: (Phi(x, sigma_1) - Phi(x, sigma_0)) times
-// alpha w / (pi h^2), with x = b^2 / h^2 and sigma = s / h. Every lane must call it;
+// memory, as (x, sigma_0, sigma_1, alpha w / (pi h^2)), and integrated 32 at a time:
+// (Phi(x, sigma_1) - Phi(x, sigma_0)) times alpha w / (pi h^2), with x = b^2 / h^2 and
+// sigma = s / h. Every lane must call it;
 // all lanes return the sum.
 __device__ __forceinline__ float sub_bucket_tau_warp(const TreeView& T, int src, int box, int si,
                                                      float px, float py, float pz, float dx,
@@ -601,7 +602,8 @@ __device__ __forceinline__ void cut_ray(const TreeView& T, const WalkParams& P, 
           const int src = __ffs(m) - 1;
           m &= m - 1u;
           const float t = sub_bucket_tau_warp(T, src, sub_box, K.i, ray.px, ray.py, ray.pz, ray.dx,
-                                              ray.dy, ray.dz, ray.s2, ray.len, sub_t0, sub_t1, queue);
+                                              ray.dy, ray.dz, ray.s2, ray.len, sub_t0, sub_t1,
+                                              queue);
           if ((int)(threadIdx.x & 31u) == src) tau.add(t);
         }
       }
@@ -802,16 +804,17 @@ __device__ __forceinline__ void cut_walk(const TreeView& T, const WalkParams& P,
   }
 }
 
-// Issue-bound: the loop over a ray's pieces is ~50 instructions on one 16-byte record that
-// L1 mostly has, and what bounds the walk is how many of them it runs. Clipping every base
-// cell and refined child instead (~120 instructions on 44 bytes, 53 a ray where 35 are
-// crossed) took 118.4 ms a step at 2^22 sinks and 2^14 clumped sources; the cut pieces take
-// 56.7 ms (21.4 and 8.3 ms at 100003 sinks, tau_ref = 0.01).
-// Blocks of 128 per SM: 8 leave the plain walk its registers (61, no spills); 12 and 16 (40
-// and 32 registers) gave 58.9 and 55.9 ms at 2^22 but 9.5 and 10.1 ms at 100003 sinks, where
-// a warp's own speed counts and 8 took 8.4. The particle trace needs 4 or 5 (57.2 ms at 2^16
-// sinks, against 66.9 at 6 and 72.4 at 8), the bands 6 (8.95 ms for three at 200003 sinks,
-// 9.2 at 8).
+// Issue-bound where a call fills the GPU (86% of the issue slots at 2^20 sinks): the loop over
+// a ray's pieces is ~60 instructions on one 16-byte record that L1 mostly has, and what bounds
+// the walk is how many of them it runs. Clipping every base cell and refined child instead
+// (~120 instructions on 44 bytes, 53 a ray where 35 are crossed) took 118.4 ms a step at 2^22
+// sinks and 2^14 clumped sources; the cut pieces took 56.7 ms and take 53.2 now (21.4, 8.3 and
+// 7.1 ms at 100003 sinks, tau_ref = 0.01).
+// Blocks of 128 per SM: 8 leave the plain walk its registers (56, no spills); 12 and 16 (40
+// and 32 registers) gave 58.9 and 55.9 ms against 57.3 at 2^22, but 9.5 and 10.1 against 8.4 ms
+// at 100003 sinks, where a warp's own speed counts. The particle trace waits for L2 and wants
+// warps: 5 blocks (94 registers) take 38.9 ms at 2^16 sinks, 4 take 44.0 and 6, which spill,
+// 43.4. The bands take 6 (8.95 ms for three at 200003 sinks, 9.2 at 8).
 constexpr int cut_blocks(bool SUB, int NB) { return SUB ? 5 : NB > 1 ? 6 : 8; }
 // warps per group at most: the particle trace keeps 5 blocks of 4
 constexpr int most_warps(bool SUB) { return SUB ? 4 : kSlots; }
@@ -952,7 +955,7 @@ __global__ void __launch_bounds__(BS, 1024 / BS) cut_walk_batched_kernel(
 }
 
 // The adjoint walk; a sink with dLoss/dF = 0 is left out. Flux and gradients of 2^20 sinks
-// and 1024 sources take 59.9 ms (119 when each cell was clipped and its bounding planes
+// and 1024 sources take 58.2 ms (121 when each cell was clipped and its bounding planes
 // tracked), 25 of them the flux; 4 to 10 blocks per SM lie within 9%, 8 is the fastest.
 template <bool SHARED, bool MERGE>
 __global__ void __launch_bounds__(SHARED ? 32 * kSlots : 128, SHARED ? 4 : 8)
@@ -993,7 +996,8 @@ int group_warps(int n_sink, int most) {
 // took 9.9 ms for 100003 sinks instead of 7.3, since what they hold is taken from L1.
 template <bool SUB>
 size_t block_bytes(int w) {
-  const size_t stacks = (w > 1 ? w : 4) * sizeof(CutStack<SUB>), sums = kSlots * 32 * sizeof(float2);
+  const size_t stacks = (w > 1 ? w : 4) * sizeof(CutStack<SUB>);
+  const size_t sums = kSlots * 32 * sizeof(float2);
   return w > 1 && stacks < sums ? sums : stacks;
 }
 
@@ -1001,7 +1005,8 @@ template <bool MERGE, bool MOM, bool BG, bool STOP, int NB, bool SUB, bool TD>
 cudaError_t launch(const TreeView& T, const long long* sink_idx, int n_sink, const WalkParams& wp,
                    const SinkOut& out, unsigned long long* stats, int* status, cudaStream_t s) {
   const int w = group_warps(n_sink, most_warps(SUB));
-  const int grid = w > 1 ? (n_sink + 31) / 32 : (n_sink + 127) / 128, threads = w > 1 ? 32 * w : 128;
+  const int grid = w > 1 ? (n_sink + 31) / 32 : (n_sink + 127) / 128;
+  const int threads = w > 1 ? 32 * w : 128;
   auto go = [&](auto kernel, unsigned long long* st) {
     kernel<<<grid, threads, block_bytes<SUB>(w), s>>>(T, sink_idx, n_sink, wp, out, st, status);
   };
@@ -1062,7 +1067,8 @@ cudaError_t launch_cut_adjoint(const TreeView& T, const long long* sink_idx, int
                                const WalkParams& wp, const AdjointArgs& J, int* status,
                                cudaStream_t s) {
   const int w = group_warps(n_sink, kSlots);
-  const int grid = w > 1 ? (n_sink + 31) / 32 : (n_sink + 127) / 128, threads = w > 1 ? 32 * w : 128;
+  const int grid = w > 1 ? (n_sink + 31) / 32 : (n_sink + 127) / 128;
+  const int threads = w > 1 ? 32 * w : 128;
   auto go = [&](auto kernel) {
     kernel<<<grid, threads, block_bytes<false>(w), s>>>(T, sink_idx, n_sink, wp, status, J);
   };

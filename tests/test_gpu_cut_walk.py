@@ -101,3 +101,25 @@ def test_stack_limit_counts_dark_cells():
         trevr.compute_flux(G, 0.1, 0.1, stats=True, stack_depth=2)
     assert ei.value.code == 3
     trevr.compute_flux(G, 0.1, 0.1, stats=True)
+
+
+def test_gradient_of_rays_with_more_segments_than_are_kept():
+    # buckets of one and full refinement: rays across the box have some 80 segments, more
+    # than the 64 that are kept for the replay, and are traced a second time; the per-lane
+    # walk traces every ray twice. Both sum fp32 terms in FP64 and other orders: d(tau)/dq
+    # is a sum of ~100 terms of both signs, 100 * 2^-24 = 6e-6 of its largest.
+    import torch
+    from paper_1902_08083_gb300 import trevr
+    P = workloads.uniform_box(n_gas=60000, n_src=8, seed=17, bucket=1)
+    P["alpha"] = np.random.default_rng(18).lognormal(0.0, 1.0, 60000).astype(np.float32)
+    G = gpu_tree(P)
+    sinks = torch.arange(0, 60000, 29, device="cuda")
+    g = torch.from_numpy(np.random.default_rng(19).standard_normal(sinks.shape[0])
+                         .astype(np.float32)).cuda()
+    _, c = trevr.compute_flux(G, 0.75, 0.0, sink_idx=sinks, counters=True)
+    assert int((c[:, 1] / c[:, 0].clamp(min=1)).max()) > 64
+    want = trevr.compute_flux_backward(G, g, 0.75, 0.0, sink_idx=sinks, walk_variant=1)
+    got = trevr.compute_flux_backward(G, g, 0.75, 0.0, sink_idx=sinks)
+    for a, b in zip(got, want):
+        assert float((a - b).norm() / b.norm()) < 2e-5
+        assert float((a - b).abs().max() / b.abs().max()) < 2e-5
