@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <cstring>
 
 #include "morton.cuh"
@@ -454,7 +455,8 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
         a.get(vals, n);
         a.get(SS.k2, nmax);
         a.get(SS.v2, nmax);
-        a.get(SS.work, sort_work_words(nmax));
+        // (not monotone: a smaller sort may have more tiles)
+        a.get(SS.work, std::max(sort_work_words(n), sort_work_words(ns)));
         a.get(TA.up, n);
         a.get(TA.range, n);
         a.get(TA.bit, n);

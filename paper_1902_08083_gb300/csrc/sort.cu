@@ -4,10 +4,10 @@
 // The sort takes 8-bit digits from the least significant. Up to kSmallSort pairs are sorted by
 // one block in one launch, the pairs in registers and shared memory throughout. Larger inputs
 // take one launch that counts every digit of every pass, and one launch per pass: a tile of
-// 4096 pairs is ranked in shared memory, its digit counts are added up over the tiles before
-// it by decoupled look-back (Merrill & Garland's single-pass scan, as Adinets & Merrill's
-// one-sweep sort uses it), and its pairs are written in runs of equal digits. So a pass reads
-// and writes each pair once (24 bytes) and nothing is counted twice.
+// 2048 or 4096 pairs is ranked in shared memory, its digit counts are added up over the tiles
+// before it by decoupled look-back (Merrill & Garland's single-pass scan, as Adinets &
+// Merrill's one-sweep sort uses it), and its pairs are written in runs of equal digits. So a
+// pass reads and writes each pair once (24 bytes) and nothing is counted twice.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -229,17 +229,18 @@ __global__ void __launch_bounds__(256) digit_count_kernel(const unsigned long lo
   }
 }
 
-// One pass: a tile of kSortTile pairs per block, in the order of the blocks' tickets, so that
+// One pass: a tile of 256 ITEMS pairs per block, in the order of the blocks' tickets, so that
 // the tiles before it are done or running. tiles_now holds this pass's words (zero at the
 // start), tiles_next is cleared for the next pass.
-__global__ void __launch_bounds__(kSortThreads, 2) sort_pass_kernel(
+template <int ITEMS>
+__global__ void __launch_bounds__(kSortThreads, ITEMS > 8 ? 2 : 3) sort_pass_kernel(
     const unsigned long long* __restrict__ kin, const unsigned* __restrict__ vin,
     unsigned long long* __restrict__ kout, unsigned* __restrict__ vout, int n, int shift,
     const unsigned* __restrict__ counts, unsigned* ticket, unsigned* tiles_now,
     unsigned* __restrict__ tiles_next, int* status) {
-  constexpr int kWarps = kSortThreads / 32;
+  constexpr int kWarps = kSortThreads / 32, kTile = kSortThreads * ITEMS;
   static_assert(kSortThreads == 256, "one thread per digit");
-  __shared__ unsigned long long stage[kSortTile];
+  __shared__ unsigned long long stage[kTile];
   __shared__ unsigned count[kWarps][256];
   __shared__ unsigned start[256];   // first place of a digit in the tile
   __shared__ unsigned target[256];  // its first place in the output, less start
@@ -253,13 +254,13 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_pass_kernel(
   for (int i = lane; i < 256; i += 32) count[warp][i] = 0;
   __syncthreads();
   const int tile = s_tile;
-  const int base = tile * kSortTile, here = min(kSortTile, n - base);
+  const int base = tile * kTile, here = min(kTile, n - base);
   tiles_next[(size_t)tile * 256 + d] = 0;
-  const int own = warp * 32 * kSortItems + lane;
-  unsigned long long key[kSortItems];
-  unsigned rank[kSortItems];
+  const int own = warp * 32 * ITEMS + lane;
+  unsigned long long key[ITEMS];
+  unsigned rank[ITEMS];
 #pragma unroll
-  for (int r = 0; r < kSortItems; ++r) {
+  for (int r = 0; r < ITEMS; ++r) {
     const int i = own + 32 * r;
     key[r] = i < here ? kin[base + i] : ~0ull;  // behind every pair of the tile
   }
@@ -273,7 +274,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_pass_kernel(
     total += c;
   }
   const unsigned off = block_exclusive_scan(total, smem, &all);
-  if (d == 255) total -= (unsigned)(kSortTile - here);  // the filling is not counted
+  if (d == 255) total -= (unsigned)(kTile - here);  // the filling is not counted
   volatile unsigned* words = tiles_now;
   unsigned before = 0;
   if (tile == 0) {
@@ -316,41 +317,46 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_pass_kernel(
     return;
   }
 #pragma unroll
-  for (int r = 0; r < kSortItems; ++r) {
+  for (int r = 0; r < ITEMS; ++r) {
     const unsigned g = digit_of(key[r], shift);
     rank[r] += start[g] + count[warp][g];
     stage[rank[r]] = key[r];
   }
   __syncthreads();
-  unsigned to[kSortItems];
+  unsigned to[ITEMS];
 #pragma unroll
-  for (int r = 0; r < kSortItems; ++r) {
+  for (int r = 0; r < ITEMS; ++r) {
     const int j = threadIdx.x + kSortThreads * r;
     const unsigned long long k = stage[j];
     to[r] = j < here ? target[digit_of(k, shift)] + (unsigned)j : ~0u;
     if (to[r] < (unsigned)n) kout[to[r]] = k;
   }
-  unsigned val[kSortItems];
+  unsigned val[ITEMS];
 #pragma unroll
-  for (int r = 0; r < kSortItems; ++r) {
+  for (int r = 0; r < ITEMS; ++r) {
     const int i = own + 32 * r;
     val[r] = i < here ? vin[base + i] : 0u;
   }
   __syncthreads();
   unsigned* vals = reinterpret_cast<unsigned*>(stage);
 #pragma unroll
-  for (int r = 0; r < kSortItems; ++r) vals[rank[r]] = val[r];
+  for (int r = 0; r < ITEMS; ++r) vals[rank[r]] = val[r];
   __syncthreads();
 #pragma unroll
-  for (int r = 0; r < kSortItems; ++r)
+  for (int r = 0; r < ITEMS; ++r)
     if (to[r] < (unsigned)n) vout[to[r]] = vals[threadIdx.x + kSortThreads * r];
 }
 
 }  // namespace
 
+// Pairs per tile: half the tile halves a block's ranking, and twice the tiles lengthen the
+// look-back. 2048 / 4096 pairs take 97 / 112 us for 5000 keys of 63 bits, 131 / 147 for 2^18,
+// 238 / 204 for 2^20 (the whole call of the allocation-free sort).
+static int sort_tile(int n) { return n <= (1 << 18) ? kSortTile / 2 : kSortTile; }
+
 size_t sort_work_words(int n) {
   if (n <= kSmallSort) return 1;
-  return (size_t)kSortHead + 2 * 256 * (size_t)((n + kSortTile - 1) / kSortTile);
+  return (size_t)kSortHead + 2 * 256 * (size_t)((n + sort_tile(n) - 1) / sort_tile(n));
 }
 
 void radix_sort(unsigned long long* k, unsigned* v, int n, int bits, const SortScratch& S,
@@ -362,7 +368,7 @@ void radix_sort(unsigned long long* k, unsigned* v, int n, int bits, const SortS
     note_launch();
     return;
   }
-  const int tiles = (n + kSortTile - 1) / kSortTile;
+  const int tile = sort_tile(n), tiles = (n + tile - 1) / tile;
   unsigned *counts = S.work, *tickets = S.work + 8 * 256;
   unsigned* words[2] = {S.work + kSortHead, S.work + kSortHead + 256 * (size_t)tiles};
   cudaMemsetAsync(S.work, 0, ((size_t)kSortHead + 256 * (size_t)tiles) * sizeof(unsigned), s);
@@ -372,9 +378,10 @@ void radix_sort(unsigned long long* k, unsigned* v, int n, int bits, const SortS
   unsigned long long *ka = k, *kb = S.k2;
   unsigned *va = v, *vb = S.v2;
   for (int p = 0; p < passes; ++p) {
-    sort_pass_kernel<<<tiles, kSortThreads, 0, s>>>(ka, va, kb, vb, n, 8 * p, counts + 256 * p,
-                                                    tickets + p, words[p & 1], words[(p & 1) ^ 1],
-                                                    status);
+    const auto pass = tile == kSortTile ? sort_pass_kernel<kSortItems>
+                                        : sort_pass_kernel<kSortItems / 2>;
+    pass<<<tiles, kSortThreads, 0, s>>>(ka, va, kb, vb, n, 8 * p, counts + 256 * p, tickets + p,
+                                        words[p & 1], words[(p & 1) ^ 1], status);
     note_launch();
     unsigned long long* tk = ka;
     ka = kb;

@@ -1,6 +1,6 @@
-"""The radix sort at the edges of its forms: one block up to 4096 pairs, tiles of 4096 with
-look-back beyond, full and ragged last tiles; keys all different, all equal, few, and clustered
-(equal high digits). Keys and order must equal a stable sort's exactly. And the walk order of
+"""The radix sort at the edges of its forms: one block up to 4096 pairs, tiles of 2048 with
+look-back beyond, of 4096 from 2^18 on, full and ragged last tiles; keys all different, all
+equal, few, and clustered (equal high digits). Keys and order must equal a stable sort's exactly. And the walk order of
 a sink list: any order and repetition of the caller's indices gives each sink's own result."""
 import numpy as np
 import pytest
@@ -26,7 +26,7 @@ def _points(kind, n):
 
 
 @pytest.mark.parametrize("kind", ["uniform", "equal", "few", "clustered"])
-@pytest.mark.parametrize("n", [1, 2, 31, 33, 256, 4095, 4096, 4097, 8192, 12289, 1 << 20])
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 256, 4095, 4096, 4097, 8192, 12289, 1 << 18, (1 << 18) + 1, 1 << 20])
 def test_keys_and_order_are_the_stable_sorts(n, kind):
     import torch
     from paper_1902_08083_gb300 import trevr
@@ -72,3 +72,19 @@ def test_sink_lists_in_any_order(m, n_src):
         keep = torch.arange(m, device="cuda") != m // 2
         np.testing.assert_allclose(out[keep].cpu().numpy(), full[idx[keep]].cpu().numpy(),
                                    rtol=1e-6)
+
+
+def test_sources_that_need_more_tiles_than_the_particles():
+    # 2^18 + 1 particles sort in 65 tiles, 2^18 sources in 128: the scratch holds either
+    from paper_1902_08083_gb300 import trevr
+    import torch
+    rng = np.random.default_rng(4)
+    n, s = (1 << 18) + 1, 1 << 18
+    gas = torch.from_numpy(_points("uniform", n)).cuda()
+    src = torch.from_numpy(_points("uniform", s)).cuda()
+    lum = torch.from_numpy(rng.random(s).astype(np.float32)).cuda()
+    tree = trevr.build_tree(gas, torch.ones(n, device="cuda"), src, lum)
+    order = tree.export()["src_order"].long()
+    assert torch.equal(order.sort().values, torch.arange(s, device="cuda"))
+    first = tree.export()["src_first"].long(), tree.export()["src_count"].long()
+    assert int(first[1][1]) == s  # the root holds them all
