@@ -111,7 +111,10 @@ typedef struct {
                            (walk_variant 3). */
 } trevr_params;
 
-/* Totals over the sinks of one call, and timings (ms, CUDA events). */
+/* Totals over the sinks of one call, and timings (ms, CUDA events). They are counted by the
+   walk that the call without them runs, and asking for them does not change the flux. A ray
+   is walked from the sink to the source: of one that tau_stop cuts off, segments and
+   refine_expansions count what came before that, cells_clipped all of its base cells. */
 typedef struct {
     long long interactions;      /* rays traced: accepted cells plus single sources */
     long long segments;          /* ray segments summed (cells whose mean absorption was used) */

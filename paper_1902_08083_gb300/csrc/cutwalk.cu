@@ -364,7 +364,8 @@ __device__ __forceinline__ void add_segments(double* G, const int2* seg, int n, 
 // One ray per lane that is `on`, from its sink to `ent` (a cell, or ~source); every lane of
 // the warp must call it. The loop ends: a refined piece goes on at a child, whose number is
 // larger than its parent's, and every entry of the list is taken once.
-// STOP: a ray whose running optical depth passes P.tau_stop ends and adds nothing (Sec. 4).
+// STOP: a ray whose running optical depth passes P.tau_stop ends and adds nothing (Sec. 4);
+// its segments and refinements are counted up to there.
 // NB > 1: every band sums its own optical depth over the shared segments.
 // SUB: a leaf whose own particles ask for refinement is integrated through them.
 // TD: the top-down ray walk: A is the only piece, and Eq. refcrit alone splits it.

@@ -18,21 +18,13 @@
 // on its offset from the origin.
 //
 // GPU form (sinks in Morton order, so the lanes of a warp are neighbours in space). This
-// file has the walks that clip every cell of a ray by itself:
-//   * Variant 1 (walk_kernel): one lane per sink, a flat loop in which one iteration is a
-//     walk step or a cell clip, cells picked with selects from one per-lane list; a lane
-//     that finishes takes the next sink of its warp's chunk.
-//   * walk_warp_kernel: the flux with early ray termination when counters are asked for
-//     (the segments of a ray that is cut off are counted in this walk's order). The 32 lanes
-//     walk one shared stack with a mask of the lanes that still need each cell; a lane keeps
-//     its next ray pending, and the pending rays of all lanes (to different cells) are traced
-//     together.
-// Everything else of variants 2 and 3 is in cutwalk.cu.
-//   * The segment cells of a ray are known without following parent links: the sibling of a
-//     cell is its index XOR 1 (children are allocated in pairs) and the common ancestor's
-//     depth is the length of the common prefix of the sink's ancestor list and the walk
-//     path, kept as a 64-bit mask. Refined children are clipped after the ray's base
-//     segments.
+// file has variant 1 (walk_kernel), which clips every cell of a ray by itself: one lane per
+// sink, a flat loop in which one iteration is a walk step or a cell clip, cells picked with
+// selects from one per-lane list; a lane that finishes takes the next sink of its warp's
+// chunk. The segment cells of a ray are known without following parent links: the sibling of
+// a cell is its index XOR 1 (children are allocated in pairs) and the common ancestor's depth
+// is the length of the common prefix of the sink's ancestor list and the walk path, kept as a
+// 64-bit mask. Variants 2 and 3 are in cutwalk.cu.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -46,9 +38,6 @@ namespace {
 constexpr int kAnc = 0;     // offsets of the three parts of the per-lane list
 constexpr int kPath = kDepth;
 constexpr int kRef = 2 * kDepth;
-// refinement stack of the warp walk: refined base segments (at most 2 x 63 + 1) are
-// queued first, then each popped pair adds at most one entry per level below
-constexpr int kRayStack = 4 * kDepth;
 
 // one slab of the clip: (lo - p) * (1/d), (hi - p) * (1/d), rounded after each step;
 // along an axis the ray does not move on, the box is half-open [lo, hi), so a ray
@@ -63,15 +52,6 @@ __device__ __forceinline__ void slab(float lo, float hi, float p, float d, float
   } else {
     miss = miss || p < lo || p >= hi;
   }
-}
-
-// the slab of an axis the ray moves along (d != 0): the same steps as slab()
-__device__ __forceinline__ void slab_nz(float lo, float hi, float p, float inv, float& t0,
-                                        float& t1) {
-  const float ta = __fmul_rn(__fsub_rn(lo, p), inv);
-  const float tb = __fmul_rn(__fsub_rn(hi, p), inv);
-  t0 = fmaxf(t0, fminf(ta, tb));
-  t1 = fminf(t1, fmaxf(ta, tb));
 }
 
 // gradient-carrying slab: remembers which axis sets t0 / t1
@@ -476,404 +456,6 @@ __global__ void __launch_bounds__(BS) walk_batched_kernel(const TreeView* __rest
   if (stats) add_stats(tot, stats);
 }
 
-// ---------------------------------------------------------------------------
-// Warp-shared walk (variant 2). The 32 lanes of a warp (32 consecutive sinks in
-// Morton order) walk ONE depth-first stack held in shared memory; each entry
-// carries the mask of lanes that still need the cell. A cell that several
-// lanes accept is traced by all of them at once, to the same pseudo-source, so
-// the cells on the pseudo-source's side and the shared part of the sinks' side
-// are the same addresses in every lane (one broadcast load). The segment order
-// is chosen for that: C, then C's side from deep to shallow, then the sink's
-// side from shallow to deep, then S.
-// ---------------------------------------------------------------------------
-struct WarpStack {
-  int node[kDepth + 2];
-  int depth[kDepth + 2];
-  unsigned mask[kDepth + 2];
-  int path[kDepth];  // the walk's depth-first path
-};
-
-// Rays from the sinks of the lanes in `on` to (q, L) inside cell C; every lane
-// of the warp must call it (the loop runs while any lane has cells left).
-// Early ray termination (Sec. 4): a lane whose running optical depth passes P.tau_stop
-// drops the rest of its ray, and the ray adds nothing.
-__device__ __forceinline__ void warp_ray(const TreeView& T, const WalkParams& P, const bool on,
-                                         const float px, const float py, const float pz,
-                                         const int S, const int dS, const int* anc, int* rst,
-                                         const unsigned long long on_path, const int* path,
-                                         const int C, const int dC, const float qx,
-                                         const float qy, const float qz, const float L,
-                                         const int box_limit, int* status, SinkCounters& cnt,
-                                         CSum& F) {
-  const unsigned FULL = 0xffffffffu;
-  float dx = 0.0f, dy = 0.0f, dz = 0.0f, s2 = 1.0f, len = 1.0f, ix = 0.0f, iy = 0.0f, iz = 0.0f;
-  int nCs = 0, nSs = 0, nb = 0, dstar = 0;
-  bool active = false;
-  if (on) {
-    dx = __fsub_rn(qx, px);
-    dy = __fsub_rn(qy, py);
-    dz = __fsub_rn(qz, pz);
-    s2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-    if (!(s2 < P.smin2)) {  // a source on top of the sink adds nothing
-      active = true;
-      len = __fsqrt_rn(s2);
-      ix = dx != 0.0f ? __frcp_rn(dx) : 0.0f;
-      iy = dy != 0.0f ? __frcp_rn(dy) : 0.0f;
-      iz = dz != 0.0f ? __frcp_rn(dz) : 0.0f;
-      if (C == S) {
-        nb = 1;
-      } else {
-        const int mn = dC < dS ? dC : dS;
-        const unsigned long long m = on_path & ((2ull << mn) - 1ull);  // mn <= 62
-        dstar = __ffsll((long long)~m) - 2;
-        nCs = dC - dstar - 1;
-        nSs = dS - dstar - 1;
-        nb = nCs + nSs + 2;
-      }
-    }
-  }
-  const bool nz = dx != 0.0f && dy != 0.0f && dz != 0.0f;  // the ray moves along every axis
-  KSum tau;
-  bool cut = false;
-  int b = 0, rsp = 0, boxes = 0;
-  int slot = -1;  // the upper child of the pair popped last: clipped next
-  while (__any_sync(FULL, active)) {
-    if (active) {
-      const bool from_stack = b >= nb && (rsp > 0 || slot >= 0);  // base segments first
-      if (!from_stack && b >= nb) {
-        if (cut) ++cnt.cut;
-        else F.add(L * expf(-tau.get()) / (kFourPi * s2));
-        ++cnt.rays;
-        active = false;
-      } else {
-        int box;
-        if (from_stack) {
-          if (slot >= 0) {
-            box = slot;
-            slot = -1;
-          } else {
-            // a refined cell's pair of children (clip the lower, keep the upper), or
-            // the one child the ray crosses
-            const int e = rst[--rsp];
-            if (e < 0) {
-              box = ~e;
-              slot = box + 1;
-            } else {
-              box = e;
-            }
-          }
-        } else {
-          if (nb == 1) {
-            box = S;
-          } else if (b <= nCs) {  // C = path[dC], then the siblings up C's path
-            box = path[dC - max(b - 1, 0)] ^ (b > 0 ? 1 : 0);
-          } else {  // the siblings down S's path, then S = anc[dS]
-            const int j = b - nCs;
-            box = anc[dstar + 1 + min(j, nSs)] ^ (j <= nSs ? 1 : 0);
-          }
-          ++b;
-        }
-        // Each iteration clips one base segment or one child of a pushed pair, and the
-        // pushes are capped by box_limit below, so a ray ends after at most
-        // nb + 2 box_limit iterations (the walk's hang guard).
-        {
-          const float4 a = __ldg(&T.nA[box]);
-          const float4 bb = __ldg(&T.nB[box]);
-          float t0 = 0.0f, t1 = 1.0f;
-          bool miss = false;
-          if (nz) {  // no axis along which the ray stays still: no face tests
-            slab_nz(a.x, bb.x, px, ix, t0, t1);
-            slab_nz(a.y, bb.y, py, iy, t0, t1);
-            slab_nz(a.z, bb.z, pz, iz, t0, t1);
-          } else {
-            slab(a.x, bb.x, px, dx, ix, t0, t1, miss);
-            slab(a.y, bb.y, py, dy, iy, t0, t1, miss);
-            slab(a.z, bb.z, pz, dz, iz, t0, t1, miss);
-          }
-          const float l = (!miss && t1 > t0) ? __fmul_rn(__fsub_rn(t1, t0), len) : 0.0f;
-          ++cnt.clip;
-          if (l > 0.0f) {
-            bool pushed = false;
-            if (P.tau_ref <= 0.0f || __fmul_rn(bb.w, l) > P.tau_ref) {
-              const int child = __ldg(&T.nT[box].x);
-              if (child >= 0) {
-                if (rsp + 1 > kRayStack) {
-                  atomicOr(status, kStatusStackOverflow);
-                  active = false;
-                } else if (++boxes > box_limit) {
-                  atomicOr(status, kStatusIterationLimit);
-                  active = false;
-                } else {
-                  ++cnt.ref;
-                  // The children's intervals are this cell's cut at the split plane,
-                  // whose t is the one their clips would compute ((P - p) * (1/d),
-                  // with min / max exact), so a child the ray misses is not queued
-                  // (22 % fewer clips on the clumpy workload, bit-identical fluxes).
-                  bool lo_t = true, hi_t = true;
-                  {
-                    const float4 r = __ldg(&T.nR[box]);
-                    const int ax = (int)(__float_as_uint(r.w) & 3u);
-                    const float Pl = r.z;
-                    const float pa = ax == 0 ? px : (ax == 1 ? py : pz);
-                    const float ia = ax == 0 ? ix : (ax == 1 ? iy : iz);
-                    if (ia != 0.0f) {
-                      const float tP = __fmul_rn(__fsub_rn(Pl, pa), ia);
-                      const bool fwd = ia > 0.0f;
-                      lo_t = fwd ? tP > t0 : tP < t1;
-                      hi_t = fwd ? tP < t1 : tP > t0;
-                    } else {  // the ray lies in a plane of this axis: half-open children
-                      lo_t = pa < Pl;
-                      hi_t = !lo_t;
-                    }
-                  }
-                  // both children, clipped after the base segments, or the crossed one
-                  rst[rsp++] = lo_t && hi_t ? ~child : (lo_t ? child : child + 1);
-                }
-                pushed = true;
-              }
-            }
-            if (!pushed) {
-              tau.add(__fmul_rn(a.w, l));
-              if (tau.get() > P.tau_stop) {
-                cut = true;  // the rest of the ray is not traced
-                b = nb;
-                rsp = 0;
-                slot = -1;
-              }
-              ++cnt.segs;
-            }
-          }
-        }
-      }
-    }
-  }
-}
-
-// Background sources (Sec. 2.2.4): the centre of luminosity c (s.xyz) of an accepted
-// cell moved radially onto the sphere of radius P.bg_radius around the domain centre
-// o (side / 2 in coordinates relative to the lower corner), in fp32 as d = c - o,
-// s = sqrt((dx^2 + dy^2) + dz^2), q = o + d * (R / s); and the leaf Y holding q (grid
-// coordinates clamped to the grid), found by descending the cut planes from the root,
-// with its ancestors cpath[0 .. dY].
-__device__ __forceinline__ void bg_move(const TreeView& T, const WalkParams& P, const float4 s,
-                                        float& qx, float& qy, float& qz, int& Y, int& dY,
-                                        int* cpath) {
-  const float ox = __fmul_rn(T.side, 0.5f), oy = ox, oz = ox;
-  const float ddx = __fsub_rn(s.x, ox), ddy = __fsub_rn(s.y, oy), ddz = __fsub_rn(s.z, oz);
-  const float sn = __fsqrt_rn(__fadd_rn(__fadd_rn(__fmul_rn(ddx, ddx), __fmul_rn(ddy, ddy)),
-                                        __fmul_rn(ddz, ddz)));
-  if (sn > 0.0f) {
-    const float kk = __fdiv_rn(P.bg_radius, sn);
-    qx = __fadd_rn(ox, __fmul_rn(ddx, kk));
-    qy = __fadd_rn(oy, __fmul_rn(ddy, kk));
-    qz = __fadd_rn(oz, __fmul_rn(ddz, kk));
-  }
-  const float scale = __fdiv_rn(2097152.0f, T.side);
-  const float q[3] = {qx, qy, qz};
-  int g[3];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    float t = __fmul_rn(q[d], scale);
-    if (!(t >= 0.0f)) t = 0.0f;
-    const unsigned v = __float2uint_rz(t);
-    g[d] = (int)(v > (unsigned)(kGridMax - 1) ? (unsigned)(kGridMax - 1) : v);
-  }
-  Y = kRoot;
-  dY = 0;
-  cpath[0] = kRoot;
-  for (int it = 0; it < kDepth - 1; ++it) {
-    const int ch = __ldg(&T.nT[Y].x);
-    if (ch < 0) break;
-    const int ax = __ldg(&T.nglo[Y].w);
-    const int4 up = __ldg(&T.nglo[ch + 1]);
-    const int plane = ax == 0 ? up.x : (ax == 1 ? up.y : up.z);
-    Y = g[ax] >= plane ? ch + 1 : ch;
-    cpath[++dY] = Y;
-  }
-}
-
-// The hot path for the 32 sinks of one warp (lane holds sorted position i if
-// `has`); every lane of the warp must call it. Accumulates the lane's flux in F.
-// A lane that accepts a cell (or reaches a single source) does not trace the ray at once;
-// it keeps it pending, and the pending rays of all lanes are traced together (each lane to
-// its own cell) when a lane needs its slot again or when the walk is about to overwrite the
-// part of the path a pending ray uses.
-// BG: background sources (Sec. 2.2.4). A merged cell's centre of
-// luminosity c is moved radially onto the sphere of radius R around the domain centre
-// o before its ray is traced, in fp32 as d = c - o, s = sqrt((dx^2 + dy^2) + dz^2),
-// q = o + d * (R / s); the ray then ends in the leaf that holds q, whose ancestors the
-// lane finds by descending the cut planes from the root and keeps for that ray.
-template <bool BG>
-__device__ __forceinline__ void warp_walk(const TreeView& T, const WalkParams& P, const bool has,
-                                          const int i, WarpStack& ws, int* status,
-                                          SinkCounters& cnt, CSum& F) {
-  const unsigned FULL = 0xffffffffu;
-  const unsigned lane = threadIdx.x & 31u;
-  const int stack_limit = P.stack_depth < kDepth ? P.stack_depth : kDepth;
-  const int box_limit = 2 * T.n_nodes_cap + 4;
-  int anc[kDepth];     // ancestors of S by depth
-  int rst[kRayStack];  // this lane's cells waiting to be clipped (refinement)
-  float px = 0.0f, py = 0.0f, pz = 0.0f;
-  int S = 0, dS = 0;
-  if (has) {
-    const float4 p = T.pos[i];
-    px = p.x;
-    py = p.y;
-    pz = p.z;
-    S = T.leaf_of[i];
-    dS = __ldg(&T.ndepth[S]);
-    int u = S;
-    for (int d = dS; d >= 0; --d) {
-      anc[d] = u;
-      u = __ldg(&T.nT[u].y);
-    }
-  }
-  unsigned long long on_path = 0;
-  const unsigned live = __ballot_sync(FULL, has);
-  if (lane == 0) {
-    ws.node[0] = kRoot;
-    ws.depth[0] = 0;
-    ws.mask[0] = live;
-  }
-  int sp = live ? 1 : 0;
-  // this lane's pending ray
-  bool pnd = false;
-  bool pbg = false;          // (BG) the pending ray ends at a moved source: path in cpath
-  int cpath[BG ? kDepth : 1] = {};  // (BG) ancestors of the leaf holding the moved source
-  int pC = 0, pdC = 0;
-  float pqx = 0.0f, pqy = 0.0f, pqz = 0.0f, pL = 0.0f;
-  auto flush = [&]() {
-    if (BG) {
-      // a ray to a moved source uses its own path: the common-prefix mask of that
-      // path and the sink's ancestors
-      unsigned long long onp = on_path;
-      const int* pp = ws.path;
-      if (pnd && pbg) {
-        onp = 0;
-        const int mn = pdC < dS ? pdC : dS;
-        for (int d = 0; d <= mn && cpath[d] == anc[d]; ++d) onp |= 1ull << d;
-        pp = cpath;
-      }
-      warp_ray(T, P, pnd, px, py, pz, S, dS, anc, rst, onp, pp, pC, pdC, pqx, pqy, pqz, pL,
-               box_limit, status, cnt, F);
-    } else {
-      warp_ray(T, P, pnd, px, py, pz, S, dS, anc, rst, on_path, ws.path, pC, pdC, pqx, pqy, pqz,
-               pL, box_limit, status, cnt, F);
-    }
-    pnd = false;
-    pbg = false;
-  };
-  __syncwarp();
-  while (sp > 0) {
-    --sp;
-    const int X = ws.node[sp], dX = ws.depth[sp];
-    const unsigned M = ws.mask[sp];
-    __syncwarp();
-    // a pending ray reads the path up to its cell's depth: trace it before that changes
-    if (__any_sync(FULL, pnd && !pbg && pdC >= dX)) flush();
-    if (lane == 0) ws.path[dX] = X;
-    const unsigned long long bit = 1ull << dX;
-    if (has) on_path = (dX <= dS && anc[dX] == X) ? (on_path | bit) : (on_path & ~bit);
-    __syncwarp();
-    const float4 s = __ldg(&T.nS[X]);
-    if (!(s.w > 0.0f)) continue;
-    bool acc = false, opn = false;
-    if ((M >> lane) & 1u) {
-      ++cnt.visit;
-      const float4 a = __ldg(&T.nA[X]);
-      const float4 bb = __ldg(&T.nB[X]);
-      const float ex = fmaxf(fmaxf(__fsub_rn(a.x, px), __fsub_rn(px, bb.x)), 0.0f);
-      const float ey = fmaxf(fmaxf(__fsub_rn(a.y, py), __fsub_rn(py, bb.y)), 0.0f);
-      const float ez = fmaxf(fmaxf(__fsub_rn(a.z, pz), __fsub_rn(pz, bb.z)), 0.0f);
-      const float r2 =
-          __fadd_rn(__fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey)), __fmul_rn(ez, ez));
-      acc = __ldg(&T.nl2[X]) < __fmul_rn(P.theta2, r2);
-      opn = !acc;
-    }
-    const unsigned opnM = __ballot_sync(FULL, opn);
-    if (__any_sync(FULL, acc && pnd)) flush();
-    if (acc) {
-      pnd = true;
-      pC = X;
-      pdC = dX;
-      pqx = s.x;
-      pqy = s.y;
-      pqz = s.z;
-      pL = s.w;
-      if (BG) {
-        bg_move(T, P, s, pqx, pqy, pqz, pC, pdC, cpath);
-        pbg = true;
-      }
-    }
-    if (opnM) {
-      const int4 t = __ldg(&T.nT[X]);
-      if (t.x < 0) {
-        for (int jj = t.z; jj < t.z + t.w; ++jj) {
-          const float4 y = __ldg(&T.src[jj]);
-          if (!(y.w > 0.0f)) continue;
-          if (__any_sync(FULL, opn && pnd)) flush();
-          if (opn) {
-            pnd = true;
-            pC = X;
-            pdC = dX;
-            pqx = y.x;
-            pqy = y.y;
-            pqz = y.z;
-            pL = y.w;
-          }
-        }
-      } else {
-        if (sp + 2 > stack_limit) {
-          if (lane == 0) atomicOr(status, kStatusStackOverflow);
-          break;
-        }
-        if (lane == 0) {
-          ws.node[sp] = t.x + 1;
-          ws.depth[sp] = dX + 1;
-          ws.mask[sp] = opnM;
-          ws.node[sp + 1] = t.x;
-          ws.depth[sp + 1] = dX + 1;
-          ws.mask[sp + 1] = opnM;
-        }
-        sp += 2;
-        __syncwarp();
-      }
-    }
-  }
-  if (__any_sync(FULL, pnd)) flush();
-}
-
-template <bool BG>
-__global__ void __launch_bounds__(128, 8) walk_warp_kernel(TreeView T, const long long* sink_idx,
-                                                           int n_sink, WalkParams P, SinkOut out,
-                                                           unsigned long long* stats,
-                                                           int* status) {
-  __shared__ WarpStack stacks[4];
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  WarpStack& ws = stacks[threadIdx.x >> 5];
-  SinkCounters cnt;
-  int i = 0, slot = 0;
-  float g = 0.0f;
-  bool has = false;
-  if (k < n_sink) {
-    PlainMap<false> map{&T, sink_idx, nullptr, status, P.order, n_sink};
-    has = map(k, i, slot, g);
-    if (!has && sink_idx && slot >= 0) {
-      if (out.flux) out.flux[slot] = 0.0f;
-      if (out.counters) reinterpret_cast<int4*>(out.counters)[slot] = make_int4(0, 0, 0, 0);
-    }
-  }
-  CSum F;
-  if (__any_sync(0xffffffffu, has)) warp_walk<BG>(T, P, has, i, ws, status, cnt, F);
-  if (has) {
-    if (out.flux) out.flux[slot] = F.get();
-    if (out.counters)
-      reinterpret_cast<int4*>(out.counters)[slot] =
-          make_int4(cnt.rays, cnt.segs, cnt.visit, cnt.ref);
-  }
-  if (stats) add_stats(cnt, stats);
-}
-
 cudaError_t launch_walk_batched(const TreeView* views, float* const* flux_out, const int2* items,
                                 int n_items, int item, unsigned* counter, const WalkParams& wp,
                                 unsigned long long* stats, int* status, int block_size,
@@ -912,17 +494,6 @@ cudaError_t launch_walk(const TreeView& T, const long long* sink_idx, int n_sink
                         cudaStream_t s) {
   if (n_sink <= 0) return cudaSuccess;
   (void)block_size;
-  if (wp.tau_stop < INFINITY && (counters || stats)) {
-    // the counters of a cut ray depend on the order of its segments: those of this walk
-    const dim3 grid((n_sink + 127) / 128);
-    const SinkOut o{flux_out, counters, nullptr, nullptr, n_sink};
-    if (wp.bg_radius > 0.0f)
-      walk_warp_kernel<true><<<grid, 128, 0, s>>>(T, sink_idx, n_sink, wp, o, stats, status);
-    else
-      walk_warp_kernel<false><<<grid, 128, 0, s>>>(T, sink_idx, n_sink, wp, o, stats, status);
-    note_launch();
-    return cudaGetLastError();
-  }
   if (wp.variant >= 2)
     return launch_cut_walk(T, sink_idx, n_sink, wp, flux_out, counters, stats, status, s);
   const int chunk = chunk_of(wp);
