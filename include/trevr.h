@@ -167,7 +167,11 @@ int trevr_build_tree(const float* gas_xyz, const float* alpha, const float* weig
  *             gas particles in the caller's order (then n_sink must be n_gas).
  *             They are walked in Morton order, whatever their own: the call
  *             sorts them in stream-ordered memory (24 bytes a sink), except
- *             while the stream is being captured.
+ *             while the stream is being captured or where there is no memory
+ *             for it; they are then walked as listed, which may take several
+ *             times as long. A sink's flux does not depend on that, nor on
+ *             which other sinks the call has: its bits are the same (with
+ *             sub_bucket, equal to rounding).
  *   prm       host pointer: theta_open, tau_ref, tuning fields.
  *   flux_out  n_sink floats: flux_out[k] is the flux at sink k.
  *   sink_counters  NULL, or 4*n_sink int32: per sink the number of rays,
@@ -230,7 +234,8 @@ int trevr_tree_set_smoothing(trevr_tree* t, const float* hsml, void* stream);
  *              b * n_sink + k.
  *   other arguments as in trevr_compute_flux. The counters and stats are those
  *   of the shared walk. bg_radius and tau_stop must be 0. walk_variant is
- *   ignored: the bands use the merged-ray walk.
+ *   ignored: the bands use the merged-ray walk. Every flux is a compensated
+ *   sum; between calls with few and with many sinks a last bit may differ.
  * Synchronises the stream and reports device errors.
  */
 int trevr_compute_flux_bands(const trevr_tree* t, const long long* sink_idx, long long n_sink,
@@ -249,6 +254,8 @@ int trevr_compute_flux_bands(const trevr_tree* t, const long long* sink_idx, lon
  *   fvec_out  3*n_sink floats, SoA: x[0..n), y[0..n), z[0..n).
  *   press_out NULL or 6*n_sink floats, SoA in the order xx, yy, zz, xy, xz, yz
  *             (its trace equals flux_out).
+ * The moments are compensated sums: between calls with few and with many sinks
+ * they may differ by rounding (2^-23 of the flux). The flux does not.
  * Synchronises the stream and reports device errors.
  */
 int trevr_compute_flux_moments(const trevr_tree* t, const long long* sink_idx, long long n_sink,

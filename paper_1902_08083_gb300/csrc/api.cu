@@ -93,7 +93,8 @@ static WalkParams walk_params(const trevr_tree* t, const trevr_params* prm) {
 // 31.2 ms, longer than all of them: 8 of 32 lanes ran at a time. Up to 32 sinks share a warp
 // in any order. The order costs a sort by rank; while a stream is being captured nothing is
 // allocated and the caller's order stays, as it does when there is no memory for it. A sink's
-// results do not depend on the order.
+// results do not depend on the order: the parts of its sums go by what its rays reach (with
+// the particle trace, whose parts go by the group, they are equal to rounding).
 struct SinkOrder {
   void* buf = nullptr;
   cudaStream_t s;

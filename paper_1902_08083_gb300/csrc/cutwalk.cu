@@ -7,9 +7,15 @@
 //
 // Where a call has too few sinks to fill the GPU with a warp per 32, a block of several warps
 // takes the same 32 sinks: each walks the source tree, and the takings (a cell accepted by some
-// lanes, a source reached) go to the warps in turn. A sink's flux is summed in kSlots
-// compensated parts, the takings in turn to each, whether or not the warps share a group, so
-// that the result does not depend on it.
+// lanes, a source reached) are dealt out to the warps by what is taken, a hash of the cell's
+// number or the source's. A sink's flux is summed in kSlots compensated parts, dealt out in the
+// same way whether or not warps share a group: it depends neither on that nor on the other
+// sinks of the group, and so not on the list that the sink stands in, or that list's order.
+// Three kinds of sums keep this to rounding only. Bands and moments are summed by warp, without
+// parts, and go by the number of warps, that is by how many sinks the call has (8 parts of each
+// in local memory took 9.3 ms for three bands of 200003 sinks instead of 8.0, and 9.5 for the
+// moments of 262144 instead of 7.5). The particle trace, whose rays are the longest, numbers
+// the takings as the group comes to them, which spreads them more evenly.
 //
 // A ray is a list of pieces along [0, 1] (p + t d). All of them are cut from the clip of
 // the common ancestor A of the sink's leaf S and the source's cell C: a cell's interval
@@ -63,11 +69,23 @@ struct __align__(16) CutStack {
   unsigned char place[kDepth + 2];
 };
 
-// A warp's share of a group's takings: those with (number & (parts - 1)) == part. parts is a
+// A warp's share of a group's takings: those whose number & (parts - 1) is part. parts is a
 // power of two, at most kSlots.
 struct Share {
   int part, parts;
+  __device__ __forceinline__ bool has(int number) const { return (number & (parts - 1)) == part; }
 };
+
+// The slot of a taking of cells, from the cell alone; a source's is its number. Against takings
+// numbered as the group comes to them, the hash takes 6.4 instead of 6.9 ms for 100003 sinks
+// and 9.2 instead of 9.5 for a background field of 32768 (more rays of a warp go to the same
+// cells), but 13.7 instead of 13.0 for the particle trace of 8000, 33.9 instead of 33.2 of
+// 65536. Numbered by lane, the rays that a warp traces together go to different cells: 12.6 ms
+// for the background field, and 57.5 instead of 56.0 at 2^22 sinks.
+__device__ __forceinline__ int cell_slot(int cell) {
+  return (int)((unsigned)cell * 2654435761u >> 29);
+}
+static_assert(kSlots == 8, "the hash has three bits");
 
 // Compensated sums of one lane's takings, one per slot.
 struct Slots {
@@ -714,8 +732,8 @@ __device__ __forceinline__ void cut_walk(const TreeView& T, const WalkParams& P,
   int j = 0, j_end = 0;   // sources of the opened leaf from j on are still to be looked at
   unsigned opened = 0;    // the lanes that opened it
   unsigned lit = 0, own = 0;  // of the 32 sources before j: those with light, this warp's of them
-  int first = 0;              // number of the takings before the first of `lit`
-  int taken = 0, w_slot = 0;  // takings so far; the slot of the waiting ray
+  int taken = 0, first = 0;   // (SUB) takings so far, and before the first of `lit`
+  int w_slot = 0;             // the waiting ray's slot
   if (!ADJ && NB == 1) flux.clear();
   __syncwarp();
   while (true) {
@@ -725,15 +743,15 @@ __device__ __forceinline__ void cut_walk(const TreeView& T, const WalkParams& P,
       const int q = __ffs(own) - 1;
       own &= own - 1u;
       ent = ~(j - 32 + q);
-      turn = first + __popc(lit & ((1u << q) - 1u));
+      turn = SUB ? first + __popc(lit & ((1u << q) - 1u)) : j - 32 + q;
       take = (opened >> lane) & 1u;
     } else if (j < j_end) {
       const int mine = j + (int)lane;
       const bool light = mine < j_end && __ldg(&T.src[mine].w) > 0.0f;
       lit = __ballot_sync(FULL, light);
       first = taken;
-      const int number = first + __popc(lit & ((1u << lane) - 1u));
-      own = __ballot_sync(FULL, light && (number & (share.parts - 1)) == share.part);
+      const int number = SUB ? first + __popc(lit & ((1u << lane) - 1u)) : mine;
+      own = __ballot_sync(FULL, light && share.has(number));
       taken += __popc(lit);
       j += 32;
       continue;
@@ -786,8 +804,8 @@ __device__ __forceinline__ void cut_walk(const TreeView& T, const WalkParams& P,
         }
       }
       if (!__any_sync(FULL, take)) continue;
-      turn = taken++;
-      if ((turn & (share.parts - 1)) != share.part) continue;
+      turn = SUB ? taken++ : cell_slot(X);
+      if (!share.has(turn)) continue;
     } else {
       done = true;
     }

@@ -1,6 +1,6 @@
 """The forms that one walk takes: with and without counters, in groups of 32 sinks that one,
 two, four or eight warps share (from the most sinks to the fewest), and over sinks in other
-company. A sink's results are its own in every form, bit for bit."""
+company. A sink's flux is its own in every form, bit for bit."""
 import numpy as np
 import pytest
 
@@ -58,3 +58,77 @@ def test_tau_stop_without_counters_against_the_oracle(n):
     of = oracle_tree(P).flux_terminated(0.6, 0.1, 2.0, sinks=sinks)
     f0 = oracle_tree(dict(P, alpha=np.zeros_like(P["alpha"]))).flux(0.6, 0.1, sinks=sinks)
     _check(f, of, f0, 2.0, f"n={n}")
+
+
+def _calls(n, s):
+    """name -> f(sink_idx): every result of a call, one row of numbers per sink."""
+    import torch
+    from paper_1902_08083_gb300 import trevr
+    P = _problem(n, s)
+    G = gpu_tree(P)
+    G.set_smoothing(torch.full((n,), 0.6 * n ** (-1 / 3), device="cuda"))
+    bg = gpu_tree(workloads.background_shell(n_gas=n, n_bg=max(s, 300), radius=0.45, alpha=8.0))
+
+    def bands(k):
+        t = {q: torch.from_numpy(P[q]).cuda() for q in ("gas_xyz", "alpha", "src_xyz", "src_lum")}
+        f = torch.arange(1, k + 1, device="cuda")[:, None].float()
+        return trevr.build_tree(t["gas_xyz"], (t["alpha"] * f).contiguous(), t["src_xyz"],
+                                (t["src_lum"] / f).contiguous())
+
+    calls = {"per lane": lambda i: trevr.compute_flux(G, 0.6, 0.1, sink_idx=i, walk_variant=1),
+             "variant 2": lambda i: trevr.compute_flux(G, 0.6, 0.1, sink_idx=i, walk_variant=2),
+             "moments": lambda i: torch.cat([x.reshape(-1, x.shape[-1]) for x in
+                                             trevr.compute_flux_moments(G, 0.6, 0.1, sink_idx=i)])}
+    for name, kw in (("plain", {}), ("stop", dict(tau_stop=2.0)), ("top-down", dict(ray_walk=1)),
+                     ("particles", dict(sub_bucket=1))):
+        calls[name] = lambda i, kw=kw: trevr.compute_flux(G, 0.6, 0.1, sink_idx=i, **kw)
+    for name, kw in (("background", {}), ("background and stop", dict(tau_stop=2.0))):
+        calls[name] = lambda i, kw=kw: trevr.compute_flux(bg, 0.6, 0.1, sink_idx=i, bg_radius=0.45,
+                                                          **kw)
+    for k in (2, 3, 4):
+        B = bands(k)
+        calls[f"{k} bands"] = lambda i, B=B: trevr.compute_flux_bands(B, 0.6, 0.1, sink_idx=i)
+    return calls
+
+
+@pytest.mark.parametrize("n,s", [(5001, 200), (60000, 60), (330000, 60)])
+def test_every_form_of_the_walk_over_lists(n, s):
+    # whole boxes of 8, 4 and 1 warps a group; lists in another order, with repeats, of 8.
+    # Bands, moments and the particle trace are other compensated parts of the same terms,
+    # good to an ulp of the sum of the terms' sizes
+    import torch
+    rng = np.random.default_rng(n)
+    wrong = []
+    for name, call in _calls(n, s).items():
+        whole = call(None)
+        for m in (1, 31, 33, 257, 5000):
+            i = torch.from_numpy(rng.integers(0, n, m)).cuda()
+            f = call(i)
+            if name in ("moments", "2 bands", "3 bands", "4 bands", "particles"):
+                size = whole[:1] if name == "moments" else whole
+                good = ((f - whole[..., i]).abs() <= 2.0 ** -22 * size[..., i]).all()
+                if name == "moments":
+                    good = good and torch.equal(f[0], whole[0, i])
+            else:
+                good = torch.equal(f, whole[..., i])
+            if not good:
+                wrong.append((name, m))
+    assert not wrong
+
+
+def test_a_captured_list_gives_the_same_bits():
+    # while a stream is captured the sinks of a list keep the caller's order
+    import torch
+    from paper_1902_08083_gb300 import trevr
+    G = gpu_tree(_problem(60000, 200))
+    i = torch.from_numpy(np.random.default_rng(3).integers(0, 60000, 9001)).cuda()
+    want = trevr.compute_flux(G, 0.6, 0.1, sink_idx=i)
+    out = torch.zeros(9001, device="cuda")
+    g, st = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    st.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(g, stream=st):
+        trevr.compute_flux(G, 0.6, 0.1, sink_idx=i, out=out, stream=torch.cuda.current_stream())
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
