@@ -123,7 +123,7 @@ typedef struct {
     long long cells_clipped;     /* cells that a ray is cut with: its base cells, and the
                                     children that it crosses of the cells it refines */
     float build_ms;
-    float walk_ms;
+    float walk_ms;               /* the walk, and the ordering of listed sinks before it */
     long long rays_terminated;   /* rays cut off by tau_stop (of the interactions) */
     long long sub_bucket_segments; /* leaf segments integrated through the particles */
 } trevr_stats;

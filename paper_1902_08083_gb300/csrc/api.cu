@@ -248,8 +248,6 @@ int trevr_compute_flux_bands(const trevr_tree* t, const long long* sink_idx, lon
   if (!flux_out) return TREVR_ERR_INVALID_ARGUMENT;
   if (!sink_idx && n_sink != t->n_gas) return TREVR_ERR_INVALID_ARGUMENT;
   cudaStream_t s = (cudaStream_t)stream;
-  WalkParams wp = walk_params(t, prm);
-  const SinkOrder sorted(t, sink_idx, n_sink, wp, s);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (stats) {
     cudaMemsetAsync(t->d_stats, 0, 7 * sizeof(unsigned long long), s);
@@ -257,6 +255,8 @@ int trevr_compute_flux_bands(const trevr_tree* t, const long long* sink_idx, lon
     cudaEventCreate(&e1);
     cudaEventRecord(e0, s);
   }
+  WalkParams wp = walk_params(t, prm);
+  const SinkOrder sorted(t, sink_idx, n_sink, wp, s);
   cudaError_t err = launch_walk_bands(t->view(), sink_idx, (int)n_sink, wp, flux_out,
                                       sink_counters, stats ? t->d_stats : nullptr, t->status, s);
   if (err != cudaSuccess) {
@@ -307,8 +307,6 @@ int trevr_compute_flux(const trevr_tree* t, const long long* sink_idx, long long
   if (!flux_out) return TREVR_ERR_INVALID_ARGUMENT;
   if (!sink_idx && n_sink != t->n_gas) return TREVR_ERR_INVALID_ARGUMENT;
   cudaStream_t s = (cudaStream_t)stream;
-  WalkParams wp = walk_params(t, prm);
-  const SinkOrder sorted(t, sink_idx, n_sink, wp, s);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (stats) {
     cudaMemsetAsync(t->d_stats, 0, 7 * sizeof(unsigned long long), s);
@@ -316,6 +314,8 @@ int trevr_compute_flux(const trevr_tree* t, const long long* sink_idx, long long
     cudaEventCreate(&e1);
     cudaEventRecord(e0, s);
   }
+  WalkParams wp = walk_params(t, prm);
+  const SinkOrder sorted(t, sink_idx, n_sink, wp, s);
   cudaError_t err = launch_walk(t->view(), sink_idx, (int)n_sink, wp, flux_out, sink_counters,
                                 stats ? t->d_stats : nullptr, t->status, prm->block_size, s);
   if (err != cudaSuccess) {
