@@ -1,7 +1,7 @@
 // Radiation-tree build on the GPU (Grond et al. 2019, Sec. 2.2 and 2.3):
 // Morton keys -> stable radix sort (sort.cu) -> binary tree of Morton prefixes (topology.cu) ->
-// source deposit -> bottom-up cell moments. The host synchronises once, after the topology, to
-// size the moment pass.
+// source deposit -> bottom-up cell moments. The host synchronises once, when the cuts are known
+// and so the number of cells, to allocate the cells and size the moment pass.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -420,9 +420,6 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
     volatile float side = dom->side;  // fp32 on the host, as on the device
     t->h = side * (1.0f / 2097152.0f);
   }
-  const size_t cap = 2 * (size_t)n + 2;
-  t->cap_nodes = cap;
-
   const int nmax = n > ns ? n : ns;
   unsigned *vals, *topo_scan, *svals;
   unsigned long long* skeys;
@@ -436,13 +433,6 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
         a.get(t->leaf_of, n);
         a.get(t->pos, n);
         a.get(t->w, n);
-        a.get(t->nfirst, cap);
-        a.get(t->ncount, cap);
-        a.get(t->nglo, cap);
-        a.get(t->nghi, cap);
-        a.get(t->nT, cap);
-        a.get(t->ndepth, cap);
-        a.get(t->nD, cap);
         a.get(t->src, ns);
         a.get(t->src_order, ns);
         a.get(t->src_leaf, ns);
@@ -513,16 +503,9 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   TA.bucket = bucket;
   TA.key = t->key;
   TA.status = t->status;
-  TA.nfirst = t->nfirst;
-  TA.ncount = t->ncount;
-  TA.nglo = t->nglo;
-  TA.nghi = t->nghi;
-  TA.nT = t->nT;
-  TA.ndepth = t->ndepth;
-  TA.nD = t->nD;
   TA.leaf_of = t->leaf_of;
   TA.levels = t->levels;
-  launch_topology(TA, topo_scan, s);
+  launch_cuts(TA, topo_scan, s);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return fail(cuda_to_error(err));
   int levels[2 * kMaxLevels];
@@ -543,6 +526,13 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   unsigned* arrived;
   t->mem[1] = allocate(
       [&](Layout& a) {
+        a.get(t->nfirst, ncell);
+        a.get(t->ncount, ncell);
+        a.get(t->nglo, ncell);
+        a.get(t->nghi, ncell);
+        a.get(t->nT, ncell);
+        a.get(t->ndepth, ncell);
+        a.get(t->nD, ncell);
         a.get(t->nA, ncell);
         a.get(t->nB, ncell);
         a.get(t->nS, ncell);
@@ -559,6 +549,14 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
       },
       s);
   if (!t->mem[1] || !sums) return fail(TREVR_ERR_OUT_OF_MEMORY);
+  TA.nfirst = t->nfirst;
+  TA.ncount = t->ncount;
+  TA.nglo = t->nglo;
+  TA.nghi = t->nghi;
+  TA.nT = t->nT;
+  TA.ndepth = t->ndepth;
+  TA.nD = t->nD;
+  launch_cells(TA, s);
 
   // 3. sources
   if (ns > 0) {

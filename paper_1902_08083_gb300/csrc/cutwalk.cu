@@ -48,13 +48,18 @@ namespace trevr {
 
 namespace {
 
-// pieces of a ray: at most 62 on either path and the path's end, and one waiting child per
-// level of the piece that is being refined; kSpare entries of the upper end for the siblings
-// set aside (at most one plane per axis lies within an ulp of a point; kSpare bounds them
-// whatever the domain's planes are)
-constexpr int kPieces = 4 * kDepth;
+// Pieces of a ray. From an ancestor A at depth ds to leaves at depth kDepth - 1 at most, either
+// path has kDepth - 2 - ds siblings and its end. The C side waits whole, behind it the entry
+// (0, t) and the S side but for the piece being walked; that one lies below depth ds + 1, and
+// has one waiting child a level. While the list is made there are no waiting children, and the
+// siblings set aside (at most one plane per axis lies within an ulp of a point; kSpare bounds
+// them whatever the domain's planes are) take the upper end: they are siblings of the path, so
+// the entries of both ends stay below kPieces together. The list is most of a thread's stack,
+// which the driver sets aside for all threads that the GPU holds.
+constexpr int kPieces = 3 * kDepth;
 constexpr int kSpare = 20;
-static_assert(3 * kDepth + 3 + 2 * kSpare <= kPieces, "the list holds every piece of a ray");
+static_assert((kDepth - 1) + 1 + (kDepth - 2) + (kDepth - 3) <= kPieces,
+              "the list holds every piece of a ray");
 constexpr int kSegBuf = 64;  // segments of one ray kept for the adjoint's replay
 
 constexpr int kSlots = 8;    // parts of a sink's flux; at most as many warps per group

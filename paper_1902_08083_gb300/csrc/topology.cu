@@ -9,11 +9,13 @@
 //   cut_kernel    range, bit and parent of every cut                      (one thread a pair)
 //   depth_kernel  depth of the kept cuts, counted by depth in tiles of the particle order
 //   a prefix sum over (depth, tile)
-//   place_kernel  breadth-first place of each kept cut: by depth, then by particle order
+//   place_kernel  breadth-first place of each kept cut: by depth, then by particle order; and
+//                 the levels' ranges of cells, which the host needs to allocate the cells
 //   cell_kernel   the cell of each kept cut and its children that are leaves, whole records
 // The children of the cut at place P are the cells 2 + 2 P and 3 + 2 P: the breadth-first
-// numbering. Six launches; a launch and two grid-wide barriers for each of ~20 levels took 266
-// us at 2^18 particles and 141 us at 4096.
+// numbering. Four launches and those of the prefix sum (one up to 16384 particles, three up to
+// 2^24); a launch and two grid-wide barriers for each of ~20 levels took 266 us at 2^18
+// particles and 141 us at 4096.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -114,6 +116,18 @@ __global__ void __launch_bounds__(kTileThreads) place_kernel(TopoArrays A, int t
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int d = lane; d < kDepths; d += 32) count[warp][d] = 0;
   __syncwarp();
+  if (blockIdx.x == 0 && threadIdx.x < kMaxLevels) {
+    // the levels' cells: a thread each, from the cuts before and up to the depth above it
+    const int d = (int)threadIdx.x - 1;
+    int begin = kRoot, end = no_tree(A) ? kRoot : kRoot + 1;
+    if (d >= 0) {
+      begin = kRoot + 1 + 2 * (int)A.counts[(size_t)min(d, kDepths) * tiles];
+      end = kRoot + 1 + 2 * (int)A.counts[(size_t)min(d + 1, kDepths) * tiles];
+      if (begin == end) begin = end = 0;
+    }
+    A.levels[2 * threadIdx.x] = begin;
+    A.levels[2 * threadIdx.x + 1] = end;
+  }
   const int own = blockIdx.x * kTile + warp * 32 * kItems + lane;
   unsigned rank[kItems];
   int depth[kItems];
@@ -167,22 +181,11 @@ __device__ __forceinline__ void write_cell(const TopoArrays& A, int X, int child
 
 __global__ void cell_kernel(TopoArrays A, int tiles) {
   const int first_thread = blockIdx.x * blockDim.x + threadIdx.x;
-  const unsigned* c = A.counts;
-  if (first_thread == 0) {
-    // the levels' cells, the unused cell 0, and a root without a cut
-    int end = kRoot + 1;
-    A.levels[0] = kRoot;
-    A.levels[1] = no_tree(A) ? kRoot : end;
-    for (int d = 0; d + 1 < kMaxLevels; ++d) {
-      const int cuts = d < kDepths ? (int)(c[(size_t)(d + 1) * tiles] - c[(size_t)d * tiles]) : 0;
-      A.levels[2 * d + 2] = cuts ? end : 0;
-      A.levels[2 * d + 3] = cuts ? end + 2 * cuts : 0;
-      end += 2 * cuts;
-    }
+  if (first_thread == 0) {  // the unused cell 0
     A.nT[0] = make_int4(-1, 0, 0, 0);
     A.nD[0] = 1ull << 63;
   }
-  const int total = (int)c[(size_t)kDepths * tiles];
+  const int total = (int)A.counts[(size_t)kDepths * tiles];
   if (total == 0) {
     const int lo[3] = {0, 0, 0}, hi[3] = {kGridMax, kGridMax, kGridMax};
     if (first_thread == 0) write_cell(A, kRoot, -1, 0, lo, hi, -1, 0, A.n, 0, 0ull);
@@ -242,15 +245,19 @@ int tiles_of(int n) { return (n + kTile - 1) / kTile; }
 
 size_t topo_count_words(int n) { return (size_t)kDepths * tiles_of(n) + 1; }
 
-void launch_topology(const TopoArrays& A, unsigned* scan_scratch, cudaStream_t s) {
+void launch_cuts(const TopoArrays& A, unsigned* scan_scratch, cudaStream_t s) {
   const int n = A.n, tiles = tiles_of(n);
   cut_kernel<<<(n + 255) / 256, 256, 0, s>>>(A);
   depth_kernel<<<tiles, kTileThreads, 0, s>>>(A, tiles);
   exclusive_scan_u32(A.counts, (int)topo_count_words(n), scan_scratch, s);
   place_kernel<<<tiles, kTileThreads, 0, s>>>(A, tiles);
-  const int blocks = n / 512 + 1;  // about one cut in six particles is kept
-  cell_kernel<<<blocks < 4096 ? blocks : 4096, 128, 0, s>>>(A, tiles);
-  note_launch(4);
+  note_launch(3);
+}
+
+void launch_cells(const TopoArrays& A, cudaStream_t s) {
+  const int blocks = A.n / 512 + 1;  // about one cut in six particles is kept
+  cell_kernel<<<blocks < 4096 ? blocks : 4096, 128, 0, s>>>(A, tiles_of(A.n));
+  note_launch();
 }
 
 }  // namespace trevr

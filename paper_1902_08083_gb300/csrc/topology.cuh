@@ -36,7 +36,10 @@ struct TopoArrays {
 };
 
 size_t topo_count_words(int n);
-// scan_scratch holds scan_scratch_words(topo_count_words(n)) words
-void launch_topology(const TopoArrays& A, unsigned* scan_scratch, cudaStream_t s);
+// The kept cuts, their places and the levels' cell ranges (an empty root level if the sort gave
+// up). scan_scratch holds scan_scratch_words(topo_count_words(n)) words.
+void launch_cuts(const TopoArrays& A, unsigned* scan_scratch, cudaStream_t s);
+// The cells: the tree's arrays, which have to hold as many as the levels end at.
+void launch_cells(const TopoArrays& A, cudaStream_t s);
 
 }  // namespace trevr

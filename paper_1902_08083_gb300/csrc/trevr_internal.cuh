@@ -103,7 +103,6 @@ struct trevr_tree {
   int max_depth;
   int bucket;
   float lo[3], side, h;
-  size_t cap_nodes;
   // particles
   unsigned long long* key;
   int* perm;
