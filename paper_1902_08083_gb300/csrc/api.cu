@@ -60,6 +60,16 @@ cudaError_t pool_malloc_async(void** p, size_t bytes, cudaStream_t s) {
   return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
 
+int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    n = 1;
+  }
+  return n;
+}
+
 int cuda_to_error(cudaError_t e) {
   if (e == cudaSuccess) return TREVR_OK;
   if (e == cudaErrorMemoryAllocation) return TREVR_ERR_OUT_OF_MEMORY;

@@ -1004,15 +1004,15 @@ __global__ void __launch_bounds__(SHARED ? 32 * kSlots : 128, SHARED ? 4 : 8)
         T, P, has, i, g, share, stacks[warp], status, J, cnt, none, nullptr, nullptr);
 }
 
-// Warps per group of 32 sinks: doubled while the call then has at most 64 warps on each of the
-// 152 SMs. At 32768 sinks of a background field 8 take 11.8 ms (1: 29.6, 4: 12.3); at 100003
-// sinks 2 take 7.80 (1: 8.31, 4: 7.83, 8: 7.99); at 65536 sinks with the particle trace 4 take
-// 39.7 (1: 59.0, 2: 50.2, 8: 43.5); at 262144 sinks one warp takes 7.5 and 2 take 8.5, since
-// every warp of a group walks the whole source tree.
+// Warps per group of 32 sinks: doubled while the call then has at most 64 warps on each SM (152
+// SMs where this was measured). At 32768 sinks of a background field 8 take 11.8 ms (1: 29.6,
+// 4: 12.3); at 100003 sinks 2 take 7.80 (1: 8.31, 4: 7.83, 8: 7.99); at 65536 sinks with the
+// particle trace 4 take 39.7 (1: 59.0, 2: 50.2, 8: 43.5); at 262144 sinks one warp takes 7.5 and
+// 2 take 8.5, since every warp of a group walks the whole source tree.
 int group_warps(int n_sink, int most) {
-  const int groups = (n_sink + 31) / 32;
+  const int groups = (n_sink + 31) / 32, fill = 64 * sm_count();
   int w = 1;
-  while (w < most && 2 * w * groups <= 64 * 152) w *= 2;
+  while (w < most && 2 * w * groups <= fill) w *= 2;
   return w;
 }
 

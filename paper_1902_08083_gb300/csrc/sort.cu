@@ -372,8 +372,8 @@ void radix_sort(unsigned long long* k, unsigned* v, int n, int bits, const SortS
   unsigned *counts = S.work, *tickets = S.work + 8 * 256;
   unsigned* words[2] = {S.work + kSortHead, S.work + kSortHead + 256 * (size_t)tiles};
   cudaMemsetAsync(S.work, 0, ((size_t)kSortHead + 256 * (size_t)tiles) * sizeof(unsigned), s);
-  const int counters = (n + kCountTile - 1) / kCountTile;
-  digit_count_kernel<<<counters < 608 ? counters : 608, 256, 0, s>>>(k, n, passes, counts);
+  const int counters = (n + kCountTile - 1) / kCountTile, fill = 4 * sm_count();
+  digit_count_kernel<<<counters < fill ? counters : fill, 256, 0, s>>>(k, n, passes, counts);
   note_launch();
   unsigned long long *ka = k, *kb = S.k2;
   unsigned *va = v, *vb = S.v2;

@@ -250,6 +250,7 @@ cudaError_t adjoint_finalize(const trevr_tree* t, const AdjointArgs& J, float* g
 // the driver at every synchronisation, and every tree build would map its buffers
 // again). Free with cudaFreeAsync, or cudaFree.
 cudaError_t pool_malloc_async(void** p, size_t bytes, cudaStream_t s);
+int sm_count();  // of the current device (1 if it cannot be asked)
 int status_to_error(int status_bits);
 void note_launch(int n = 1);  // count kernels launched by the library
 int cuda_to_error(cudaError_t e);
