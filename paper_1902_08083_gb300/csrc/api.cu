@@ -124,8 +124,8 @@ struct SinkOrder {
       return;
     }
     unsigned* order = static_cast<unsigned*>(buf);
-    sink_order(t, sink_idx, (int)n, static_cast<unsigned char*>(buf) + own, order, s);
-    wp.order = order;
+    if (sink_order(t, sink_idx, (int)n, static_cast<unsigned char*>(buf) + own, order, s))
+      wp.order = order;
   }
   ~SinkOrder() {
     if (buf) cudaFreeAsync(buf, s);

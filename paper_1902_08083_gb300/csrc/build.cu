@@ -65,7 +65,7 @@ size_t sink_order_bytes(int n) {
   return 2 * align256((size_t)n * 8) + align256((size_t)n * 4) + align256(sort_work_words(n) * 4);
 }
 
-void sink_order(const trevr_tree* t, const long long* sink_idx, int n, void* scratch,
+bool sink_order(const trevr_tree* t, const long long* sink_idx, int n, void* scratch,
                 unsigned* order, cudaStream_t s) {
   unsigned char* p = static_cast<unsigned char*>(scratch);
   auto take = [&](size_t bytes) {
@@ -78,12 +78,14 @@ void sink_order(const trevr_tree* t, const long long* sink_idx, int n, void* scr
   S.k2 = static_cast<unsigned long long*>(take((size_t)n * 8));
   S.v2 = static_cast<unsigned*>(take((size_t)n * 4));
   S.work = static_cast<unsigned*>(take(sort_work_words(n) * 4));
+  S.size = (size_t)n;
+  S.words = sort_work_words(n);
   const int n_gas = (int)t->n_gas;
   sink_keys_kernel<<<(n + 255) / 256, 256, 0, s>>>(sink_idx, n, n_gas, t->rank, keys, order);
   note_launch();
   int bits = 1;  // keys are ranks, and n_gas itself
   while (bits < 31 && (n_gas >> bits)) ++bits;
-  radix_sort(keys, order, n, bits, S, t->status, s);
+  return radix_sort(keys, order, n, bits, S, t->status, s);
 }
 
 // ------------------------------------------------------------------------------------
@@ -424,6 +426,9 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   unsigned *vals, *topo_scan, *svals;
   unsigned long long* skeys;
   SortScratch SS;
+  SS.size = (size_t)nmax;
+  // (not monotone: a smaller sort may have more tiles)
+  SS.words = std::max(sort_work_words(n), sort_work_words(ns));
   TopoArrays TA;
   t->mem[0] = allocate(
       [&](Layout& a) {
@@ -443,10 +448,9 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   void* scratch = allocate(
       [&](Layout& a) {
         a.get(vals, n);
-        a.get(SS.k2, nmax);
-        a.get(SS.v2, nmax);
-        // (not monotone: a smaller sort may have more tiles)
-        a.get(SS.work, std::max(sort_work_words(n), sort_work_words(ns)));
+        a.get(SS.k2, SS.size);
+        a.get(SS.v2, SS.size);
+        a.get(SS.work, SS.words);
         a.get(TA.up, n);
         a.get(TA.range, n);
         a.get(TA.bit, n);
@@ -494,7 +498,7 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
   keys_kernel<<<grid_for(n, 256), 256, 0, s>>>(gas_xyz, alpha, weight, n, D, t->key, vals,
                                                  t->status);
   note_launch();
-  radix_sort(t->key, vals, n, 63, SS, t->status, s);
+  if (!radix_sort(t->key, vals, n, 63, SS, t->status, s)) return fail(TREVR_ERR_CUDA);
   gather_particles_kernel<<<grid_for(n, 256), 256, 0, s>>>(gas_xyz, alpha, weight, n, D, vals,
                                                             t->pos, t->w, t->perm, t->rank);
   note_launch();
@@ -565,7 +569,7 @@ int build_tree_impl(const float* gas_xyz, const float* alpha, const float* weigh
     note_launch();
     int bits = 1;  // keys are particle numbers
     while (bits < 31 && ((n - 1) >> bits)) ++bits;
-    radix_sort(skeys, svals, ns, bits, SS, t->status, s);
+    if (!radix_sort(skeys, svals, ns, bits, SS, t->status, s)) return fail(TREVR_ERR_CUDA);
     gather_sources_kernel<<<grid_for(ns, 256), 256, 0, s>>>(src_xyz, src_lum, ns, n, D, svals,
                                                              skeys, t->leaf_of, t->src,
                                                              t->src_order, t->src_leaf);

@@ -93,7 +93,6 @@ extern "C" int trevr_morton_sort_noalloc(const float* gas_xyz, long long n_gas,
   for (int d = 0; d < 3; ++d)
     if (!std::isfinite(dom->lo[d]) || !std::isfinite(dom->lo[d] + dom->side))
       return TREVR_ERR_INVALID_ARGUMENT;
-  if (sort_work_words((int)n_gas) > kWorkWords) return TREVR_ERR_INVALID_ARGUMENT;
   unsigned char* base = nullptr;
   cudaError_t err = scratch_on_current_device(&base);
   if (err != cudaSuccess) return cuda_to_error(err);
@@ -103,6 +102,8 @@ extern "C" int trevr_morton_sort_noalloc(const float* gas_xyz, long long n_gas,
   S.k2 = reinterpret_cast<unsigned long long*>(base + kOffK2);
   S.v2 = reinterpret_cast<unsigned*>(base + kOffV2);
   S.work = reinterpret_cast<unsigned*>(base + kOffWork);
+  S.size = kMaxN;
+  S.words = kWorkWords;
   int* status = reinterpret_cast<int*>(base + kOffStatus);
   // the status word must start at zero; the rest of the scratch is fully
   // overwritten before it is read
@@ -123,7 +124,8 @@ extern "C" int trevr_morton_sort_noalloc(const float* gas_xyz, long long n_gas,
                                                        reinterpret_cast<unsigned*>(perm_out),
                                                        status);
   note_launch();
-  radix_sort(keys_out, reinterpret_cast<unsigned*>(perm_out), n, 63, S, status, s);
+  if (!radix_sort(keys_out, reinterpret_cast<unsigned*>(perm_out), n, 63, S, status, s))
+    return TREVR_ERR_CUDA;
   int h_status = 0;
   err = cudaMemcpyAsync(&h_status, status, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);

@@ -359,15 +359,16 @@ size_t sort_work_words(int n) {
   return (size_t)kSortHead + 2 * 256 * (size_t)((n + sort_tile(n) - 1) / sort_tile(n));
 }
 
-void radix_sort(unsigned long long* k, unsigned* v, int n, int bits, const SortScratch& S,
+bool radix_sort(unsigned long long* k, unsigned* v, int n, int bits, const SortScratch& S,
                 int* status, cudaStream_t s) {
-  if (n <= 1) return;
+  if (n <= 1) return true;
   const int passes = (bits + 7) / 8;
   if (n <= kSmallSort) {
     small_sort_kernel<<<1, kSmallThreads, 0, s>>>(k, v, n, passes);
     note_launch();
-    return;
+    return true;
   }
+  if (S.size < (size_t)n || S.words < sort_work_words(n)) return false;
   const int tile = sort_tile(n), tiles = (n + tile - 1) / tile;
   unsigned *counts = S.work, *tickets = S.work + 8 * 256;
   unsigned* words[2] = {S.work + kSortHead, S.work + kSortHead + 256 * (size_t)tiles};
@@ -394,6 +395,7 @@ void radix_sort(unsigned long long* k, unsigned* v, int n, int bits, const SortS
     cudaMemcpyAsync(k, ka, (size_t)n * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s);
     cudaMemcpyAsync(v, va, (size_t)n * sizeof(unsigned), cudaMemcpyDeviceToDevice, s);
   }
+  return true;
 }
 
 }  // namespace trevr

@@ -170,11 +170,14 @@ struct SortScratch {
   unsigned long long* k2;  // n keys
   unsigned* v2;            // n values
   unsigned* work;          // sort_work_words(n)
+  size_t size;             // what k2 and v2 hold
+  size_t words;            // what work holds
 };
 size_t sort_work_words(int n);
 // sorts (k, v) in place by bits [0, bits) of k, with every key < 2^bits; a look-back that does
-// not end in time sets kStatusIterationLimit in *status
-void radix_sort(unsigned long long* k, unsigned* v, int n, int bits, const SortScratch& S,
+// not end in time sets kStatusIterationLimit in *status. A scratch that is too small
+// sorts nothing: false.
+bool radix_sort(unsigned long long* k, unsigned* v, int n, int bits, const SortScratch& S,
                 int* status, cudaStream_t s);
 size_t scan_scratch_words(int n);
 // exclusive prefix sum of n words in place; scratch holds scan_scratch_words(n) words
@@ -185,7 +188,7 @@ int set_smoothing_impl(trevr_tree* t, const float* h, cudaStream_t s);
 // ---- build.cu: the positions [0, n) of sink_idx in Morton order of their particles (those
 // out of range last) in `order`; `scratch` holds sink_order_bytes(n)
 size_t sink_order_bytes(int n);
-void sink_order(const trevr_tree* t, const long long* sink_idx, int n, void* scratch,
+bool sink_order(const trevr_tree* t, const long long* sink_idx, int n, void* scratch,
                 unsigned* order, cudaStream_t s);
 
 // ---- walk.cu
