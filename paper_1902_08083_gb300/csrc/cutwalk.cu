@@ -700,8 +700,8 @@ __device__ __forceinline__ void cut_ray(const TreeView& T, const WalkParams& P, 
 // A step of the walk is a chain of loads for all lanes, and below some 10^5 sinks that chain is
 // what it takes. So a cell is two 16-byte loads that are on their way together (they were five
 // in three arrays, one behind another), dark children are never pushed, and an opened leaf's
-// sources are looked at 32 at a time: 7.35 -> 7.05 ms at 100003 sinks, 10.8 -> 9.6 for a
-// background field at 32768, 0.52 -> 0.48 for a step of 4096, 54.1 -> 53.2 at 2^22.
+// sources are looked at 32 at a time: side by side, 7.35 -> 7.05 ms at 100003 sinks, 10.8 -> 9.6
+// for a background field at 32768, 0.52 -> 0.48 for a step of 4096, 54.1 -> 53.2 at 2^22.
 template <bool ADJ, bool MERGE, bool MOM, bool BG, bool STOP, int NB, bool SUB, bool CNT, bool TD>
 __device__ __forceinline__ void cut_walk(const TreeView& T, const WalkParams& P, const bool has,
                                          const int i, const float grad, const Share share,
@@ -831,14 +831,14 @@ __device__ __forceinline__ void cut_walk(const TreeView& T, const WalkParams& P,
 // Issue-bound where a call fills the GPU (86% of the issue slots at 2^20 sinks): the loop over
 // a ray's pieces is ~60 instructions on one 16-byte record that L1 mostly has, and what bounds
 // the walk is how many of them it runs. Clipping every base cell and refined child instead
-// (~120 instructions on 44 bytes, 53 a ray where 35 are crossed) took 118.4 ms a step at 2^22
-// sinks and 2^14 clumped sources; the cut pieces took 56.7 ms and take 53.2 now (21.4, 8.3 and
-// 7.1 ms at 100003 sinks, tau_ref = 0.01).
-// Blocks of 128 per SM: 8 leave the plain walk its registers (56, no spills); 12 and 16 (40
-// and 32 registers) gave 58.9 and 55.9 ms against 57.3 at 2^22, but 9.5 and 10.1 against 8.4 ms
-// at 100003 sinks, where a warp's own speed counts. The particle trace waits for L2 and wants
-// warps: 5 blocks (94 registers) take 38.9 ms at 2^16 sinks, 4 take 44.0 and 6, which spill,
-// 43.4. The bands take 6 (8.95 ms for three at 200003 sinks, 9.2 at 8).
+// (~120 instructions on 44 bytes, 53 a ray where 35 are crossed) takes 124 ms a step at 2^22
+// sinks and 2^14 clumped sources, the cut pieces take 60 (in turn, among other work; a rested
+// GPU takes 118 and 52), and 22.3 and 6.7 ms at 100003 sinks, tau_ref = 0.01.
+// Blocks of 128 per SM: 8 leave the plain walk its registers (54, no spills); when it took 57.3
+// ms at 2^22 sinks and 8.4 at 100003, 12 and 16 blocks (40 and 32 registers) gave 58.9 and 55.9,
+// but 9.5 and 10.1 at 100003, where a warp's own speed counts. The particle trace waits for L2
+// and wants warps: 5 blocks (94 registers) take 33.0 ms at 2^16 sinks, 4 take 36.8 and 6, which
+// spill, 36.1. The bands take 6 (8.95 ms for three at 200003 sinks, 9.2 at 8; 8.1 now).
 constexpr int cut_blocks(bool SUB, int NB) { return SUB ? 5 : NB > 1 ? 6 : 8; }
 // warps per group at most: the particle trace keeps 5 blocks of 4
 constexpr int most_warps(bool SUB) { return SUB ? 4 : kSlots; }
@@ -1005,10 +1005,10 @@ __global__ void __launch_bounds__(SHARED ? 32 * kSlots : 128, SHARED ? 4 : 8)
 }
 
 // Warps per group of 32 sinks: doubled while the call then has at most 64 warps on each SM (152
-// SMs where this was measured). At 32768 sinks of a background field 8 take 11.8 ms (1: 29.6,
-// 4: 12.3); at 100003 sinks 2 take 7.80 (1: 8.31, 4: 7.83, 8: 7.99); at 65536 sinks with the
-// particle trace 4 take 39.7 (1: 59.0, 2: 50.2, 8: 43.5); at 262144 sinks one warp takes 7.5 and
-// 2 take 8.5, since every warp of a group walks the whole source tree.
+// SMs where this was measured). At 32768 sinks of a background field 8 take 9.2 ms (1: 28.4,
+// 2: 15.5, 4: 10.2); at 100003 sinks 2 take 6.37 (1: 7.27, 4: 6.25, 8: 6.82); at 65536 sinks with
+// the particle trace 4 take 33.2 (1: 52.4, 2: 39.2); at 262144 sinks one warp takes 7.10 and 2
+// take 7.18, 4 take 7.94, since every warp of a group walks the whole source tree.
 int group_warps(int n_sink, int most) {
   const int groups = (n_sink + 31) / 32, fill = 64 * sm_count();
   int w = 1;
